@@ -72,6 +72,8 @@ _PROTOS = {
     "dpsr_mesh_extract": (_c_int, [_vp, _c_int, ctypes.c_float, _vp, _vp, _c_i64, _vp, _vp]),
     "dpsr_mesh_surrogate_splat": (_c_int, [_vp, _c_int, _vp, _vp, _vp, _c_i64, _c_int, _vp]),
     "dpsr_chamfer": (_c_int, [_vp, _c_i64, _vp, _c_i64, _vp, _vp, _vp, _vp, _vp]),
+    "dpsr_chamfer_ws_bytes": (_c_sz, [_c_i64, _c_i64]),
+    "dpsr_chamfer_tree": (_c_int, [_vp, _c_i64, _vp, _c_i64, _vp, _c_sz, _vp, _vp, _vp, _vp]),
     "dpsr_largest_region": (_c_int, [_vp, _c_int, ctypes.c_float, _vp, _vp, _vp, _vp, _vp]),
     "dpsr_mesh_extract_region": (_c_int, [_vp, _c_int, ctypes.c_float, _vp, _c_int, _vp, _vp, _c_i64, _vp, _vp]),
     "dpsr_mesh_sample": (_c_int, [_vp, _vp, _c_i64, _c_i64, ctypes.c_uint64, _vp, _vp, _vp, _vp]),
@@ -387,6 +389,16 @@ def dpsr_mesh_surrogate_splat(dchi: int, r: int, points: int, normals: int, dldp
 def dpsr_chamfer(a: int, na: int, b: int, nb: int, ws_idx: int, ws_d2: int, grad_a: int, loss: int,
                  stream: int = 0) -> None:
     check(load().dpsr_chamfer(a, int(na), b, int(nb), ws_idx, ws_d2, grad_a, loss, stream), "dpsr_chamfer")
+
+
+def dpsr_chamfer_ws_bytes(na: int, nb: int) -> int:
+    return int(load().dpsr_chamfer_ws_bytes(int(na), int(nb)))
+
+
+def dpsr_chamfer_tree(a: int, na: int, b: int, nb: int, ws: int, ws_bytes: int, grad_a: int, loss: int,
+                      loss32: int = 0, stream: int = 0) -> None:
+    check(load().dpsr_chamfer_tree(a, int(na), b, int(nb), ws, int(ws_bytes), grad_a, loss, loss32 or None, stream),
+          "dpsr_chamfer_tree")
 
 
 def dpsr_largest_region(chi: int, r: int, level: float, labels: int, ws: int, best: int, err: int,

@@ -31,21 +31,22 @@ PAPER_LEVELS = ((32, 2.0, 1000), (64, 2.0, 1000), (128, 3.0, 1000), (256, 3.0, 2
 
 class ChamferLoss(torch.autograd.Function):
     """Bi-directional L2 Chamfer distance between a (differentiable) and b
-    (dpsr_chamfer: brute-force nearest neighbours in both directions)."""
+    (dpsr_chamfer_tree: exact nearest neighbours in both directions)."""
 
     @staticmethod
     def forward(ctx, a, b):
         a, b = a.contiguous(), b.contiguous()
         na, nb = a.shape[0], b.shape[0]
         st = torch.cuda.current_stream(a.device).cuda_stream
-        ws_idx = torch.empty(na + nb, dtype=torch.int32, device=a.device)
-        ws_d2 = torch.empty(na + nb, device=a.device)
+        nws = L.dpsr_chamfer_ws_bytes(na, nb)
+        ws = torch.empty(max(nws, 1), dtype=torch.uint8, device=a.device)
         grad = torch.empty_like(a)
         loss = torch.empty(1, dtype=torch.float64, device=a.device)
-        L.dpsr_chamfer(a.data_ptr(), na, b.data_ptr(), nb, ws_idx.data_ptr(), ws_d2.data_ptr(), grad.data_ptr(),
-                       loss.data_ptr(), st)
+        loss32 = torch.empty((), dtype=torch.float32, device=a.device)
+        L.dpsr_chamfer_tree(a.data_ptr(), na, b.data_ptr(), nb, ws.data_ptr(), nws, grad.data_ptr(), loss.data_ptr(),
+                            loss32.data_ptr(), st)
         ctx.save_for_backward(grad)
-        return loss.to(a.dtype).reshape(())
+        return loss32 if a.dtype == torch.float32 else loss.to(a.dtype).reshape(())
 
     @staticmethod
     def backward(ctx, g):

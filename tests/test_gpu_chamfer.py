@@ -1,0 +1,96 @@
+"""The Chamfer distance by the box tree against FP64 brute force, at the sizes
+where its packets, leaves, box levels and cell grids begin and end, and with
+equal points, points far from the other set and points that are not finite."""
+import numpy as np
+import pytest
+
+from paper_2106_03452_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2106_03452_gb300 import build
+    build.build()
+
+
+def _run(a, b):
+    import torch
+    from paper_2106_03452_gb300.optimize import chamfer
+    A = torch.from_numpy(a).cuda().requires_grad_(True)
+    loss = chamfer(A, torch.from_numpy(b).cuda())
+    (g,) = torch.autograd.grad(loss, A)
+    return float(loss.detach()), g.cpu().numpy()
+
+
+def _reference(a, b):
+    """Brute force in FP64 on neighbours picked as in FP32 (ties to the lowest index)."""
+    def nearest(q, t):
+        idx = np.empty(len(q), np.int64)
+        for k in range(0, len(q), 256):
+            d = (q[k:k + 256, None, :] - t[None]).astype(np.float64)
+            v = np.float32(d[..., 2] ** 2)  # fma(dx, dx, fma(dy, dy, dz * dz)) in FP32
+            for c in (1, 0):
+                v = np.float32(d[..., c] ** 2 + v)
+            idx[k:k + 256] = v.argmin(1)
+        return idx
+    i, j = nearest(a, b), nearest(b, a)
+    a64, b64 = a.astype(np.float64), b.astype(np.float64)
+    loss = ((a64 - b64[i]) ** 2).sum(1).mean() + ((b64 - a64[j]) ** 2).sum(1).mean()
+    g = 2.0 * (a64 - b64[i]) / len(a)
+    np.add.at(g, j, 2.0 * (a64[j] - b64) / len(b))
+    return loss, g
+
+
+SIZES = [(1, 1), (1, 1000), (16, 17), (31, 33), (1024, 1025), (32768, 40), (70, 32769), (5001, 3003)]
+
+
+@pytest.mark.parametrize("na,nb", SIZES)
+@pytest.mark.parametrize("kind", ["surface", "volume", "grid", "apart"])
+def test_tree_matches_bruteforce(na, nb, kind):
+    rng = synth.Rng(na * 7 + nb + len(kind))
+    if kind == "surface":
+        a, b = (synth.sphere_cloud(rng, n, jitter=0.01)[0] for n in (na, nb))
+    elif kind == "volume":
+        a, b = rng.uniform(na, 3) * 2 - 1, rng.uniform(nb, 3) * 2 - 1
+    elif kind == "grid":  # equal points and equal distances everywhere
+        a, b = (np.floor(rng.uniform(n, 3) * 9) for n in (na, nb))
+    else:  # the sets far from each other, one of them flat, and a stray point
+        a, b = rng.uniform(na, 3) * [1, 1, 0], rng.uniform(nb, 3) + [40, 0, 0]
+        a[0] = [-1e6, 3, 5]
+    a, b = a.astype(np.float32), b.astype(np.float32)
+    loss, g = _run(a, b)
+    rloss, rg = _reference(a, b)
+    # FP32 squared distances (relative 2^-22), and sums of at most nb + 1 terms per gradient
+    assert abs(loss - rloss) <= 1e-6 * rloss
+    assert np.max(np.abs(g - rg)) <= 1e-5 * np.max(np.abs(rg))
+
+
+def test_points_that_are_not_finite():
+    rng = synth.Rng(5)
+    a, b = rng.uniform(700, 3).astype(np.float32), rng.uniform(900, 3).astype(np.float32)
+    a[3, 1], a[200, 0], b[17, 2], b[500] = np.nan, np.inf, np.nan, -np.inf
+    loss, g = _run(a, b)
+    fa, fb = np.isfinite(a).all(1), np.isfinite(b).all(1)
+    _, rg = _reference(a[fa], b[fb])
+    assert not np.isfinite(loss) and np.isnan(g[~fa]).all()
+    # the finite points' neighbours are the finite ones; the weights count every point
+    i = np.nonzero(fa)[0]
+    d = a[fa][:, None, :].astype(np.float64) - b[fb][None]
+    ab, ba = (d ** 2).sum(-1).argmin(1), (d ** 2).sum(-1).argmin(0)
+    want = 2.0 * (a[fa] - b[fb][ab].astype(np.float64)) / len(a)
+    np.add.at(want, ba, 2.0 * (a[fa][ba].astype(np.float64) - b[fb]) / len(b))
+    assert np.max(np.abs(g[i] - want)) <= 1e-5 * np.max(np.abs(want))
+
+
+def test_workspace_is_checked():
+    from paper_2106_03452_gb300 import libdpsr as L
+    assert L.dpsr_chamfer_ws_bytes(0, 5) == 0 and L.dpsr_chamfer_ws_bytes(5, 2 ** 31) == 0
+    n = L.dpsr_chamfer_ws_bytes(10, 10)
+    lib = L.load()
+    for ws, nb in ((256, n - 1), (264, n), (0, n)):  # too small, misaligned, NULL: refused before any launch
+        assert lib.dpsr_chamfer_tree(256, 10, 256, 10, ws or None, nb, 256, 256, None, None) == L.DPSR_EINVAL
