@@ -1,0 +1,59 @@
+"""Sampling on a triangle soup at the edges of its scan blocks (1 024
+triangles), of its searches and of its vector loads, against FP64 on the same
+draws."""
+import numpy as np
+import pytest
+
+from paper_2106_03452_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2106_03452_gb300 import build
+    build.build()
+
+
+@pytest.mark.parametrize("offset", [0, 1])  # of the soup in floats: off a 16-byte boundary too
+@pytest.mark.parametrize("T", [1, 2, 1023, 1024, 1025, 4099, 2048 * 1024 + 5])
+def test_sample_matches_fp64(T, offset):
+    import torch
+    from paper_2106_03452_gb300.mesh import sample
+    rng = synth.Rng(T + offset)
+    M, seed = 3001, 77 + T
+    tris = (rng.uniform(min(T, 5000), 3, 3) - 0.3).astype(np.float32)
+    tris = np.tile(tris, (-(-T // len(tris)), 1, 1))[:T]
+    tris[T // 2] = tris[T // 2, 0]  # a triangle without area
+    if T == 1:
+        tris[0] = [[0, 0, 0], [1, 0, 0], [0, 1, 0]]
+    nrm = rng.normal(T, 3).astype(np.float32)
+    buf = torch.empty(9 * T + 4, device="cuda")
+    t = buf[offset:offset + 9 * T].view(T, 3, 3)
+    t.copy_(torch.from_numpy(tris))
+    P, N = (x.cpu().numpy().astype(np.float64) for x in sample(t, torch.from_numpy(nrm).cuda(), M, seed))
+    t64 = tris.astype(np.float64)
+    area = 0.5 * np.linalg.norm(np.cross(t64[:, 1] - t64[:, 0], t64[:, 2] - t64[:, 0]), axis=1)
+    cum = np.cumsum(area)
+    def u01(i):
+        z = np.uint64(seed) + np.uint64(0x9E3779B97F4A7C15) * (i.astype(np.uint64) + np.uint64(1))
+        z = (z ^ (z >> np.uint64(30))) * np.uint64(0xBF58476D1CE4E5B9)
+        z = (z ^ (z >> np.uint64(27))) * np.uint64(0x94D049BB133111EB)
+        return ((z ^ (z >> np.uint64(31))) >> np.uint64(11)).astype(np.float64) / 2.0 ** 53
+    i = np.arange(M)
+    x = u01(3 * i) * cum[-1]
+    k = np.minimum(np.searchsorted(cum, x, side="right"), T - 1)
+    # a draw within rounding of a boundary (1e-12 of the total) may fall to either side
+    clear = np.minimum(np.abs(cum[k] - x), np.abs(x - np.where(k > 0, cum[k - 1], 0))) > 1e-12 * cum[-1]
+    assert clear.sum() > 0.99 * M
+    u, v = u01(3 * i + 1), u01(3 * i + 2)
+    flip = u + v > 1
+    u, v = np.where(flip, 1 - u, u)[:, None], np.where(flip, 1 - v, v)[:, None]
+    c = t64[k]
+    want = c[:, 0] + u * (c[:, 1] - c[:, 0]) + v * (c[:, 2] - c[:, 0])
+    # FP32 edge vectors and one rounding of the point: 3 x 2^-24 of coordinates below 1
+    assert np.max(np.abs(P - want)[clear]) <= 3e-7
+    assert np.array_equal(N[clear], nrm.astype(np.float64)[k][clear])
