@@ -385,6 +385,16 @@ int make_tensor_maps(Solve& s, int r) {
       if (rc != CUDA_SUCCESS) return DPSR_ECUDA;
     }
   }
+  if (r < 64) return DPSR_OK;  // kSkip: the parts of tiles below are not used
+  const cuuint32_t boxb[3] = {16, 16, 1}, boxc[3] = {16, 1, (cuuint32_t)(r / kXChunks)};
+  for (int k = 0; k < kNSpec + 4; ++k) {
+    const bool b = k < kNSpec;
+    CUresult rc = enc(b ? &s.tmb[k] : &s.tmc[k - kNSpec], CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3,
+                      (void*)s.spec[b ? k : k - kNSpec], dims, strides, b ? boxb : boxc, es,
+                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                      CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (rc != CUDA_SUCCESS) return DPSR_ECUDA;
+  }
   return DPSR_OK;
 }
 }  // namespace dpsr
@@ -789,6 +799,17 @@ int dpsr_debug_read_spectrum(dpsr_plan p, int which, void* out_host) {
                    (size_t)r * r, cudaMemcpyDeviceToHost) != cudaSuccess) {
     cudaGetLastError();
     return DPSR_ECUDA;
+  }
+  if (which < 3 && r >= 64) {  // the splat's spectra are zero, and not stored, in x-chunks without points
+    unsigned chunks = 0;
+    if (cudaMemcpy(&chunks, dpsr::occ_words(p->s.bins, r) + r, sizeof(unsigned), cudaMemcpyDeviceToHost) !=
+        cudaSuccess) {
+      cudaGetLastError();
+      return DPSR_ECUDA;
+    }
+    const size_t part = w * (size_t)r * (size_t)(r / dpsr::kXChunks);
+    for (int c = 0; c < dpsr::kXChunks; ++c)
+      if (!((chunks >> c) & 1u)) memset((char*)out_host + c * part, 0, part);
   }
   return DPSR_OK;
 }

@@ -237,6 +237,9 @@ __device__ __forceinline__ void zfwd_tile(const Solve& S, int X, int y0, float* 
     c3 = c2 + (e2 - q2);
     c4 = c3 + (e3 - q3);
   }
+  __shared__ unsigned char touched[YB];  // rows that points reach
+  if (tid < YB) touched[tid] = 0;
+  __syncthreads();
   for (int v = tid; v < c4; v += P::ZNT) {
     const int k = v < c1 ? 0 : (v < c2 ? 1 : (v < c3 ? 2 : 3));
     const int i = k == 0 ? q0 + v : (k == 1 ? q1 + (v - c1) : (k == 2 ? q2 + (v - c2) : q3 + (v - c3)));
@@ -252,6 +255,7 @@ __device__ __forceinline__ void zfwd_tile(const Solve& S, int X, int y0, float* 
     for (int dy = 0; dy < 2; ++dy) {
       const int ly = (dy ? ay.i1 : ay.i0) - y0;
       if ((unsigned)ly >= (unsigned)YB) continue;
+      touched[ly] = 1;  // the same value from every point
       const float f = wx * tri_w(dy, ay.t);
       const float f0 = f * (1.f - az.t), f1 = f * az.t;
 #pragma unroll
@@ -272,7 +276,12 @@ __device__ __forceinline__ void zfwd_tile(const Solve& S, int X, int y0, float* 
       const bool vz = pi >= YB / 2 && pi < YB;
       const int ch = (2 * pi) / YB, ly = (2 * pi) % YB;  // rows ly, ly + 1 of channel ch
       float2* ga = S.spec[ch] + ((size_t)X * L + y0 + ly) * P::KP;
-      r2c_pair_st<L>(t, twr, rows + pair_off<L>(pi), vz ? iu : nullptr, ga, ga + P::KP);
+      if (kSkip<L> && !(touched[ly] | touched[ly + 1])) {  // a pair without points: its spectrum is zero
+#pragma unroll
+        for (int j = 0; j < P::R1 / 2; ++j) ga[t + P::T * j] = ga[P::KP + t + P::T * j] = czero();
+      } else {
+        r2c_pair_st<L>(t, twr, rows + pair_off<L>(pi), vz ? iu : nullptr, ga, ga + P::KP);
+      }
     }
   }
 }
@@ -291,12 +300,16 @@ __global__ void __launch_bounds__(Pen<L>::ZNT, L >= 512 ? 1 : (L >= 256 ? 3 : 4)
   float2* twt = reinterpret_cast<float2*>(rows + RF);
   float* iu = reinterpret_cast<float*>(twt + L);
   pdl_trigger();
+  if constexpr (kSkip<L>) {  // a tile that no stencil reaches is not stored: the y pass does not load it
+    pdl_wait();
+    if (!((reach_mask(tile_mask(S, L, X), P::NYB) >> (y0 / YB)) & 1u)) return;
+  }
   for (int i = tid; i < L; i += P::ZNT) {
     twt[i] = S.tw[i];
     iu[i] = S.iu[2 * L + i];  // z axis
   }
   for (int i = tid; i < RF / 4; i += P::ZNT) smem4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-  pdl_wait();
+  if constexpr (!kSkip<L>) pdl_wait();
   __syncthreads();
   zfwd_tile<L>(S, X, y0, rows, twt, iu);
 }
@@ -340,6 +353,23 @@ __device__ __forceinline__ YfwdBufs yfwd_bufs(int kind) {
   return b;
 }
 
+// Warp 0: the loads of the y-blocks `rows` of a forward y-pass tile (the other
+// blocks hold no points and were not stored), a lane per block.
+template <int L>
+__device__ __forceinline__ void yfwd_issue_rows(const Solve& S, int X, int kz0, int kind, unsigned rows, float2* box,
+                                                uint64_t* bar) {
+  using P = Pen<L>;
+  const YfwdBufs b = yfwd_bufs<L, false>(kind);
+  const int lane = threadIdx.x;
+  if (lane == 0) mbar_expect_tx(bar, __popc(rows) * (b.two ? 2 : 1) * 16 * P::YB * (uint32_t)sizeof(float2));
+  __syncwarp();
+  if (lane < P::NYB && ((rows >> lane) & 1u)) {
+    const int y = lane * P::YB;
+    tma_load_3d(box + y * 16, &S.tmb[b.buf0], kz0, y, X, bar);
+    if (b.two) tma_load_3d(box + P::BOX + y * 16, &S.tmb[b.buf1], kz0, y, X, bar);
+  }
+}
+
 // Thread 0: the TMA tile loads of a y-pass tile, completion on `bar`.
 template <int L, bool BWD>
 __device__ __forceinline__ void yfwd_issue(const Solve& S, int X, int kz0, int kind, float2* box,
@@ -359,7 +389,7 @@ __device__ __forceinline__ void yfwd_issue(const Solve& S, int X, int kz0, int k
 template <int L, bool BWD>
 __device__ __forceinline__ bool yfwd_tile(const Solve& S, int X, int kz0, int kind, float2* box,
                                           const float2* twt, const float* iu, uint64_t* bar,
-                                          uint32_t phase) {
+                                          uint32_t phase, unsigned rows = 0xffffffffu) {
   using P = Pen<L>;
   constexpr int H = P::H;
   const YfwdBufs bb = yfwd_bufs<L, BWD>(kind);
@@ -379,8 +409,10 @@ __device__ __forceinline__ bool yfwd_tile(const Solve& S, int X, int kz0, int ki
     float2* b0 = box;
     auto c0 = [b0, g](int e) -> float2& { return b0[bx(e, g)]; };
     float2 a[P::R1];
+    // rows of blocks that were not loaded are zero (T divides a block)
+    auto has = [rows](int j) { return BWD || !kSkip<L> || ((rows >> (P::T * j / P::YB)) & 1u); };
 #pragma unroll
-    for (int j = 0; j < P::R1; ++j) a[j] = c0(t + P::T * j);
+    for (int j = 0; j < P::R1; ++j) a[j] = has(j) ? c0(t + P::T * j) : czero();
     fft_r<L, -1, IL>(a, t, c0, twr);
 #pragma unroll
     for (int j = 0; j < P::R1; ++j) c0(t + P::T * j) = a[j];
@@ -388,7 +420,7 @@ __device__ __forceinline__ bool yfwd_tile(const Solve& S, int X, int kz0, int ki
       float2* b1 = box + P::BOX;
       auto c1 = [b1, g](int e) -> float2& { return b1[bx(e, g)]; };
 #pragma unroll
-      for (int j = 0; j < P::R1; ++j) a[j] = c1(t + P::T * j);
+      for (int j = 0; j < P::R1; ++j) a[j] = has(j) ? c1(t + P::T * j) : czero();
       fft_r<L, -1, IL>(a, t, c1, twr);
       if (kind == 0) {  // D = FFT(i u_z v_z) + i u_y FFT(v_y); this lane wrote c0 above
 #pragma unroll
@@ -448,13 +480,22 @@ __global__ void __launch_bounds__(ynt<L>(), L >= 512 ? 1 : (BWD ? 4 : (L >= 256 
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   pdl_wait();
-  if (tid == 0) yfwd_issue<L, BWD>(S, X, kz0, kind, box, &bar);
+  unsigned rows = 0xffffffffu;
+  if constexpr (!BWD && kSkip<L>) {
+    rows = reach_mask(tile_mask(S, L, X), P::NYB);
+    // a plane without points: not stored either where its whole x-chunk is
+    // empty (the x pass does not load it), else stored as zeros
+    if (rows == 0u && !((chunk_mask(S, L) >> (X / (L / kXChunks))) & 1u)) return;
+    if (tid < 32) yfwd_issue_rows<L>(S, X, kz0, kind, rows, box, &bar);
+  } else if (tid == 0) {
+    yfwd_issue<L, BWD>(S, X, kz0, kind, box, &bar);
+  }
   for (int i = tid; i < L; i += NT) {
     twt[i] = S.tw[i];
     iu[i] = S.iu[L + i];  // y axis
   }
   __syncthreads();
-  yfwd_tile<L, BWD>(S, X, kz0, kind, box, twt, iu, &bar, 0);
+  yfwd_tile<L, BWD>(S, X, kz0, kind, box, twt, iu, &bar, 0, rows);
 }
 
 // ===========================================================================
@@ -498,7 +539,7 @@ __device__ __forceinline__ void yinv_issue(const Solve& S, int X, int kz0, int p
 template <int L, int NCH>
 __device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int part, float2* box,
                                           const float2* twt, const float* iu, uint64_t* bar,
-                                          uint32_t phase) {
+                                          uint32_t phase, unsigned rows = 0xffffffffu) {
   using P = Pen<L>;
   constexpr int H = P::H;
   constexpr bool IL = P::T == 16;  // interleaved groups: conflict-free column accesses
@@ -564,7 +605,18 @@ __device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int pa
   }
   fence_async_smem();
   __syncthreads();
-  if (tid == 0) {
+  if constexpr (NCH == 3 && kSkip<L>) {  // warp 0: the y-blocks that the z pass reads, a lane each
+    if (tid < P::NYB && ((rows >> tid) & 1u)) {
+      const int y = tid * P::YB;
+      if (do0) tma_store_3d(&S.tmb[kSpC], kz0, y, X, box + y * 16);
+      if (do1) {
+        tma_store_3d(&S.tmb[kSpYa], kz0, y, X, box + P::BOX + y * 16);
+        tma_store_3d(&S.tmb[kSpYb], kz0, y, X, box + 2 * P::BOX + y * 16);
+      }
+      tma_store_commit();
+      tma_store_wait_read();
+    }
+  } else if (tid == 0) {
     for (int y = 0; y < L; y += tma_rows(L)) {
       if constexpr (NCH == 1) {
         tma_store_3d(&S.tmy[kSpYa], kz0, y, X, box + y * 16);
@@ -604,6 +656,11 @@ __global__ void __launch_bounds__(16 * Shape<L>::T >= 32 ? 16 * Shape<L>::T : 32
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   pdl_wait();
+  unsigned rows = 0xffffffffu;
+  if constexpr (NCH == 3 && kSkip<L>) {
+    rows = reach_mask(tile_mask(S, L, X), P::NYB);
+    if (rows == 0u) return;  // no points gather from this plane
+  }
   const int part = yinv_split<L, NCH>() ? (int)blockIdx.y : -1;  // -1: all fields
   if (tid == 0) yinv_issue<L, NCH>(S, X, kz0, part, box, &bar);
   for (int i = tid; i < L; i += NT) {
@@ -611,7 +668,7 @@ __global__ void __launch_bounds__(16 * Shape<L>::T >= 32 ? 16 * Shape<L>::T : 32
     iu[i] = S.iu[L + i];  // y axis
   }
   __syncthreads();
-  yinv_tile<L, NCH>(S, X, kz0, part, box, twt, iu, &bar, 0);
+  yinv_tile<L, NCH>(S, X, kz0, part, box, twt, iu, &bar, 0, rows);
 }
 
 // ===========================================================================
@@ -778,6 +835,64 @@ __device__ __forceinline__ bool zinv_tile(const Solve& S, int tile, float2* sb, 
   return true;
 }
 
+// The tiles (plane, y-block) with points to gather at, in order: tile k by a
+// search over the planes' running counts, so that persistent CTAs share them
+// evenly without a list in memory.
+template <int L, int NT>
+struct TileList {
+  unsigned mask[L];
+  unsigned short first[L];  // tiles of the planes before
+  int wsum[NT / 32];
+  // All NT threads, after the binning is visible; the caller synchronises
+  // the block before tile().
+  __device__ int build(const Solve& S) {
+    constexpr int PT = (L + NT - 1) / NT;  // consecutive planes per thread
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    int run = 0, n[PT];
+#pragma unroll
+    for (int j = 0; j < PT; ++j) {
+      const int X = tid * PT + j;
+      n[j] = 0;
+      if (X < L) {
+        const unsigned m = tile_mask(S, L, X);
+        mask[X] = m;
+        n[j] = __popc(m);
+      }
+      run += n[j];
+    }
+    int incl = run;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= d) incl += v;
+    }
+    if (lane == 31) wsum[w] = incl;
+    __syncthreads();
+    int pos = incl - run, total = 0;
+#pragma unroll
+    for (int k = 0; k < NT / 32; ++k) {
+      pos += k < w ? wsum[k] : 0;
+      total += wsum[k];
+    }
+#pragma unroll
+    for (int j = 0; j < PT; ++j) {
+      const int X = tid * PT + j;
+      if (X < L) first[X] = (unsigned short)pos;
+      pos += n[j];
+    }
+    return total;
+  }
+  __device__ int tile(int k) const {
+    int lo = 0;  // the last plane whose first tile is at most k: it has tiles, the next starts beyond
+#pragma unroll
+    for (int d = L / 2; d > 0; d >>= 1)
+      if ((int)first[lo + d] <= k) lo += d;
+    unsigned m = mask[lo];
+    for (int q = k - (int)first[lo]; q > 0; --q) m &= m - 1u;
+    return lo * (L / ybin(L)) + __ffs(m) - 1;
+  }
+};
+
 template <int L, int NCH>
 __global__ void __launch_bounds__(ZiGeo<L, NCH>::NT, L >= 512 ? 1 : (NCH == 1 ? 4 : (L >= 256 ? 2 : 3)))
     k_zinv(const __grid_constant__ Solve s0, const Solve* __restrict__ tab) {
@@ -790,6 +905,8 @@ __global__ void __launch_bounds__(ZiGeo<L, NCH>::NT, L >= 512 ? 1 : (NCH == 1 ? 
   float2* stg = reinterpret_cast<float2*>(smem4);  // 2 stages, row (ch, ly) at row_off(ch NR + ly)
   float2* twt = stg + 2 * Z::STAGE;
   __shared__ uint64_t bar[2];
+  constexpr bool LIST = NCH == 3 && kSkip<L>;
+  __shared__ TileList<LIST ? L : 1, NT> list;
   pdl_trigger();
   for (int i = tid; i < L; i += NT) twt[i] = S.tw[i];
   if (tid == 0) {
@@ -798,21 +915,28 @@ __global__ void __launch_bounds__(ZiGeo<L, NCH>::NT, L >= 512 ? 1 : (NCH == 1 ? 
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   pdl_wait();
+  int ntiles = L * P::NYB;
+  if constexpr (LIST) ntiles = list.build(S);
   __syncthreads();
-  constexpr int ntiles = L * P::NYB;
+  auto at = [&](int k) {  // the k-th tile to do
+    if constexpr (LIST) return list.tile(k);
+    else return k;
+  };
   float a_chi = 0.f, b_chi = 0.f;
   if constexpr (NCH == 1) {
     a_chi = S.sc->a_chi;
     b_chi = S.sc->b_chi;
   }
   uint32_t ph = 0u;  // bit st: parity of stage st's next completion
-  int tile = blockIdx.x;
-  if (tid == 0 && tile < ntiles) zinv_issue<L, NCH>(S, tile, stg, &bar[0]);
-  for (int it = 0; tile < ntiles; ++it, tile += gridDim.x) {
+  int k = blockIdx.x;
+  int tile = k < ntiles ? at(k) : 0;
+  if (tid == 0 && k < ntiles) zinv_issue<L, NCH>(S, tile, stg, &bar[0]);
+  for (int it = 0; k < ntiles; ++it, k += gridDim.x) {
     const int st = it & 1;
-    const int next = tile + gridDim.x;
+    const int next = k + gridDim.x;
+    const int next_tile = next < ntiles ? at(next) : 0;
     // released at the end of the last iteration
-    if (tid == 0 && next < ntiles) zinv_issue<L, NCH>(S, next, stg + (st ^ 1) * Z::STAGE, &bar[st ^ 1]);
+    if (tid == 0 && next < ntiles) zinv_issue<L, NCH>(S, next_tile, stg + (st ^ 1) * Z::STAGE, &bar[st ^ 1]);
     bool ok = zinv_tile<L, NCH>(S, tile, stg + st * Z::STAGE, twt, a_chi, b_chi, [&]() {
       const bool landed = __syncthreads_and(mbar_wait(&bar[st], (ph >> st) & 1u));
       ph ^= 1u << st;
@@ -825,6 +949,7 @@ __global__ void __launch_bounds__(ZiGeo<L, NCH>::NT, L >= 512 ? 1 : (NCH == 1 ? 
       }
       break;
     }
+    tile = next_tile;
   }
 }
 

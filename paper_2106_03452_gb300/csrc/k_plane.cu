@@ -778,6 +778,7 @@ __global__ void __launch_bounds__(binv_threads<L, C>(), binv_smem<L, C>() <= 113
     twt[i] = S.tw[i];
   }
   pdl_wait();
+  if (tile_mask(S, L, X) == 0u) return;  // no points gather from this plane (the whole cluster leaves)
   const int s_first = c * SPC;
   if (tid == 0) {
     mbar_init(&barL[0], 1);
@@ -978,6 +979,7 @@ __global__ void __launch_bounds__(BinvChGeo<L>::NT, 3)
     twt[i] = S.tw[i];
   }
   pdl_wait();
+  if (tile_mask(S, L, X) == 0u) return;  // no points gather from this plane
   // X channel from Q2 = IFFT_x(-i u_x F), Y and Z from Q1 = IFFT_x(F)
   const int sp = ch == 0 ? kSpChi : kSpD;
   if (tid == 0) {

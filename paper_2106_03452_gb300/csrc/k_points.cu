@@ -75,6 +75,7 @@ __global__ void __launch_bounds__(256) k_bin_scatter(const __grid_constant__ Sol
   constexpr int NT = 256;
   extern __shared__ int h[];
   __shared__ int wsum[NT / 32];
+  __shared__ unsigned socc[512], schunk;
   pdl_trigger();
   pdl_wait();
   const Solve& S = tab ? tab[blockIdx.z] : s0;
@@ -115,6 +116,26 @@ __global__ void __launch_bounds__(256) k_bin_scatter(const __grid_constant__ Sol
   __syncthreads();
   if (blockIdx.x == 0) {
     for (int i = tid; i < nb; i += NT) off[i] = h[scan_slot(i)];
+    // occupancy of the bins (see bins_ints): a bin's count is the step to the next offset
+    const int ny = nybins(r);
+    unsigned* occ = reinterpret_cast<unsigned*>(cur + nb);
+    if (tid == 0) schunk = 0u;
+    for (int x = tid; x < r; x += NT) {
+      unsigned m = 0u;
+      for (int b = 0; b < ny; ++b) {
+        const int i = x * ny + b, end = i + 1 < nb ? h[scan_slot(i + 1)] : total;
+        m |= (end > h[scan_slot(i)] ? 1u : 0u) << b;
+      }
+      socc[x] = m;
+      occ[x] = m;
+    }
+    __syncthreads();
+    unsigned c = 0u;
+    for (int x = tid; x < r; x += NT)
+      if (socc[x] | socc[(x - 1) & (r - 1)]) c |= 1u << (x / (r / kXChunks));
+    if (c) atomicOr(&schunk, c);
+    __syncthreads();
+    if (tid == 0) occ[r] = schunk;
     if (tid == 0) {
       off[nb] = total;
       S.sc->ticket[0] = 0;

@@ -94,16 +94,35 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 1 : (L >= 256 ? (BWD ?
   pdl_wait();
   // the binning of this forward pass is done: its counters start the next one at zero
   if constexpr (!BWD) clear_bin_counters(S, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
-  if (tid == 0) {
+  // From r = 64 on the splat's spectra (D, C, W~) are only loaded for the
+  // x-chunks that points touch, a lane of warp 0 per chunk; the rest is zero.
+  const unsigned chunks = kSkip<L> ? chunk_mask(S, L) : 0xffu;
+  constexpr int XC = L / kXChunks;
+  auto has = [chunks](int j) { return !kSkip<L> || ((chunks >> (P::T * j / XC)) & 1u); };  // x = t + T j, t < T
+  auto load_chunks = [&](int buf, int c) {  // warp 0
+    if (tid == 0) mbar_expect_tx(&bar[c], __popc(chunks) * XC * P::KC * (uint32_t)sizeof(float2));
+    __syncwarp();
+    if (tid < kXChunks && ((chunks >> tid) & 1u))
+      tma_load_3d(box + c * P::BOX + tid * XC * P::KC, &S.tmc[buf], kz0, ky, tid * XC, &bar[c]);
+  };
+  auto load_all = [&](int buf, int c) {  // thread 0
+    mbar_expect_tx(&bar[c], P::BOX * (uint32_t)sizeof(float2));
+    for (int x = 0; x < L; x += tma_rows(L))
+      tma_load_3d(box + c * P::BOX + x * P::KC, &S.tmx[buf], kz0, ky, x, &bar[c]);
+  };
+  if (tid < 32) {
+    if (tid == 0) {
 #pragma unroll
-    for (int c = 0; c < NCH; ++c) mbar_init(&bar[c], 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-#pragma unroll
-    for (int c = 0; c < NCH; ++c) {
-      mbar_expect_tx(&bar[c], P::BOX * (uint32_t)sizeof(float2));
-      for (int x = 0; x < L; x += tma_rows(L))
-        tma_load_3d(box + c * P::BOX + x * P::KC, &S.tmx[c == 0 ? src0 : (c == 1 ? src1 : kSpW)], kz0, ky,
-                    x, &bar[c]);
+      for (int c = 0; c < NCH; ++c) mbar_init(&bar[c], 1);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if constexpr (kSkip<L>) {
+      if (!BWD) load_chunks(src0, 0);
+      else if (tid == 0) load_all(src0, 0);
+      load_chunks(src1, 1);
+    } else if (tid == 0) {
+      load_all(src0, 0);
+      load_all(src1, 1);
     }
   }
   for (int i = tid; i < L; i += P::NT) {
@@ -155,7 +174,7 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 1 : (L >= 256 ? (BWD ?
       // FFT_x(D) goes back to its column, FFT_x(C) meets it there.
       box_wait(0);
 #pragma unroll
-      for (int j = 0; j < P::R1; ++j) a[j] = c0(t + P::T * j);
+      for (int j = 0; j < P::R1; ++j) a[j] = has(j) ? c0(t + P::T * j) : czero();
       fft_r<L, -1, IL>(a, t, c0, twr);
       if (own) {  // groups past the last column (tiny r) only shadow it
 #pragma unroll
@@ -163,7 +182,7 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 1 : (L >= 256 ? (BWD ?
       }
       box_wait(1);
 #pragma unroll
-      for (int j = 0; j < P::R1; ++j) a[j] = c1(t + P::T * j);
+      for (int j = 0; j < P::R1; ++j) a[j] = has(j) ? c1(t + P::T * j) : czero();
       fft_r<L, -1, IL>(a, t, c1, twr);
 #pragma unroll
       for (int j = 0; j < P::R1; ++j) {
@@ -177,11 +196,8 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 1 : (L >= 256 ? (BWD ?
       // there (the fence orders this thread's writes to it before the copy's)
       fence_async_smem();
       __syncthreads();
-      if (tid == 0 && ok) {
-        mbar_expect_tx(&bar[1], P::BOX * (uint32_t)sizeof(float2));
-        for (int x = 0; x < L; x += tma_rows(L))
-          tma_load_3d(box + P::BOX + x * P::KC, &S.tmx[kSpW], kz0, ky, x, &bar[1]);
-      }
+      static_assert(kSkip<L>, "loaded by chunks");
+      if (tid < 32 && __all_sync(0xffffffffu, ok)) load_chunks(kSpW, 1);
       w_reload = true;
     }
     if (valid) {
@@ -194,14 +210,14 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 1 : (L >= 256 ? (BWD ?
         box_wait(1, 1u);
 #pragma unroll
         for (int j = 0; j < P::R1; ++j) {
-          const float2 w = c1(t + P::T * j);
+          const float2 w = has(j) ? c1(t + P::T * j) : czero();
           am += w.x * a[j].x + w.y * a[j].y;
         }
       } else {
         const float2* wc = S.spec[kSpW] + (size_t)ky * P::KP + kz;
 #pragma unroll
         for (int j = 0; j < P::R1; ++j) {
-          const float2 w = __ldcg(wc + (size_t)(t + P::T * j) * L * P::KP);
+          const float2 w = has(j) ? __ldcg(wc + (size_t)(t + P::T * j) * L * P::KP) : czero();
           am += w.x * a[j].x + w.y * a[j].y;
         }
       }
@@ -240,7 +256,7 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 1 : (L >= 256 ? (BWD ?
 #pragma unroll
     for (int j = 0; j < P::R1; ++j) {
       const int x = t + P::T * j;
-      a[j] = cadd(cscale(c0(x), ga), cscale(c1(x), gw));
+      a[j] = cadd(cscale(c0(x), ga), has(j) ? cscale(c1(x), gw) : czero());
       if (x == 0) a[j].x += gs;
     }
     fft_r<L, -1, IL>(a, t, c0, twr);
