@@ -23,7 +23,8 @@ __device__ __forceinline__ int bin_key(int ix, int iy, int r) { return ix * nybi
 // global add per touched bin. The counts must be zero on entry: the forward
 // x-pass clears them (and the scatter cursors) once the scatter is done.
 // Dynamic shared memory: the histogram, nbins(r) ints.
-__global__ void __launch_bounds__(256) k_bin_count(const __grid_constant__ Solve s0,
+template <int NT>
+__global__ void __launch_bounds__(NT) k_bin_count(const __grid_constant__ Solve s0,
                                                    const Solve* __restrict__ tab) {
   extern __shared__ int h[];
   pdl_trigger();
@@ -70,9 +71,9 @@ __host__ __device__ constexpr int scan_slot(int i) { return i + (i >> 5); }
 // counters of the solve's last-block reductions. A point's slot is its bin's
 // offset plus a ticket from that bin's cursor (zero on entry; cleared again
 // by the forward x-pass). Dynamic shared memory: scan_slot(nbins(r)) ints.
-__global__ void __launch_bounds__(256) k_bin_scatter(const __grid_constant__ Solve s0,
-                                                     const Solve* __restrict__ tab) {
-  constexpr int NT = 256;
+template <int NT>
+__global__ void __launch_bounds__(NT) k_bin_scatter(const __grid_constant__ Solve s0,
+                                                    const Solve* __restrict__ tab) {
   extern __shared__ int h[];
   __shared__ int wsum[NT / 32];
   __shared__ unsigned socc[512], schunk;
@@ -167,22 +168,31 @@ __global__ void __launch_bounds__(256) k_bin_scatter(const __grid_constant__ Sol
   }
 }
 
-cudaError_t launch_bin(const Solve& s, const Solve* tab, int count, int nmax, int r, cudaStream_t st) {
-  const int blocks = min(max((nmax + 255) / 256, 1), 1184);
+// Threads of the binning blocks: 256 up to r = 128; 1 024 from r = 256 on (4 096
+// to 16 384 bins), where a block's own scan of the counts, bins / threads steps
+// in series, is most of its time and fewer blocks repeat it: 100 000 points at
+// r = 256 21.4 -> 16.7 us for both kernels, 200 000 at r = 512 67.6 -> 33.5.
+template <int NT>
+static cudaError_t launch_bin_t(const Solve& s, const Solve* tab, int count, int nmax, int r, cudaStream_t st) {
+  const int blocks = min(max((nmax + NT - 1) / NT, 1), 1184 * 256 / NT);
   const size_t hc = sizeof(int) * nbins(r), hs = sizeof(int) * scan_slot(nbins(r));
   static bool attr_set = false;  // 16384 bins at r = 512 need more than the default 48 KB
   if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_bin_count, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(k_bin_count<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)(sizeof(int) * nbins(512)));
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_bin_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      e = cudaFuncSetAttribute(k_bin_scatter<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)(sizeof(int) * scan_slot(nbins(512))));
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
-  cudaError_t e = launch_k(k_bin_count, dim3(blocks, 1, count), dim3(256), hc, st, 0, s, tab);
-  if (e == cudaSuccess) e = launch_k(k_bin_scatter, dim3(blocks, 1, count), dim3(256), hs, st, 0, s, tab);
+  cudaError_t e = launch_k(k_bin_count<NT>, dim3(blocks, 1, count), dim3(NT), hc, st, 0, s, tab);
+  if (e == cudaSuccess) e = launch_k(k_bin_scatter<NT>, dim3(blocks, 1, count), dim3(NT), hs, st, 0, s, tab);
   return e;
+}
+
+cudaError_t launch_bin(const Solve& s, const Solve* tab, int count, int nmax, int r, cudaStream_t st) {
+  return r >= 256 ? launch_bin_t<1024>(s, tab, count, nmax, r, st) : launch_bin_t<256>(s, tab, count, nmax, r, st);
 }
 
 // dpoints = (sum of the two plane sides of the weight-derivative terms

@@ -115,3 +115,21 @@ def test_sparse_clouds_on_the_largest_grids(r):
         assert relmax(cpu(dp), cpu(rdp)) <= 1e-4 + slack and relmax(cpu(dn), cpu(rdn)) <= 1e-4 + slack, kind
         del ref, rdp, rdn
     plan.close()
+
+
+@pytest.mark.parametrize("n", [1023, 1025, 303105])
+def test_point_counts_at_the_edges_of_the_binning_blocks(n):
+    """r = 256: one point short of and past a block of 1 024, and past the
+    last point that the grid's blocks take one each (296 of them)."""
+    import torch
+    import bench
+    from gpu_util import relmax
+    from paper_2106_03452_gb300.dpsr import Plan
+    pts, nrm = (torch.from_numpy(x).cuda() for x in synth.sphere_cloud(synth.Rng(n), n))
+    plan = Plan(256, 2.0)
+    chi = plan.forward(pts, nrm)
+    assert plan.sync() == 0
+    with torch.no_grad():
+        ref = bench.torch_ops_dpsr(pts.double(), nrm.double(), 256, 2.0)
+    assert relmax(chi.cpu().numpy(), ref.cpu().numpy()) <= 1e-5
+    plan.close()
