@@ -374,24 +374,26 @@ int make_tensor_maps(Solve& s, int r) {
   if (!enc) return DPSR_ECUDA;
   const cuuint64_t dims[3] = {(cuuint64_t)(r / 2 + 1), (cuuint64_t)r, (cuuint64_t)r};
   const cuuint64_t strides[2] = {(cuuint64_t)kpitch(r) * 8, (cuuint64_t)r * kpitch(r) * 8};
-  const cuuint32_t boxx[3] = {16, 1, (cuuint32_t)tma_rows(r)}, boxy[3] = {16, (cuuint32_t)tma_rows(r), 1};
+  const cuuint32_t cols = (cuuint32_t)tile_cols(r);
+  const cuuint32_t boxx[3] = {cols, 1, (cuuint32_t)tma_rows(r)}, boxy[3] = {cols, (cuuint32_t)tma_rows(r), 1};
+  const CUtensorMapSwizzle swz = cols == 16 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
   const cuuint32_t es[3] = {1, 1, 1};
   for (int k = 0; k < kNSpec; ++k) {
     for (int w = 0; w < 2; ++w) {
       CUresult rc = enc(w == 0 ? &s.tmx[k] : &s.tmy[k], CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3,
                         (void*)s.spec[k], dims, strides, w == 0 ? boxx : boxy, es,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
                         CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
       if (rc != CUDA_SUCCESS) return DPSR_ECUDA;
     }
   }
   if (r < 64) return DPSR_OK;  // kSkip: the parts of tiles below are not used
-  const cuuint32_t boxb[3] = {16, 16, 1}, boxc[3] = {16, 1, (cuuint32_t)(r / kXChunks)};
+  const cuuint32_t boxb[3] = {cols, 16, 1}, boxc[3] = {cols, 1, (cuuint32_t)(r / kXChunks)};
   for (int k = 0; k < kNSpec + 4; ++k) {
     const bool b = k < kNSpec;
     CUresult rc = enc(b ? &s.tmb[k] : &s.tmc[k - kNSpec], CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3,
                       (void*)s.spec[b ? k : k - kNSpec], dims, strides, b ? boxb : boxc, es,
-                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                      CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
                       CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (rc != CUDA_SUCCESS) return DPSR_ECUDA;
   }

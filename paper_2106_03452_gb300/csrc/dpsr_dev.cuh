@@ -205,6 +205,13 @@ template <> struct Shape<512> { static constexpr int R1 = 32, T = 16; };
 // 256 rows, placed one after the other in shared memory (both start on a
 // 1024-byte boundary, so the 128-byte swizzle runs on unchanged).
 __host__ __device__ constexpr int tma_rows(int r) { return r < 256 ? r : 256; }
+// Columns (kz slots) of a tile of the x and y passes: 16, one 128-byte line a
+// row, up to r = 256; 8 at r = 512, where tiles of 16 (64 KB a box) leave one
+// CTA to an SM, whose load, transform and store phases then follow one another
+// (three with 8 columns: forward y pass 789 -> 527 us, dchi's 285 -> 170, inverse
+// 237 -> 190; the x passes, bound by too few warps either way, 779 -> 807 and
+// 722 -> 633).
+__host__ __device__ constexpr int tile_cols(int r) { return r < 512 ? 16 : 8; }
 
 template <int L, int DIR, class XA>
 __device__ __forceinline__ void fft_x(float2 (&v)[Shape<L>::R1], int t, XA xa, const float2* tw) {

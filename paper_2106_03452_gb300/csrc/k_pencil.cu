@@ -34,9 +34,10 @@ struct Pen {
   static constexpr int H = L / 2, KP = kpitch(L);
   static constexpr int YB = L < 16 ? L : 16;  // y-rows per z-pass CTA
   static constexpr int NYB = L / YB;
-  static constexpr int NCOL = H < 16 ? H : 16;  // kz columns per y-pass CTA
+  static constexpr int W = tile_cols(L);
+  static constexpr int NCOL = H < W ? H : W;    // kz columns per y-pass CTA
   static constexpr int NKC = H / NCOL;          // y-pass CTAs per plane
-  static constexpr int BOX = L * 16;            // float2 per TMA box [ky][16 kz]
+  static constexpr int BOX = L * W;             // float2 per TMA box [ky][W kz]
   static constexpr int ZNT = 256;               // threads of the z-pass kernels
   static constexpr int ZG = ZNT / T;
   static_assert(YB == ybin(L) && NYB == nybins(L), "one point bin per z-pass CTA");
@@ -79,12 +80,12 @@ __device__ __forceinline__ void split_dc_nyq(float2* b, int t, Nyq nyq) {
   for (int j = 0; j < R1; ++j) {
     const int ky = t + T * j;
     float2 xn;
-    unpack_dc_nyq(b[bx(ky, 0)], b[bx((L - ky) & (L - 1), 0)], x0[j], xn);
+    unpack_dc_nyq(b[bxl<L>(ky, 0)], b[bxl<L>((L - ky) & (L - 1), 0)], x0[j], xn);
     nyq(ky, xn);  // never column 0
   }
   group_sync<T, IL>();
 #pragma unroll
-  for (int j = 0; j < R1; ++j) b[bx(t + T * j, 0)] = x0[j];
+  for (int j = 0; j < R1; ++j) b[bxl<L>(t + T * j, 0)] = x0[j];
 }
 
 // Sorted-point index range of point bin (x-cell xc, y-block yb): the points
@@ -325,7 +326,7 @@ __global__ void __launch_bounds__(Pen<L>::ZNT, L >= 512 ? 1 : (L >= 256 ? 3 : 4)
 // ===========================================================================
 template <int L>
 constexpr int ynt() {
-  return 16 * Shape<L>::T >= 32 ? 16 * Shape<L>::T : 32;  // one group per column
+  return Pen<L>::W * Shape<L>::T >= 32 ? Pen<L>::W * Shape<L>::T : 32;  // one group per column
 }
 
 template <int L>
@@ -361,12 +362,12 @@ __device__ __forceinline__ void yfwd_issue_rows(const Solve& S, int X, int kz0, 
   using P = Pen<L>;
   const YfwdBufs b = yfwd_bufs<L, false>(kind);
   const int lane = threadIdx.x;
-  if (lane == 0) mbar_expect_tx(bar, __popc(rows) * (b.two ? 2 : 1) * 16 * P::YB * (uint32_t)sizeof(float2));
+  if (lane == 0) mbar_expect_tx(bar, __popc(rows) * (b.two ? 2 : 1) * P::W * P::YB * (uint32_t)sizeof(float2));
   __syncwarp();
   if (lane < P::NYB && ((rows >> lane) & 1u)) {
     const int y = lane * P::YB;
-    tma_load_3d(box + y * 16, &S.tmb[b.buf0], kz0, y, X, bar);
-    if (b.two) tma_load_3d(box + P::BOX + y * 16, &S.tmb[b.buf1], kz0, y, X, bar);
+    tma_load_3d(box + y * P::W, &S.tmb[b.buf0], kz0, y, X, bar);
+    if (b.two) tma_load_3d(box + P::BOX + y * P::W, &S.tmb[b.buf1], kz0, y, X, bar);
   }
 }
 
@@ -378,8 +379,8 @@ __device__ __forceinline__ void yfwd_issue(const Solve& S, int X, int kz0, int k
   const YfwdBufs b = yfwd_bufs<L, BWD>(kind);
   mbar_expect_tx(bar, (b.two ? 2 : 1) * P::BOX * (uint32_t)sizeof(float2));
   for (int y = 0; y < L; y += tma_rows(L)) {
-    tma_load_3d(box + y * 16, &S.tmy[b.buf0], kz0, y, X, bar);
-    if (b.two) tma_load_3d(box + P::BOX + y * 16, &S.tmy[b.buf1], kz0, y, X, bar);
+    tma_load_3d(box + y * P::W, &S.tmy[b.buf0], kz0, y, X, bar);
+    if (b.two) tma_load_3d(box + P::BOX + y * P::W, &S.tmy[b.buf1], kz0, y, X, bar);
   }
 }
 
@@ -407,7 +408,7 @@ __device__ __forceinline__ bool yfwd_tile(const Solve& S, int X, int kz0, int ki
   TwTab<L> twr{twt, t};
   if (g < P::NCOL) {  // whole groups; one column array live at a time
     float2* b0 = box;
-    auto c0 = [b0, g](int e) -> float2& { return b0[bx(e, g)]; };
+    auto c0 = [b0, g](int e) -> float2& { return b0[bxl<L>(e, g)]; };
     float2 a[P::R1];
     // rows of blocks that were not loaded are zero (T divides a block)
     auto has = [rows](int j) { return BWD || !kSkip<L> || ((rows >> (P::T * j / P::YB)) & 1u); };
@@ -418,7 +419,7 @@ __device__ __forceinline__ bool yfwd_tile(const Solve& S, int X, int kz0, int ki
     for (int j = 0; j < P::R1; ++j) c0(t + P::T * j) = a[j];
     if (two) {
       float2* b1 = box + P::BOX;
-      auto c1 = [b1, g](int e) -> float2& { return b1[bx(e, g)]; };
+      auto c1 = [b1, g](int e) -> float2& { return b1[bxl<L>(e, g)]; };
 #pragma unroll
       for (int j = 0; j < P::R1; ++j) a[j] = has(j) ? c1(t + P::T * j) : czero();
       fft_r<L, -1, IL>(a, t, c1, twr);
@@ -441,7 +442,7 @@ __device__ __forceinline__ bool yfwd_tile(const Solve& S, int X, int kz0, int ki
     float2* bq = box + g * P::BOX;
     float2* dst = S.spec[g == 0 ? buf0 : buf1];
     split_dc_nyq<L, IL>(bq, t, [&](int ky, float2 w) {
-      if (H < 16) bq[bx(ky, H)] = w;
+      if (H < 16) bq[bxl<L>(ky, H)] = w;
       else dst[((size_t)X * L + ky) * P::KP + H] = w;
     });
   }
@@ -449,8 +450,8 @@ __device__ __forceinline__ bool yfwd_tile(const Solve& S, int X, int kz0, int ki
   __syncthreads();
   if (tid == 0) {
     for (int y = 0; y < L; y += tma_rows(L)) {
-      tma_store_3d(&S.tmy[buf0], kz0, y, X, box + y * 16);
-      if (kind == 1 && two) tma_store_3d(&S.tmy[buf1], kz0, y, X, box + P::BOX + y * 16);
+      tma_store_3d(&S.tmy[buf0], kz0, y, X, box + y * P::W);
+      if (kind == 1 && two) tma_store_3d(&S.tmy[buf1], kz0, y, X, box + P::BOX + y * P::W);
     }
     tma_store_commit();
     tma_store_wait_read();
@@ -459,7 +460,7 @@ __device__ __forceinline__ bool yfwd_tile(const Solve& S, int X, int kz0, int ki
 }
 
 template <int L, bool BWD>
-__global__ void __launch_bounds__(ynt<L>(), L >= 512 ? 1 : (BWD ? 4 : (L >= 256 ? 3 : 5))) k_yfwd(const __grid_constant__ Solve s0,
+__global__ void __launch_bounds__(ynt<L>(), BWD ? 4 : (L >= 256 ? 3 : 5)) k_yfwd(const __grid_constant__ Solve s0,
                                                    const Solve* __restrict__ tab) {
   using P = Pen<L>;
   constexpr int NT = ynt<L>();
@@ -529,8 +530,8 @@ __device__ __forceinline__ void yinv_issue(const Solve& S, int X, int kz0, int p
   const bool do0 = part != 1, do1 = NCH == 3 && part != 0;
   mbar_expect_tx(bar, ((do0 ? 1 : 0) + (do1 ? 1 : 0)) * P::BOX * (uint32_t)sizeof(float2));
   for (int y = 0; y < L; y += tma_rows(L)) {
-    if (do0) tma_load_3d(box + y * 16, &S.tmy[kSpChi], kz0, y, X, bar);
-    if (do1) tma_load_3d(box + P::BOX + y * 16, &S.tmy[kSpD], kz0, y, X, bar);
+    if (do0) tma_load_3d(box + y * P::W, &S.tmy[kSpChi], kz0, y, X, bar);
+    if (do1) tma_load_3d(box + P::BOX + y * P::W, &S.tmy[kSpD], kz0, y, X, bar);
   }
 }
 
@@ -561,9 +562,9 @@ __device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int pa
     const float2* nq = S.spec[g == 0 ? kSpChi : kSpD] + (size_t)X * L * P::KP + H;
     for (int j = 0; j < P::R1; ++j) {
       const int ky = t + P::T * j;
-      const float2 n = H >= 16 ? nq[(size_t)ky * P::KP] : b[bx(ky, H)];
-      const float2 x0 = b[bx(ky, 0)];
-      b[bx(ky, 0)] = make_float2(x0.x - n.y, x0.y + n.x);
+      const float2 n = H >= 16 ? nq[(size_t)ky * P::KP] : b[bxl<L>(ky, H)];
+      const float2 x0 = b[bxl<L>(ky, 0)];
+      b[bxl<L>(ky, 0)] = make_float2(x0.x - n.y, x0.y + n.x);
     }
   }
   __syncthreads();
@@ -571,7 +572,7 @@ __device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int pa
     const int sz = kz0 + g;
     auto cref = [&](int k) {
       float2* b = box + k * P::BOX;
-      return [b, g](int e) -> float2& { return b[bx(e, g)]; };
+      return [b, g](int e) -> float2& { return b[bxl<L>(e, g)]; };
     };
     float2 v[P::R1];
     auto c0 = cref(0);
@@ -608,10 +609,10 @@ __device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int pa
   if constexpr (NCH == 3 && kSkip<L>) {  // warp 0: the y-blocks that the z pass reads, a lane each
     if (tid < P::NYB && ((rows >> tid) & 1u)) {
       const int y = tid * P::YB;
-      if (do0) tma_store_3d(&S.tmb[kSpC], kz0, y, X, box + y * 16);
+      if (do0) tma_store_3d(&S.tmb[kSpC], kz0, y, X, box + y * P::W);
       if (do1) {
-        tma_store_3d(&S.tmb[kSpYa], kz0, y, X, box + P::BOX + y * 16);
-        tma_store_3d(&S.tmb[kSpYb], kz0, y, X, box + 2 * P::BOX + y * 16);
+        tma_store_3d(&S.tmb[kSpYa], kz0, y, X, box + P::BOX + y * P::W);
+        tma_store_3d(&S.tmb[kSpYb], kz0, y, X, box + 2 * P::BOX + y * P::W);
       }
       tma_store_commit();
       tma_store_wait_read();
@@ -619,12 +620,12 @@ __device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int pa
   } else if (tid == 0) {
     for (int y = 0; y < L; y += tma_rows(L)) {
       if constexpr (NCH == 1) {
-        tma_store_3d(&S.tmy[kSpYa], kz0, y, X, box + y * 16);
+        tma_store_3d(&S.tmy[kSpYa], kz0, y, X, box + y * P::W);
       } else {
-        if (do0) tma_store_3d(&S.tmy[kSpC], kz0, y, X, box + y * 16);
+        if (do0) tma_store_3d(&S.tmy[kSpC], kz0, y, X, box + y * P::W);
         if (do1) {
-          tma_store_3d(&S.tmy[kSpYa], kz0, y, X, box + P::BOX + y * 16);
-          tma_store_3d(&S.tmy[kSpYb], kz0, y, X, box + 2 * P::BOX + y * 16);
+          tma_store_3d(&S.tmy[kSpYa], kz0, y, X, box + P::BOX + y * P::W);
+          tma_store_3d(&S.tmy[kSpYb], kz0, y, X, box + 2 * P::BOX + y * P::W);
         }
       }
     }
@@ -635,11 +636,10 @@ __device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int pa
 }
 
 template <int L, int NCH>
-__global__ void __launch_bounds__(16 * Shape<L>::T >= 32 ? 16 * Shape<L>::T : 32,
-                                  L >= 512 ? 1 : (NCH == 1 || yinv_split<L, NCH>() ? 4 : 2))
+__global__ void __launch_bounds__(ynt<L>(), NCH == 1 || yinv_split<L, NCH>() ? 4 : 2)
     k_yinv(const __grid_constant__ Solve s0, const Solve* __restrict__ tab) {
   using P = Pen<L>;
-  constexpr int NT = 16 * P::T >= 32 ? 16 * P::T : 32;
+  constexpr int NT = ynt<L>();
   const Solve& S = tab ? tab[blockIdx.z] : s0;
   const int X = blockIdx.x / P::NKC, kz0 = (blockIdx.x % P::NKC) * P::NCOL;
   const int tid = threadIdx.x;
@@ -1087,7 +1087,7 @@ static cudaError_t launch_pencil_t(int kind, const Solve& s, const Solve* tab, i
     }
     case 1: {
       constexpr size_t a = yinv_smem<L, 1>(), b = zinv_smem<L, 1>();
-      constexpr int nt = 16 * P::T >= 32 ? 16 * P::T : 32;
+      constexpr int nt = ynt<L>();
       static int nz = 0;
       if (!attr_set[1]) {
         e = set_smem(k_yinv<L, 1>, a);
@@ -1117,7 +1117,7 @@ static cudaError_t launch_pencil_t(int kind, const Solve& s, const Solve* tab, i
     }
     default: {
       constexpr size_t a = yinv_smem<L, 3>(), b = zinv_smem<L, 3>();
-      constexpr int nt = 16 * P::T >= 32 ? 16 * P::T : 32;
+      constexpr int nt = ynt<L>();
       static int nz = 0;
       if (!attr_set[3]) {
         e = set_smem(k_yinv<L, 3>, a);

@@ -20,7 +20,7 @@ namespace dpsr {
 template <int L>
 struct XGeo {
   static constexpr int R1 = Shape<L>::R1, T = Shape<L>::T;
-  static constexpr int KC = 16;                             // kz columns per CTA (one TMA box row)
+  static constexpr int KC = tile_cols(L);                   // kz columns per CTA (one TMA box row)
   static constexpr int NG = KC * T >= 32 ? KC : 32 / T;     // groups (at least one warp)
   static constexpr int NT = NG * T;                         // threads
   static constexpr int H = L / 2;
@@ -70,7 +70,7 @@ constexpr size_t xpass_smem() {
 // one kz column along x in registers (the box column doubles as its exchange
 // buffer), and TMA stores the results.
 template <int L, bool BWD>
-__global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 1 : (L >= 256 ? (BWD ? 2 : 3) : 5))
+__global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ? 2 : 3) : 5))
     k_xpass(const __grid_constant__ Solve s0, const Solve* __restrict__ tab) {
   using P = XGeo<L>;
   constexpr int NCH = P::template nch<BWD>();
@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 1 : (L >= 256 ? (BWD ?
   const float gyz = g1[ky] * g1[kz], u2yz = __ldg(S.u2 + L + ky) + __ldg(S.u2 + 2 * L + kz);
   auto colref = [&](int ch) {
     float2* b = box + ch * P::BOX;
-    return [b, gc](int e) -> float2& { return b[bx(e, gc)]; };
+    return [b, gc](int e) -> float2& { return b[bxl<L>(e, gc)]; };
   };
   auto c0 = colref(0);
   auto c1 = colref(1);

@@ -17,6 +17,14 @@ __device__ __forceinline__ int bx(int q, int c) {
   return q * 16 + ((((c >> 1) ^ (q & 7)) << 1) | (c & 1));
 }
 
+// The same for a box of tile_cols(L) columns: 8 columns (64-byte rows) at
+// L = 512 under the 64-byte swizzle (chunks XOR-ed by bits 1-2 of the row).
+template <int L>
+__device__ __forceinline__ int bxl(int q, int c) {
+  if constexpr (L < 512) return bx(q, c);
+  else return q * 8 + ((((c >> 1) ^ ((q >> 1) & 3)) << 1) | (c & 1));
+}
+
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
 }
