@@ -1,0 +1,92 @@
+// A column of a swizzled TMA box (see bxl) as one thread of its FFT group sees
+// it: its own elements t + T j, and the group FFT's exchange in place.
+//
+// An exchange index is k1 T + (t ^ k1 mod T), and the swizzle XORs a row's low
+// bits into its address as well, so the address of exchange step k1 is the
+// thread's own (row t) XOR a constant, plus a constant: one logic operation an
+// access where the general index arithmetic takes four or five. The column
+// passes issue some 100 such accesses per transform next to 400 FP32
+// operations, and are bound by issue slots as much as by HBM.
+#pragma once
+
+#include "dpsr_dev.cuh"
+#include "tma.cuh"
+
+namespace dpsr {
+
+// Alignment of the boxes: the bits that the XOR touches (T rows) must be the
+// box offset's own.
+template <int L>
+constexpr int box_align() {
+  return Shape<L>::T * tile_cols(L) * 8 > 1024 ? Shape<L>::T * tile_cols(L) * 8 : 1024;
+}
+
+template <int L, bool FAST = (Shape<L>::T >= 8)>
+struct Col {  // T a multiple of the swizzle's 8 rows: rows t + T j share row t's pattern
+  static constexpr int T = Shape<L>::T, RB = tile_cols(L) * 8;  // row bytes
+  uint32_t p, px;  // row t; exchange row t T + t
+  __device__ __forceinline__ Col(const float2* box, int t, int c) {
+    p = smem_u32(box) + (uint32_t)bxl<L>(t, c) * 8u;
+    px = p + (uint32_t)t * (T * RB);
+  }
+  // XOR of rows s and s ^ k (k < T): the row's offset and its swizzled chunk
+  static __device__ __forceinline__ constexpr uint32_t flip(int k) {
+    return (uint32_t)(k * RB | (RB == 128 ? (k & 7) << 4 : ((k >> 1) & 3) << 4));
+  }
+  static __device__ __forceinline__ float2 ld(uint32_t a) {
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+    return v;
+  }
+  static __device__ __forceinline__ void st(uint32_t a, float2 v) {
+    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+  }
+  __device__ __forceinline__ float2 get(int j) const { return ld(p + j * (T * RB)); }
+  __device__ __forceinline__ void put(int j, float2 v) const { st(p + j * (T * RB), v); }
+  __device__ __forceinline__ void xput(int k1, float2 v) const { st((p ^ flip(k1 % T)) + k1 * (T * RB), v); }
+  __device__ __forceinline__ float2 xget(int m, int n2) const { return ld((px ^ flip(n2)) + m * (T * T * RB)); }
+};
+
+template <int L>
+struct Col<L, false> {
+  static constexpr int T = Shape<L>::T;
+  float2* b;
+  int t, c;
+  __device__ __forceinline__ Col(float2* box, int t_, int c_) : b(box), t(t_), c(c_) {}
+  __device__ __forceinline__ float2 get(int j) const { return b[bxl<L>(t + T * j, c)]; }
+  __device__ __forceinline__ void put(int j, float2 v) const { b[bxl<L>(t + T * j, c)] = v; }
+  __device__ __forceinline__ void xput(int k1, float2 v) const { b[bxl<L>(k1 * T + (t ^ (k1 % T)), c)] = v; }
+  __device__ __forceinline__ float2 xget(int m, int n2) const { return b[bxl<L>((t + T * m) * T + (n2 ^ t), c)]; }
+};
+
+// The group FFT of fft_r with its exchange in a box column.
+template <int L, int DIR, bool IL>
+__device__ __forceinline__ void fft_c(float2 (&v)[Shape<L>::R1], const Col<L>& col, const TwTab<L>& tw) {
+  constexpr int R1 = Shape<L>::R1, T = Shape<L>::T, M = R1 / T;
+  if constexpr (T == 1) {
+    Dft<L, DIR>::run(v);
+  } else {
+    Dft<R1, DIR>::run(v);
+#pragma unroll
+    for (int k1 = 1; k1 < R1; ++k1) {
+      float2 w = tw(k1);
+      if (DIR > 0) w.y = -w.y;
+      v[k1] = cmul(v[k1], w);
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < R1; ++k1) col.xput(k1, v[k1]);
+    group_sync<T, IL>();
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+      float2 u[T];
+#pragma unroll
+      for (int n2 = 0; n2 < T; ++n2) u[n2] = col.xget(m, n2);
+      Dft<T, DIR>::run(u);
+#pragma unroll
+      for (int k2 = 0; k2 < T; ++k2) v[m + M * k2] = u[k2];
+    }
+    group_sync<T, IL>();
+  }
+}
+
+}  // namespace dpsr

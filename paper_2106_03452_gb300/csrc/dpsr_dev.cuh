@@ -167,8 +167,8 @@ __device__ __forceinline__ void group_sync() {
 // Two Cooley-Tukey stages L = R1 * T: an R1-point DFT per thread over the
 // stride-T subsequence, a twiddle W_L^(t*k1), an exchange through shared
 // memory (XOR-swizzled so neither side conflicts), and T-point DFTs.
-// tw[m] = exp(-2 pi i m / L), m < L (FP64-computed, rounded to FP32).
-// xch: L float2 of shared memory owned by the group. Every lane of the warp
+// tw(k1): the thread's stage twiddle (TwTab). xa(i): L float2 of shared memory
+// owned by the group. Every lane of the warp
 // must call this together (they synchronise through group_sync).
 // ---------------------------------------------------------------------------
 // Group and lane-in-group of thread tid. Contiguous: group g holds lanes
@@ -213,66 +213,18 @@ __host__ __device__ constexpr int tma_rows(int r) { return r < 256 ? r : 256; }
 // 722 -> 633).
 __host__ __device__ constexpr int tile_cols(int r) { return r < 512 ? 16 : 8; }
 
-template <int L, int DIR, class XA>
-__device__ __forceinline__ void fft_x(float2 (&v)[Shape<L>::R1], int t, XA xa, const float2* tw) {
-  constexpr int R1 = Shape<L>::R1, T = Shape<L>::T;
-  if constexpr (T == 1) {
-    Dft<L, DIR>::run(v);
-  } else {
-    Dft<R1, DIR>::run(v);
-#pragma unroll
-    for (int k1 = 1; k1 < R1; ++k1) {
-      float2 w = tw[t * k1];
-      if (DIR > 0) w.y = -w.y;
-      v[k1] = cmul(v[k1], w);
-    }
-#pragma unroll
-    for (int k1 = 0; k1 < R1; ++k1) xa(k1 * T + (t ^ (k1 % T))) = v[k1];
-    group_sync<T>();
-    constexpr int M = R1 / T;
-#pragma unroll
-    for (int m = 0; m < M; ++m) {
-      float2 u[T];
-      const int k1 = t + T * m;
-#pragma unroll
-      for (int n2 = 0; n2 < T; ++n2) u[n2] = xa(k1 * T + (n2 ^ t));
-      Dft<T, DIR>::run(u);
-#pragma unroll
-      for (int k2 = 0; k2 < T; ++k2) v[m + M * k2] = u[k2];
-    }
-    group_sync<T>();
-  }
-}
-
-template <int L, int DIR>
-__device__ __forceinline__ void fft(float2 (&v)[Shape<L>::R1], int t, float2* xch,
-                                    const float2* tw) {
-  fft_x<L, DIR>(v, t, [xch](int i) -> float2& { return xch[i]; }, tw);
-}
-
-// The stage twiddles W_L^(t*k1), k1 = 1..R1-1, of thread t held in registers
-// (the same for every transform the thread performs).
-template <int L>
-struct Twid {
-  float2 w[Shape<L>::R1];
-  __device__ __forceinline__ void load(int t, const float2* tw) {
-#pragma unroll
-    for (int k1 = 0; k1 < Shape<L>::R1; ++k1)
-      w[k1] = Shape<L>::T == 1 ? make_float2(1.f, 0.f) : tw[(t * k1) & (L - 1)];
-  }
-  __device__ __forceinline__ float2 operator()(int k1) const { return w[k1]; }
-};
-
-// The same stage twiddles read from a shared-memory table at each use
-// (fewer live registers than Twid).
+// The stage twiddles W_L^(t*k1) of thread t, read from a shared-memory copy of
+// Solve::tw at each use: entry k1 T + t, so that a group's lanes read
+// consecutive entries (with exp(-2 pi i m / L) at entry m instead, the even k1
+// are bank conflicts, eight-fold at k1 = 8) at constant offsets.
 template <int L>
 struct TwTab {
-  const float2* tab;  // exp(-2 pi i m / L), m < L, in shared memory
+  const float2* tab;
   int t;
-  __device__ __forceinline__ float2 operator()(int k1) const { return tab[(t * k1) & (L - 1)]; }
+  __device__ __forceinline__ float2 operator()(int k1) const { return tab[k1 * Shape<L>::T + t]; }
 };
 
-// Group FFT with register twiddles (see fft_x).
+// The group FFT over an exchange area that xa(i) addresses.
 template <int L, int DIR, bool IL = false, class XA, class TW>
 __device__ __forceinline__ void fft_r(float2 (&v)[Shape<L>::R1], int t, XA xa, const TW& tw) {
   constexpr int R1 = Shape<L>::R1, T = Shape<L>::T;
@@ -450,7 +402,7 @@ struct Solve {
   float4* part;     // per-block partial sums, float-float pairs (a.hi, a.lo, b.hi, b.lo)
   Scalars* sc;
   unsigned* status;
-  const float2* tw;  // r
+  const float2* tw;  // r: stage twiddles exp(-2 pi i t k1 / r) at k1 T + t (see TwTab)
   // Spectral tables, indexed by the integer frequency index k of an axis
   // (f = k below r/2, k - r above, |f| = r/2 at Nyquist):
   const float* g1;   // r: exp(-2 sigma^2 f^2 / r^2), the same on every axis
@@ -458,13 +410,17 @@ struct Solve {
   const float* iu;   // 3 x r, axis-major: f / L_d, 0 at Nyquist (spectral derivative)
 };
 
+// Threads of a group FFT (Shape<r>::T), for the host.
+inline int group_threads(int r) { return r <= 16 ? 1 : (r == 32 ? 4 : (r <= 128 ? 8 : 16)); }
+
 // Host side: the spectral tables of one plan, computed in FP64 and rounded
-// to FP32. tw[r]: twiddles exp(-2 pi i m / r); tab[7r]: g1 (r), u2 (3r) and
+// to FP32. tw[r]: twiddles exp(-2 pi i t k1 / r) at k1 T + t; tab[7r]: g1 (r), u2 (3r) and
 // iu (3r) as laid out in Solve. box: side lengths L_d (nullptr: unit cube).
 inline void spectral_tables(int r, double sigma, const double* box, float2* tw, float* tab) {
   const double pi = 3.14159265358979323846264338327950288;
   for (int m = 0; m < r; ++m) {
-    const double ang = -2.0 * pi * (double)m / (double)r;
+    const int T = group_threads(r);
+    const double ang = -2.0 * pi * (double)((m % T) * (m / T) % r) / (double)r;
     tw[m] = make_float2((float)cos(ang), (float)sin(ang));
     const double f = m < r / 2 ? (double)m : (m == r / 2 ? (double)(r / 2) : (double)(m - r));
     tab[m] = (float)exp(-2.0 * sigma * sigma * f * f / ((double)r * r));

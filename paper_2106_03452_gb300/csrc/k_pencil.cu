@@ -21,6 +21,7 @@
 //
 // Half spectra along z are stored "packed" between the passes: slot 0 holds
 // the DC and Nyquist terms of a real row as one complex number.
+#include "col.cuh"
 #include "dpsr_dev.cuh"
 #include "finalize.cuh"
 #include "launch.h"
@@ -336,7 +337,7 @@ constexpr bool yfwd_merge() {
 
 template <int L, bool BWD>
 constexpr size_t yfwd_smem() {
-  return 1024 + sizeof(float2) * ((size_t)(BWD ? 1 : 2) * Pen<L>::BOX + L) + sizeof(float) * L;
+  return box_align<L>() + sizeof(float2) * ((size_t)(BWD ? 1 : 2) * Pen<L>::BOX + L) + sizeof(float) * L;
 }
 
 // Input buffers of a y-pass tile of kind `kind` (see k_yfwd): box 0 holds
@@ -407,31 +408,29 @@ __device__ __forceinline__ bool yfwd_tile(const Solve& S, int X, int kz0, int ki
   }
   TwTab<L> twr{twt, t};
   if (g < P::NCOL) {  // whole groups; one column array live at a time
-    float2* b0 = box;
-    auto c0 = [b0, g](int e) -> float2& { return b0[bxl<L>(e, g)]; };
+    const Col<L> c0(box, t, g);
     float2 a[P::R1];
     // rows of blocks that were not loaded are zero (T divides a block)
     auto has = [rows](int j) { return BWD || !kSkip<L> || ((rows >> (P::T * j / P::YB)) & 1u); };
 #pragma unroll
-    for (int j = 0; j < P::R1; ++j) a[j] = has(j) ? c0(t + P::T * j) : czero();
-    fft_r<L, -1, IL>(a, t, c0, twr);
+    for (int j = 0; j < P::R1; ++j) a[j] = has(j) ? c0.get(j) : czero();
+    fft_c<L, -1, IL>(a, c0, twr);
 #pragma unroll
-    for (int j = 0; j < P::R1; ++j) c0(t + P::T * j) = a[j];
+    for (int j = 0; j < P::R1; ++j) c0.put(j, a[j]);
     if (two) {
-      float2* b1 = box + P::BOX;
-      auto c1 = [b1, g](int e) -> float2& { return b1[bxl<L>(e, g)]; };
+      const Col<L> c1(box + P::BOX, t, g);
 #pragma unroll
-      for (int j = 0; j < P::R1; ++j) a[j] = has(j) ? c1(t + P::T * j) : czero();
-      fft_r<L, -1, IL>(a, t, c1, twr);
+      for (int j = 0; j < P::R1; ++j) a[j] = has(j) ? c1.get(j) : czero();
+      fft_c<L, -1, IL>(a, c1, twr);
       if (kind == 0) {  // D = FFT(i u_z v_z) + i u_y FFT(v_y); this lane wrote c0 above
 #pragma unroll
         for (int j = 0; j < P::R1; ++j) {
           const int ky = t + P::T * j;
-          c0(ky) = cadd(a[j], cmul_iu(c0(ky), iu[ky]));
+          c0.put(j, cadd(a[j], cmul_iu(c0.get(j), iu[ky])));
         }
       } else {
 #pragma unroll
-        for (int j = 0; j < P::R1; ++j) c1(t + P::T * j) = a[j];
+        for (int j = 0; j < P::R1; ++j) c1.put(j, a[j]);
       }
     }
   }
@@ -469,7 +468,8 @@ __global__ void __launch_bounds__(ynt<L>(), BWD ? 4 : (L >= 256 ? 3 : 5)) k_yfwd
   const int kind = BWD ? 3 : (int)blockIdx.y;
   const int tid = threadIdx.x;
   extern __shared__ unsigned char smem_raw[];
-  const uint32_t pad = (1024u - (smem_u32(smem_raw) & 1023u)) & 1023u;
+  constexpr uint32_t AL = box_align<L>();
+  const uint32_t pad = (AL - (smem_u32(smem_raw) & (AL - 1u))) & (AL - 1u);
   float2* box = reinterpret_cast<float2*>(smem_raw + pad);  // 1 or 2 boxes
   float2* twt = box + (BWD ? 1 : 2) * P::BOX;
   float* iu = reinterpret_cast<float*>(twt + L);
@@ -516,7 +516,7 @@ constexpr bool yinv_split() {
 
 template <int L, int NCH>
 constexpr size_t yinv_smem() {
-  return 1024 + sizeof(float2) * ((size_t)NCH * Pen<L>::BOX + L) + sizeof(float) * L;
+  return box_align<L>() + sizeof(float2) * ((size_t)NCH * Pen<L>::BOX + L) + sizeof(float) * L;
 }
 
 // Thread 0: the TMA tile loads of an inverse y-pass tile (part: -1 all
@@ -570,38 +570,35 @@ __device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int pa
   __syncthreads();
   if (g < P::NCOL) {
     const int sz = kz0 + g;
-    auto cref = [&](int k) {
-      float2* b = box + k * P::BOX;
-      return [b, g](int e) -> float2& { return b[bxl<L>(e, g)]; };
-    };
+    auto cref = [&](int k) { return Col<L>(box + k * P::BOX, t, g); };
     float2 v[P::R1];
-    auto c0 = cref(0);
+    const auto c0 = cref(0);
     if (do0) {
 #pragma unroll
-      for (int j = 0; j < P::R1; ++j) v[j] = c0(t + P::T * j);
-      fft_r<L, +1, IL>(v, t, c0, twr);
+      for (int j = 0; j < P::R1; ++j) v[j] = c0.get(j);
+      fft_c<L, +1, IL>(v, c0, twr);
 #pragma unroll
-      for (int j = 0; j < P::R1; ++j) c0(t + P::T * j) = v[j];
+      for (int j = 0; j < P::R1; ++j) c0.put(j, v[j]);
     }
     if (do1) {
-      auto c1 = cref(1);
-      auto c2 = cref(2);
+      const auto c1 = cref(1);
+      const auto c2 = cref(2);
 #pragma unroll
       for (int j = 0; j < P::R1; ++j) {
-        v[j] = c1(t + P::T * j);
-        c2(t + P::T * j) = v[j];
+        v[j] = c1.get(j);
+        c2.put(j, v[j]);
         v[j] = cmul_iu(v[j], -iu[t + P::T * j]);
       }
-      fft_r<L, +1, IL>(v, t, c1, twr);
+      fft_c<L, +1, IL>(v, c1, twr);
 #pragma unroll
-      for (int j = 0; j < P::R1; ++j) c1(t + P::T * j) = v[j];
+      for (int j = 0; j < P::R1; ++j) c1.put(j, v[j]);
       group_sync<P::T, IL>();
 #pragma unroll
-      for (int j = 0; j < P::R1; ++j) v[j] = c2(t + P::T * j);
-      fft_r<L, +1, IL>(v, t, c2, twr);
+      for (int j = 0; j < P::R1; ++j) v[j] = c2.get(j);
+      fft_c<L, +1, IL>(v, c2, twr);
       const float ez = sz == 0 ? 0.f : -__ldg(S.iu + 2 * L + sz);  // z axis
 #pragma unroll
-      for (int j = 0; j < P::R1; ++j) c2(t + P::T * j) = cmul_iu(v[j], ez);
+      for (int j = 0; j < P::R1; ++j) c2.put(j, cmul_iu(v[j], ez));
     }
   }
   fence_async_smem();
@@ -644,7 +641,8 @@ __global__ void __launch_bounds__(ynt<L>(), NCH == 1 || yinv_split<L, NCH>() ? 4
   const int X = blockIdx.x / P::NKC, kz0 = (blockIdx.x % P::NKC) * P::NCOL;
   const int tid = threadIdx.x;
   extern __shared__ unsigned char smem_raw[];
-  const uint32_t pad = (1024u - (smem_u32(smem_raw) & 1023u)) & 1023u;
+  constexpr uint32_t AL = box_align<L>();
+  const uint32_t pad = (AL - (smem_u32(smem_raw) & (AL - 1u))) & (AL - 1u);
   float2* box = reinterpret_cast<float2*>(smem_raw + pad);
   float2* twt = box + NCH * P::BOX;
   float* iu = reinterpret_cast<float*>(twt + L);

@@ -10,6 +10,7 @@
 // Backward: F = G(k) (g_a FFT(dchi) + g_s + g_w W~);  Q1 = IFFT_x(F),
 //           Q2 = IFFT_x(-i u_x F)  (the adjoint of Eq. 3, conj(H_a) = -H_a).
 // Three FFTs of length r per column in each direction.
+#include "col.cuh"
 #include "dpsr_dev.cuh"
 #include "launch.h"
 #include "finalize.cuh"
@@ -46,23 +47,11 @@ __device__ __forceinline__ float spectral_G(int kx, float gyz, float u2yz, const
   return __fdividef(g1[kx] * gyz, -6.28318530717958647692f * s);
 }
 
-// Stage twiddles of the thread (see Twid / TwTab).
-template <int L, class Tw>
-__device__ __forceinline__ Tw make_tw(const float2* tw, int t) {
-  if constexpr (std::is_same<Tw, Twid<L>>::value) {
-    Tw w;
-    w.load(t, tw);
-    return w;
-  } else {
-    return Tw{tw, t};
-  }
-}
-
 template <int L, bool BWD>
 constexpr size_t xpass_smem() {
   using P = XGeo<L>;
   constexpr int NCH = P::template nch<BWD>();
-  return 1024 + sizeof(float2) * ((size_t)NCH * P::BOX + L) + 3 * sizeof(float) * L;
+  return box_align<L>() + sizeof(float2) * ((size_t)NCH * P::BOX + L) + 3 * sizeof(float) * L;
 }
 
 // One CTA per (kz tile of 16, ky): TMA loads the tiles [x][16 kz] of the
@@ -80,8 +69,9 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
   using LN = Lanes<P::T, IL>;
   const int tid = threadIdx.x, g = LN::group(tid), t = LN::lane(tid);
   extern __shared__ unsigned char smem_raw[];
-  const uint32_t pad = (1024u - (smem_u32(smem_raw) & 1023u)) & 1023u;
-  float2* box = reinterpret_cast<float2*>(smem_raw + pad);  // NCH boxes, 1024-aligned
+  constexpr uint32_t AL = box_align<L>();
+  const uint32_t pad = (AL - (smem_u32(smem_raw) & (AL - 1u))) & (AL - 1u);
+  float2* box = reinterpret_cast<float2*>(smem_raw + pad);  // NCH boxes
   float2* tw = box + NCH * P::BOX;
   float* g1 = reinterpret_cast<float*>(tw + L);
   float* u2 = g1 + L;
@@ -154,16 +144,10 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
   const bool valid = own && kz0 + g <= P::H;
   // shared-memory twiddles and one live column array: at r = 256 three CTAs
   // per SM forward (two backward, where three would spill), five below
-  using Tw = TwTab<L>;
-  Tw twr = make_tw<L, Tw>(tw, t);
+  const TwTab<L> twr{tw, t};
   // u2 in shared memory is the x axis' table; the y and z axes' come from global memory
   const float gyz = g1[ky] * g1[kz], u2yz = __ldg(S.u2 + L + ky) + __ldg(S.u2 + 2 * L + kz);
-  auto colref = [&](int ch) {
-    float2* b = box + ch * P::BOX;
-    return [b, gc](int e) -> float2& { return b[bxl<L>(e, gc)]; };
-  };
-  auto c0 = colref(0);
-  auto c1 = colref(1);
+  const Col<L> c0(box, t, gc), c1(box + P::BOX, t, gc);
   float2 a[P::R1];
   if constexpr (!BWD) {
     // Columns past Nyquist (the last kz tile) hold zeros and are not stored:
@@ -174,21 +158,21 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
       // FFT_x(D) goes back to its column, FFT_x(C) meets it there.
       box_wait(0);
 #pragma unroll
-      for (int j = 0; j < P::R1; ++j) a[j] = has(j) ? c0(t + P::T * j) : czero();
-      fft_r<L, -1, IL>(a, t, c0, twr);
+      for (int j = 0; j < P::R1; ++j) a[j] = has(j) ? c0.get(j) : czero();
+      fft_c<L, -1, IL>(a, c0, twr);
       if (own) {  // groups past the last column (tiny r) only shadow it
 #pragma unroll
-        for (int j = 0; j < P::R1; ++j) c0(t + P::T * j) = a[j];
+        for (int j = 0; j < P::R1; ++j) c0.put(j, a[j]);
       }
       box_wait(1);
 #pragma unroll
-      for (int j = 0; j < P::R1; ++j) a[j] = has(j) ? c1(t + P::T * j) : czero();
-      fft_r<L, -1, IL>(a, t, c1, twr);
+      for (int j = 0; j < P::R1; ++j) a[j] = has(j) ? c1.get(j) : czero();
+      fft_c<L, -1, IL>(a, c1, twr);
 #pragma unroll
       for (int j = 0; j < P::R1; ++j) {
         const int kx = t + P::T * j;  // this lane wrote c0(kx) above
         const float G = spectral_G(kx, gyz, u2yz, g1, u2);
-        a[j] = cscale(cadd(c0(kx), cmul_iu(a[j], iu[kx])), G);
+        a[j] = cscale(cadd(c0.get(j), cmul_iu(a[j], iu[kx])), G);
       }
     }
     if constexpr (!P::WL2) {
@@ -201,7 +185,7 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
       w_reload = true;
     }
     if (valid) {
-      fft_r<L, +1, IL>(a, t, c0, twr);  // P = unnormalised IFFT_x(chi~)
+      fft_c<L, +1, IL>(a, c0, twr);  // P = unnormalised IFFT_x(chi~)
       // Spectral sums of Eq. 4, by Parseval along x against the x-domain W~
       // (its tile, or up to r = 128 its column straight from L2):
       // sum_kx conj(W~(kx)) chi~(kx) = sum_x conj(W~_x(x)) P(x),
@@ -210,7 +194,7 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
         box_wait(1, 1u);
 #pragma unroll
         for (int j = 0; j < P::R1; ++j) {
-          const float2 w = has(j) ? c1(t + P::T * j) : czero();
+          const float2 w = has(j) ? c1.get(j) : czero();
           am += w.x * a[j].x + w.y * a[j].y;
         }
       } else {
@@ -225,7 +209,7 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
       wz = (kz == 0 || kz == P::H) ? 1.f : 2.f;
       if (own) {
 #pragma unroll
-        for (int j = 0; j < P::R1; ++j) c0(t + P::T * j) = a[j];
+        for (int j = 0; j < P::R1; ++j) c0.put(j, a[j]);
       }
     }
     FF fm = {am * wz, 0.f}, fs = {as * wz, 0.f};  // wz in {1, 2}: exact
@@ -256,10 +240,10 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
 #pragma unroll
     for (int j = 0; j < P::R1; ++j) {
       const int x = t + P::T * j;
-      a[j] = cadd(cscale(c0(x), ga), has(j) ? cscale(c1(x), gw) : czero());
+      a[j] = cadd(cscale(c0.get(j), ga), has(j) ? cscale(c1.get(j), gw) : czero());
       if (x == 0) a[j].x += gs;
     }
-    fft_r<L, -1, IL>(a, t, c0, twr);
+    fft_c<L, -1, IL>(a, c0, twr);
     {
       // F = G (.); Q2's input -i u_x F goes to the column of W~ (read above by
       // this group), Q1 = IFFT_x(F) is transformed from registers first
@@ -267,20 +251,20 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
       for (int j = 0; j < P::R1; ++j) {
         const int kx = t + P::T * j;
         a[j] = cscale(a[j], spectral_G(kx, gyz, u2yz, g1, u2));
-        if (own) c1(kx) = cmul_iu(a[j], -iu[kx]);
+        if (own) c1.put(j, cmul_iu(a[j], -iu[kx]));
       }
-      fft_r<L, +1, IL>(a, t, c0, twr);
+      fft_c<L, +1, IL>(a, c0, twr);
       if (own) {
 #pragma unroll
-        for (int j = 0; j < P::R1; ++j) c0(t + P::T * j) = a[j];
+        for (int j = 0; j < P::R1; ++j) c0.put(j, a[j]);
       }
       group_sync<P::T, IL>();
 #pragma unroll
-      for (int j = 0; j < P::R1; ++j) a[j] = c1(t + P::T * j);
-      fft_r<L, +1, IL>(a, t, c1, twr);
+      for (int j = 0; j < P::R1; ++j) a[j] = c1.get(j);
+      fft_c<L, +1, IL>(a, c1, twr);
       if (own) {
 #pragma unroll
-        for (int j = 0; j < P::R1; ++j) c1(t + P::T * j) = a[j];
+        for (int j = 0; j < P::R1; ++j) c1.put(j, a[j]);
       }
     }
     fence_async_smem();
