@@ -39,8 +39,6 @@ struct Pen {
   static constexpr int NCOL = H < W ? H : W;    // kz columns per y-pass CTA
   static constexpr int NKC = H / NCOL;          // y-pass CTAs per plane
   static constexpr int BOX = L * W;             // float2 per TMA box [ky][W kz]
-  static constexpr int ZNT = 256;               // threads of the z-pass kernels
-  static constexpr int ZG = ZNT / T;
   static_assert(YB == ybin(L) && NYB == nybins(L), "one point bin per z-pass CTA");
 };
 
@@ -201,26 +199,61 @@ __device__ __forceinline__ void c2r_acc(int t, const Tw& tw, Acc x) {
 // ===========================================================================
 // Forward z pass: splat of the four channels into YB rows of plane X, R2C.
 // ===========================================================================
+// One CTA per tile (plane X, rows y0 .. y0 + YB - 1) with its four channels, or
+// at r = 512 per tile and channel: there four channels (131 KB) leave one CTA to
+// an SM, idle while it zeroes, splats or waits (345 us; 268 by channel, which
+// reads the points four times). At r = 256 both take 47 us, and below, where a
+// tile has many points, one read of them wins (batch of r = 64: 38 against 45).
+template <int L>
+struct ZfGeo {
+  static constexpr int T = Shape<L>::T, YB = Pen<L>::YB;
+  static constexpr int NCC = L >= 512 ? 1 : 4;  // channels per CTA
+  static constexpr int NP = NCC * YB / 2;       // row pairs
+  static constexpr int NT = L >= 512 ? YB / 2 * T : 256;
+  static constexpr int MINB = L >= 512 ? 4 : (L >= 256 ? 3 : 4);
+  static constexpr int RF = pairs_floats<L>(NP);
+};
+
 template <int L>
 constexpr size_t zfwd_smem() {
-  using P = Pen<L>;
-  return sizeof(float) * (pairs_floats<L>(2 * P::YB) + L) + sizeof(float2) * L;
+  return sizeof(float) * (ZfGeo<L>::RF + L) + sizeof(float2) * L;
 }
 
-// One z-pass tile (plane X, rows y0 .. y0 + YB - 1) on zeroed `rows`:
-// splat, R2C, bulk stores of the packed rows.
 template <int L>
-__device__ __forceinline__ void zfwd_tile(const Solve& S, int X, int y0, float* rows,
-                                          const float2* twt, const float* iu) {
+__global__ void __launch_bounds__(ZfGeo<L>::NT, ZfGeo<L>::MINB) k_zfwd(const __grid_constant__ Solve s0,
+                                                                       const Solve* __restrict__ tab) {
   using P = Pen<L>;
-  constexpr int YB = P::YB, H = P::H;
+  using Z = ZfGeo<L>;
+  constexpr int YB = P::YB, NT = Z::NT, RF = Z::RF;
+  const Solve& S = tab ? tab[blockIdx.z] : s0;
+  // channels v_y, v_z, v_x, w (buffers 0..3), the CTA's from ch0 on
+  constexpr int NCC = Z::NCC, PER = 4 / NCC;
+  const int ch0 = (int)(blockIdx.x % PER) * NCC, tile = blockIdx.x / PER;
+  const int X = tile / P::NYB, yb = tile % P::NYB, y0 = yb * YB;
   const int tid = threadIdx.x, g = tid / P::T, t = tid % P::T;
+  extern __shared__ float4 smem4[];
+  float* rows = reinterpret_cast<float*>(smem4);  // row ly of its k-th channel at row_off(k YB + ly)
+  float2* twt = reinterpret_cast<float2*>(rows + RF);
+  float* iu = reinterpret_cast<float*>(twt + L);
+  __shared__ unsigned char touched[YB];  // rows that points reach
+  pdl_trigger();
+  if constexpr (kSkip<L>) {  // a tile that no stencil reaches is not stored: the y pass does not load it
+    pdl_wait();
+    if (!((reach_mask(tile_mask(S, L, X), P::NYB) >> yb) & 1u)) return;
+  }
+  for (int i = tid; i < L; i += NT) {
+    twt[i] = S.tw[i];
+    iu[i] = S.iu[2 * L + i];  // z axis
+  }
+  for (int i = tid; i < RF / 4; i += NT) smem4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (tid < YB) touched[tid] = 0;
+  if constexpr (!kSkip<L>) pdl_wait();
   // Rasterization (Eq. A2): points of x-cells X (dx = 0) and X - 1 (dx = 1)
   // whose stencil rows i0 or i1 fall in [y0, y0 + YB), i.e. i0 in
   // [y0 - 1, y0 + YB - 1] (mod L): per side the CTA's own bin and the
   // previous y-block's bin (its last row only). The four ranges are read up
   // front and visited as one sequence, so that their loads overlap.
-  const int yb = y0 / YB, ylast = (y0 - 1) & (L - 1);
+  const int ylast = (y0 - 1) & (L - 1);
   int q0, q1, q2, q3, c1, c2, c3, c4;  // range starts, cumulative counts
   {
     const int* off = S.bins + nbins(L);
@@ -239,10 +272,8 @@ __device__ __forceinline__ void zfwd_tile(const Solve& S, int X, int y0, float* 
     c3 = c2 + (e2 - q2);
     c4 = c3 + (e3 - q3);
   }
-  __shared__ unsigned char touched[YB];  // rows that points reach
-  if (tid < YB) touched[tid] = 0;
   __syncthreads();
-  for (int v = tid; v < c4; v += P::ZNT) {
+  for (int v = tid; v < c4; v += NT) {
     const int k = v < c1 ? 0 : (v < c2 ? 1 : (v < c3 ? 2 : 3));
     const int i = k == 0 ? q0 + v : (k == 1 ? q1 + (v - c1) : (k == 2 ? q2 + (v - c2) : q3 + (v - c3)));
     const int side = k >> 1, part = k & 1;
@@ -261,59 +292,29 @@ __device__ __forceinline__ void zfwd_tile(const Solve& S, int X, int y0, float* 
       const float f = wx * tri_w(dy, ay.t);
       const float f0 = f * (1.f - az.t), f1 = f * az.t;
 #pragma unroll
-      for (int ch = 0; ch < 4; ++ch) {
-        float* row = rows + row_off<L>(ch * YB + ly);
-        atomicAdd(row + az.i0, f0 * val[ch]);
-        atomicAdd(row + az.i1, f1 * val[ch]);
+      for (int k = 0; k < NCC; ++k) {
+        float* row = rows + row_off<L>(k * YB + ly);
+        const float w = NCC == 4 ? val[k] : (ch0 == 0 ? val[0] : (ch0 == 1 ? val[1] : (ch0 == 2 ? val[2] : val[3])));
+        atomicAdd(row + az.i0, f0 * w);
+        atomicAdd(row + az.i1, f1 * w);
       }
     }
   }
   __syncthreads();
   TwTab<L> twr{twt, t};
-  constexpr int NP = 4 * YB / 2;
-  for (int p0 = 0; p0 < NP; p0 += P::ZG) {
+  for (int p0 = 0; p0 < Z::NP; p0 += NT / P::T) {
     const int pi = p0 + g;
-    if (pi < NP) {  // whole groups
-      // the v_z rows (pairs YB/2 .. YB-1) take i u_z (zero at DC and Nyquist)
-      const bool vz = pi >= YB / 2 && pi < YB;
-      const int ch = (2 * pi) / YB, ly = (2 * pi) % YB;  // rows ly, ly + 1 of channel ch
+    if (pi < Z::NP) {  // whole groups
+      const int ch = ch0 + (2 * pi) / YB, ly = (2 * pi) % YB;  // rows ly, ly + 1; v_z takes i u_z (zero at DC, Nyquist)
       float2* ga = S.spec[ch] + ((size_t)X * L + y0 + ly) * P::KP;
       if (kSkip<L> && !(touched[ly] | touched[ly + 1])) {  // a pair without points: its spectrum is zero
 #pragma unroll
         for (int j = 0; j < P::R1 / 2; ++j) ga[t + P::T * j] = ga[P::KP + t + P::T * j] = czero();
       } else {
-        r2c_pair_st<L>(t, twr, rows + pair_off<L>(pi), vz ? iu : nullptr, ga, ga + P::KP);
+        r2c_pair_st<L>(t, twr, rows + pair_off<L>(pi), ch == 1 ? iu : nullptr, ga, ga + P::KP);
       }
     }
   }
-}
-
-template <int L>
-__global__ void __launch_bounds__(Pen<L>::ZNT, L >= 512 ? 1 : (L >= 256 ? 3 : 4)) k_zfwd(const __grid_constant__ Solve s0,
-                                                      const Solve* __restrict__ tab) {
-  using P = Pen<L>;
-  constexpr int YB = P::YB;
-  const Solve& S = tab ? tab[blockIdx.z] : s0;
-  const int X = blockIdx.x / P::NYB, y0 = (blockIdx.x % P::NYB) * YB;
-  const int tid = threadIdx.x;
-  extern __shared__ float4 smem4[];
-  constexpr int RF = pairs_floats<L>(2 * YB);
-  float* rows = reinterpret_cast<float*>(smem4);  // rows ch * YB + ly (row_off): v_y, v_z, v_x, w
-  float2* twt = reinterpret_cast<float2*>(rows + RF);
-  float* iu = reinterpret_cast<float*>(twt + L);
-  pdl_trigger();
-  if constexpr (kSkip<L>) {  // a tile that no stencil reaches is not stored: the y pass does not load it
-    pdl_wait();
-    if (!((reach_mask(tile_mask(S, L, X), P::NYB) >> (y0 / YB)) & 1u)) return;
-  }
-  for (int i = tid; i < L; i += P::ZNT) {
-    twt[i] = S.tw[i];
-    iu[i] = S.iu[2 * L + i];  // z axis
-  }
-  for (int i = tid; i < RF / 4; i += P::ZNT) smem4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-  if constexpr (!kSkip<L>) pdl_wait();
-  __syncthreads();
-  zfwd_tile<L>(S, X, y0, rows, twt, iu);
 }
 
 // ===========================================================================
@@ -688,7 +689,10 @@ struct ZiGeo {
   // the C2R makes 64-bit accesses only, spread needed below T = 16
   static constexpr bool SP = Shape<L>::T < 16;
   static constexpr int STAGE = pairs_floats<L, SP>(NCH * NR / 2) / 2;
-  static constexpr int NT = 256;
+  // the forward's nine pairs on ten groups of 16 lanes (256 threads would idle
+  // seven of 16 groups and, at r = 512, leave one CTA to an SM: 371 us, now 245;
+  // r = 256: 37 -> 35)
+  static constexpr int NT = NCH == 1 && Shape<L>::T == 16 ? 160 : 256;
 };
 
 template <int L, int NCH>
@@ -892,7 +896,7 @@ struct TileList {
 };
 
 template <int L, int NCH>
-__global__ void __launch_bounds__(ZiGeo<L, NCH>::NT, L >= 512 ? 1 : (NCH == 1 ? 4 : (L >= 256 ? 2 : 3)))
+__global__ void __launch_bounds__(ZiGeo<L, NCH>::NT, L >= 512 ? (NCH == 1 ? 2 : 1) : (NCH == 1 ? (L >= 256 ? 5 : 4) : (L >= 256 ? 2 : 3)))
     k_zinv(const __grid_constant__ Solve s0, const Solve* __restrict__ tab) {
   using P = Pen<L>;
   using Z = ZiGeo<L, NCH>;
@@ -1065,7 +1069,7 @@ template <int L>
 static cudaError_t launch_pencil_t(int kind, const Solve& s, const Solve* tab, int count,
                                    cudaStream_t st) {
   using P = Pen<L>;
-  const dim3 gz(L * P::NYB, 1, count), gy(L * P::NKC, 1, count);
+  const dim3 gy(L * P::NKC, 1, count);
   static bool attr_set[4] = {false, false, false, false};
   cudaError_t e = cudaSuccess;
   switch (kind) {
@@ -1077,7 +1081,7 @@ static cudaError_t launch_pencil_t(int kind, const Solve& s, const Solve* tab, i
         if (e != cudaSuccess) return e;
         attr_set[0] = true;
       }
-      e = launch_k(k_zfwd<L>, gz, dim3(P::ZNT), a, st, 0, s, tab);
+      e = launch_k(k_zfwd<L>, dim3(4 / ZfGeo<L>::NCC * L * P::NYB, 1, count), dim3(ZfGeo<L>::NT), a, st, 0, s, tab);
       if (e == cudaSuccess)
         e = launch_k(k_yfwd<L, false>, dim3(L * P::NKC, yfwd_merge<L>() ? 2 : 3, count), dim3(ynt<L>()),
                      b, st, 0, s, tab);
