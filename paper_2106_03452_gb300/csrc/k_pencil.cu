@@ -22,6 +22,7 @@
 // Half spectra along z are stored "packed" between the passes: slot 0 holds
 // the DC and Nyquist terms of a real row as one complex number.
 #include "col.cuh"
+#include "coldir.cuh"
 #include "dpsr_dev.cuh"
 #include "finalize.cuh"
 #include "launch.h"
@@ -511,11 +512,6 @@ __global__ void __launch_bounds__(ynt<L>(), BWD ? 4 : (L >= 256 ? 3 : 5)) k_yfwd
 // r = 256, bound by bandwidth, one CTA does all three.
 // ===========================================================================
 template <int L, int NCH>
-constexpr bool yinv_split() {
-  return NCH == 3 && L < 256;
-}
-
-template <int L, int NCH>
 constexpr size_t yinv_smem() {
   return box_align<L>() + sizeof(float2) * ((size_t)NCH * Pen<L>::BOX + L) + sizeof(float) * L;
 }
@@ -541,7 +537,7 @@ __device__ __forceinline__ void yinv_issue(const Solve& S, int X, int kz0, int p
 template <int L, int NCH>
 __device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int part, float2* box,
                                           const float2* twt, const float* iu, uint64_t* bar,
-                                          uint32_t phase, unsigned rows = 0xffffffffu) {
+                                          uint32_t phase) {
   using P = Pen<L>;
   constexpr int H = P::H;
   constexpr bool IL = P::T == 16;  // interleaved groups: conflict-free column accesses
@@ -604,18 +600,7 @@ __device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int pa
   }
   fence_async_smem();
   __syncthreads();
-  if constexpr (NCH == 3 && kSkip<L>) {  // warp 0: the y-blocks that the z pass reads, a lane each
-    if (tid < P::NYB && ((rows >> tid) & 1u)) {
-      const int y = tid * P::YB;
-      if (do0) tma_store_3d(&S.tmb[kSpC], kz0, y, X, box + y * P::W);
-      if (do1) {
-        tma_store_3d(&S.tmb[kSpYa], kz0, y, X, box + P::BOX + y * P::W);
-        tma_store_3d(&S.tmb[kSpYb], kz0, y, X, box + 2 * P::BOX + y * P::W);
-      }
-      tma_store_commit();
-      tma_store_wait_read();
-    }
-  } else if (tid == 0) {
+  if (tid == 0) {
     for (int y = 0; y < L; y += tma_rows(L)) {
       if constexpr (NCH == 1) {
         tma_store_3d(&S.tmy[kSpYa], kz0, y, X, box + y * P::W);
@@ -634,7 +619,7 @@ __device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int pa
 }
 
 template <int L, int NCH>
-__global__ void __launch_bounds__(ynt<L>(), NCH == 1 || yinv_split<L, NCH>() ? 4 : 2)
+__global__ void __launch_bounds__(ynt<L>(), 4)
     k_yinv(const __grid_constant__ Solve s0, const Solve* __restrict__ tab) {
   using P = Pen<L>;
   constexpr int NT = ynt<L>();
@@ -655,19 +640,99 @@ __global__ void __launch_bounds__(ynt<L>(), NCH == 1 || yinv_split<L, NCH>() ? 4
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   pdl_wait();
-  unsigned rows = 0xffffffffu;
-  if constexpr (NCH == 3 && kSkip<L>) {
-    rows = reach_mask(tile_mask(S, L, X), P::NYB);
-    if (rows == 0u) return;  // no points gather from this plane
-  }
-  const int part = yinv_split<L, NCH>() ? (int)blockIdx.y : -1;  // -1: all fields
+  const int part = NCH == 3 ? (int)blockIdx.y : -1;
   if (tid == 0) yinv_issue<L, NCH>(S, X, kz0, part, box, &bar);
   for (int i = tid; i < L; i += NT) {
     twt[i] = S.tw[i];
     iu[i] = S.iu[L + i];  // y axis
   }
   __syncthreads();
-  yinv_tile<L, NCH>(S, X, kz0, part, box, twt, iu, &bar, 0, rows);
+  yinv_tile<L, NCH>(S, X, kz0, part, box, twt, iu, &bar, 0);
+}
+
+// ===========================================================================
+// The adjoint's y pass from r = 64 on: columns in registers from load to store
+// (see ColDir), in two CTA kinds (blockIdx.y): 0 V_bar_x from Q2, 1 V_bar_y and
+// V_bar_z from Q1, which is loaded once. k_yinv's tiles of all three fields
+// (99 KB at r = 256) leave two CTAs to an SM; here shared memory holds the
+// exchange only, and the y-blocks without points are simply not stored.
+// r = 256: 54 -> 41.5 us, r = 512: 387 -> 309. The passes that store every row
+// and transform a field once stay with the tiles: from global memory the
+// forward y pass took 73 us against 65, that of dchi 33 against 22.
+// ===========================================================================
+template <int L>
+struct YDir {
+  using D = ColDir<L>;
+  static constexpr int H = L / 2, KP = kpitch(L), NKC = H / D::C;
+  static constexpr size_t STEP = (size_t)D::T * KP;  // from element j to j + 1
+  // y-block of element j (T divides a block)
+  static __device__ __forceinline__ bool has(unsigned rows, int j) {
+    return (rows >> (D::T * j / ybin(L))) & 1u;
+  }
+};
+
+template <int L>
+constexpr size_t ydir_smem() {
+  using D = ColDir<L>;
+  return sizeof(float2) * (D::NBUF * D::XCH + L);
+}
+
+template <int L>
+__global__ void __launch_bounds__(ColDir<L>::NT, L >= 512 ? 3 : (L >= 128 ? 4 : 6))
+    k_yadj(const __grid_constant__ Solve s0, const Solve* __restrict__ tab) {
+  using D = ColDir<L>;
+  using P = YDir<L>;
+  constexpr int R1 = D::R1, T = D::T;
+  const Solve& S = tab ? tab[blockIdx.z] : s0;
+  const int tid = threadIdx.x, c = tid % D::C, t = tid / D::C;
+  const int X = blockIdx.x / P::NKC, kz0 = (blockIdx.x % P::NKC) * D::C;
+  const bool two = blockIdx.y == 1;
+  extern __shared__ float4 smem4[];
+  float2* xch = reinterpret_cast<float2*>(smem4);
+  float2* twt = xch + D::NBUF * D::XCH;
+  pdl_trigger();
+  for (int i = tid; i < L; i += D::NT) twt[i] = S.tw[i];
+  pdl_wait();
+  const unsigned rows = reach_mask(tile_mask(S, L, X), nybins(L));
+  if (rows == 0u) return;  // no points gather from this plane
+  const int in = two ? kSpD : kSpChi;
+  const size_t first = ((size_t)X * L + t) * P::KP + kz0 + c;
+  const float2* p = S.spec[in] + first;
+  float2 a[R1];
+#pragma unroll
+  for (int j = 0; j < R1; ++j) a[j] = ld_once(p + j * P::STEP);
+  if (kz0 == 0 && c == 0) {  // column 0 becomes X0 + i Xn (Xn: the Nyquist column)
+    const float2* nq = S.spec[in] + ((size_t)X * L + t) * P::KP + P::H;
+#pragma unroll
+    for (int j = 0; j < R1; ++j) {
+      const float2 n = ld_once(nq + j * P::STEP);
+      a[j] = make_float2(a[j].x - n.y, a[j].y + n.x);
+    }
+  }
+  const TwTab<L> tw{twt, t};
+  auto store = [&](int buf, const float2 (&v)[R1]) {  // the y-blocks that the z pass reads
+    float2* o = S.spec[buf] + first;
+#pragma unroll
+    for (int j = 0; j < R1; ++j)
+      if (P::has(rows, j)) o[j * P::STEP] = v[j];
+  };
+  __syncthreads();  // the twiddles
+  if (!two) {
+    fft_d<L, +1>(a, t, c, tw, xch, 0);
+    store(kSpC, a);
+  } else {
+    float2 b[R1];
+#pragma unroll
+    for (int j = 0; j < R1; ++j) b[j] = cmul_iu(a[j], -__ldg(S.iu + L + t + T * j));
+    fft_d<L, +1>(b, t, c, tw, xch, 0);
+    store(kSpYa, b);
+    fft_d<L, +1>(a, t, c, tw, xch, 1);
+    const int kz = kz0 + c;
+    const float ez = kz == 0 ? 0.f : -__ldg(S.iu + 2 * L + kz);
+#pragma unroll
+    for (int j = 0; j < R1; ++j) a[j] = cmul_iu(a[j], ez);
+    store(kSpYb, a);
+  }
 }
 
 // ===========================================================================
@@ -1118,21 +1183,31 @@ static cudaError_t launch_pencil_t(int kind, const Solve& s, const Solve* tab, i
       return e;
     }
     default: {
-      constexpr size_t a = yinv_smem<L, 3>(), b = zinv_smem<L, 3>();
-      constexpr int nt = ynt<L>();
+      constexpr size_t b = zinv_smem<L, 3>();
       static int nz = 0;
+      if constexpr (L >= 64) {
+        constexpr size_t a = ydir_smem<L>();
+        if (!attr_set[3]) {
+          e = set_smem(k_yadj<L>, a);
+          if (e != cudaSuccess) return e;
+        }
+        e = launch_k(k_yadj<L>, dim3(L * YDir<L>::NKC, 2, count), dim3(ColDir<L>::NT), a, st, 0, s, tab);
+      } else {
+        constexpr size_t a = yinv_smem<L, 3>();
+        if (!attr_set[3]) {
+          e = set_smem(k_yinv<L, 3>, a);
+          if (e != cudaSuccess) return e;
+        }
+        e = launch_k(k_yinv<L, 3>, dim3(L * P::NKC, 2, count), dim3(ynt<L>()), a, st, 0, s, tab);
+      }
+      if (e != cudaSuccess) return e;
       if (!attr_set[3]) {
-        e = set_smem(k_yinv<L, 3>, a);
-        if (e == cudaSuccess) e = set_smem(k_zinv<L, 3>, b);
+        e = set_smem(k_zinv<L, 3>, b);
         if (e != cudaSuccess) return e;
         nz = persistent_ctas(k_zinv<L, 3>, ZiGeo<L, 3>::NT, b, L * P::NYB, 1);
         attr_set[3] = true;
       }
-      e = launch_k(k_yinv<L, 3>, dim3(L * P::NKC, yinv_split<L, 3>() ? 2 : 1, count), dim3(nt), a, st, 0,
-                   s, tab);
-      if (e == cudaSuccess)
-        e = launch_k(k_zinv<L, 3>, dim3(nz, 1, count), dim3(ZiGeo<L, 3>::NT), b, st, 0, s, tab);
-      return e;
+      return launch_k(k_zinv<L, 3>, dim3(nz, 1, count), dim3(ZiGeo<L, 3>::NT), b, st, 0, s, tab);
     }
   }
 }
@@ -1160,7 +1235,7 @@ size_t pencil_smem_bytes(int kind, int r) {
       case 0: a = zfwd_smem<L>(); b = yfwd_smem<L, false>(); break;
       case 1: a = yinv_smem<L, 1>(); b = zinv_smem<L, 1>(); break;
       case 2: a = zbfwd_smem<L>(); b = yfwd_smem<L, true>(); break;
-      default: a = yinv_smem<L, 3>(); b = zinv_smem<L, 3>(); break;
+      default: a = L >= 64 ? ydir_smem<L>() : yinv_smem<L, 3>(); b = zinv_smem<L, 3>(); break;
     }
     return a > b ? a : b;
   };
