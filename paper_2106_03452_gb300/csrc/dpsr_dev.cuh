@@ -212,6 +212,8 @@ __host__ __device__ constexpr int tma_rows(int r) { return r < 256 ? r : 256; }
 // 237 -> 190; the x passes, bound by too few warps either way, 779 -> 807 and
 // 722 -> 633).
 __host__ __device__ constexpr int tile_cols(int r) { return r < 512 ? 16 : 8; }
+// Tiles (blocks, and partial sums) of the x pass.
+__host__ __device__ constexpr int x_tiles(int r) { return (r / 2 + tile_cols(r)) / tile_cols(r) * r; }
 
 // The stage twiddles W_L^(t*k1) of thread t, read from a shared-memory copy of
 // Solve::tw at each use: entry k1 T + t, so that a group's lanes read
@@ -343,9 +345,9 @@ struct Scalars {
   float g_a, g_s, g_w;    // backward: G^ = g_a * FFT(dchi) + g_s + g_w * W^
   float c_mu;             // backward: weight of the stored lookup gradient
   double loss;            // L_DPSR of Eq. 9 (mean squared error against a target grid)
-  // arrival counters of the last-block reductions: [0] forward x-pass,
-  // [1] backward plane pass, [2] the L_DPSR loss (all reset by the binning's
-  // scatter of every forward, and each by its own last block)
+  // arrival counters of the last-block reductions: [1] backward plane pass,
+  // [2] the L_DPSR loss (reset by the binning's scatter of every forward, and
+  // each by its own last block)
   unsigned ticket[3];
 };
 

@@ -76,32 +76,41 @@ __device__ __forceinline__ void block_sum_ff(FF& a, FF& b) {
   }
 }
 
+// The scalars of Eq. 4 from the forward's reduced sums:
+// mu = <W, chi'> / N, chi'(0) = sum_k chi~ / n, s = chi'(0) - mu.
+struct FwdScalars {
+  double mu, s, alpha;
+  float a_chi, b_chi;
+  bool bad;
+};
+__device__ __forceinline__ FwdScalars fwd_scalars(const Solve& S, double a, double b) {
+  FwdScalars q;
+  // r^3 is a power of two: its reciprocal is exact in FP32
+  const double inv_n = (double)__frcp_rn((float)S.r * (float)S.r * (float)S.r);
+  q.mu = a * inv_n * S.inv_N;
+  const double chi0 = b * inv_n;
+  q.s = chi0 - q.mu;
+  q.bad = !isfinite(q.s) || !(fabs(q.s) > 1e-7 * (fabs(chi0) + fabs(q.mu)) + 1e-37);
+  q.alpha = q.bad ? 0.0 : (double)kM / fabs(q.s);
+  q.a_chi = (float)(q.alpha * inv_n);
+  q.b_chi = (float)(-q.alpha * q.mu);
+  return q;
+}
+
 // Thread 0: the scalars from the reduced sums.
 __device__ inline void finalize_scalars(const Solve& S, double a, double b, bool bwd) {
   Scalars* sc = S.sc;
-  // r^3 is a power of two: its reciprocal is exact in FP32
   const double inv_n = (double)__frcp_rn((float)S.r * (float)S.r * (float)S.r);
   if (!bwd) {
-    // mu = <W, chi'> / N, chi'(0) = sum_k chi~ / n, s = chi'(0) - mu (Eq. 4)
-    const double mu = a * inv_n * S.inv_N;
-    const double chi0 = b * inv_n;
-    const double s = chi0 - mu;
+    const FwdScalars q = fwd_scalars(S, a, b);
     sc->acc_mu = a;
     sc->acc_s0 = b;
-    sc->mu = mu;
-    sc->s = s;
-    const bool bad = !isfinite(s) || !(fabs(s) > 1e-7 * (fabs(chi0) + fabs(mu)) + 1e-37);
-    if (bad) {
-      atomicOr(S.status, kStDegenerate);
-      sc->alpha = 0;
-      sc->a_chi = 0.f;
-      sc->b_chi = 0.f;
-    } else {
-      const double alpha = (double)kM / fabs(s);
-      sc->alpha = alpha;
-      sc->a_chi = (float)(alpha * inv_n);
-      sc->b_chi = (float)(-alpha * mu);
-    }
+    sc->mu = q.mu;
+    sc->s = q.s;
+    sc->alpha = q.alpha;
+    sc->a_chi = q.a_chi;
+    sc->b_chi = q.b_chi;
+    if (q.bad) atomicOr(S.status, kStDegenerate);
   } else {
     // a = sum dchi, b = sum dchi * chi = alpha * sum dchi (chi' - mu);
     // with alpha = m / |s|: D = b / alpha = b |s| / m and
@@ -120,6 +129,21 @@ __device__ inline void finalize_scalars(const Solve& S, double a, double b, bool
     sc->g_w = (float)(mu_bar * inv_n * S.inv_N);
     sc->c_mu = sc->g_w;
   }
+}
+
+// The `n` block partials of S.part summed by every thread of a block (each a
+// strided subset, loads in flight together, then the block tree: a fixed
+// order); the sums are valid in thread 0.
+template <int NT>
+__device__ __forceinline__ void sum_partials(const Solve& S, int n, FF& x, FF& y) {
+  x = y = FF{0.f, 0.f};
+#pragma unroll 8
+  for (int i = threadIdx.x; i < n; i += NT) {
+    const float4 p = __ldcg(S.part + i);
+    x = ff_add(x, FF{p.x, p.y});
+    y = ff_add(y, FF{p.z, p.w});
+  }
+  block_sum_ff<NT>(x, y);
 }
 
 // Every thread of the block calls this after the block sums (a, b) are in
@@ -142,14 +166,8 @@ __device__ inline void last_block_finalize(const Solve& S, int ticket, int nbloc
   }
   __syncthreads();
   if (!last) return;
-  FF x = {0.f, 0.f}, y = {0.f, 0.f};
-#pragma unroll 4
-  for (int i = tid; i < nblocks; i += NT) {
-    const float4 p = __ldcg(S.part + i);
-    x = ff_add(x, FF{p.x, p.y});
-    y = ff_add(y, FF{p.z, p.w});
-  }
-  block_sum_ff<NT>(x, y);
+  FF x, y;
+  sum_partials<NT>(S, nblocks, x, y);
   if (tid == 0) {
     finalize_scalars(S, ff_to_double(x), ff_to_double(y), bwd);
     S.sc->ticket[ticket] = 0;

@@ -640,6 +640,12 @@ __global__ void __launch_bounds__(ynt<L>(), 4)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   pdl_wait();
+  if (NCH == 1 && blockIdx.x == L * P::NKC) {  // one more CTA: the scalars of Eq. 4, read by the z pass
+    FF x, y;
+    sum_partials<NT>(S, x_tiles(L), x, y);
+    if (tid == 0) finalize_scalars(S, ff_to_double(x), ff_to_double(y), false);
+    return;
+  }
   const int part = NCH == 3 ? (int)blockIdx.y : -1;
   if (tid == 0) yinv_issue<L, NCH>(S, X, kz0, part, box, &bar);
   for (int i = tid; i < L; i += NT) {
@@ -1163,7 +1169,7 @@ static cudaError_t launch_pencil_t(int kind, const Solve& s, const Solve* tab, i
         nz = persistent_ctas(k_zinv<L, 1>, ZiGeo<L, 1>::NT, b, L * P::NYB, 1);
         attr_set[1] = true;
       }
-      e = launch_k(k_yinv<L, 1>, gy, dim3(nt), a, st, 0, s, tab);
+      e = launch_k(k_yinv<L, 1>, dim3(L * P::NKC + 1, 1, count), dim3(nt), a, st, 0, s, tab);
       if (e == cudaSuccess)
         e = launch_k(k_zinv<L, 1>, dim3(nz, 1, count), dim3(ZiGeo<L, 1>::NT), b, st, 0, s, tab);
       return e;

@@ -470,17 +470,29 @@ __global__ void __launch_bounds__(kNT, plane_minb<L, C>(1))
   for (int i = tid; i < L; i += kNT) twt[i] = S.tw[i];
   TwTab<L> twr{twt, t};
   pdl_wait();
-  const float a_chi = S.sc->a_chi, b_chi = S.sc->b_chi;
   if (tid == 0) {
     mbar_init(&bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    chunk_load<L, C>(&S.tmy[kSpChi], sbox, c * P::SPC, X, &bar);
   }
-  __syncthreads();
+  // While the first tiles land, every CTA sums the x pass's partials into the
+  // scalars of Eq. 4 for itself; the first one publishes them.
+  __shared__ float scale[2];
+  {
+    FF x, y;
+    sum_partials<kNT>(S, x_tiles(L), x, y);  // synchronises the block
+    if (tid == 0) {
+      const FwdScalars q = fwd_scalars(S, ff_to_double(x), ff_to_double(y));
+      scale[0] = q.a_chi;
+      scale[1] = q.b_chi;
+      if (blockIdx.x == 0) finalize_scalars(S, ff_to_double(x), ff_to_double(y), false);
+    }
+  }
   uint32_t phase = 0;
   bool alive = true;
   for (int cb = 0; cb < P::SPC && alive; cb += P::CHK) {
     const int s_first = c * P::SPC + cb;
-    if (tid == 0) chunk_load<L, C>(&S.tmy[kSpChi], sbox, s_first, X, &bar);
+    if (tid == 0 && cb > 0) chunk_load<L, C>(&S.tmy[kSpChi], sbox, s_first, X, &bar);
     const bool head = (c == 0 && cb == 0);
     float2 nyq[P::R1];
     if (head && g == 0 && P::H >= 16) {
@@ -511,6 +523,7 @@ __global__ void __launch_bounds__(kNT, plane_minb<L, C>(1))
   }
   cl.sync();
   if (!alive) return;
+  const float a_chi = scale[0], b_chi = scale[1];
   // C2R along z of row pairs (2p, 2p+1); output written in place as pairs
   // (y_2p[z], y_2p+1[z]) at logical slot z of the pair.
   float* chi = S.chi;

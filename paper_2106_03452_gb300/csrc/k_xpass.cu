@@ -25,7 +25,7 @@ struct XGeo {
   static constexpr int NG = KC * T >= 32 ? KC : 32 / T;     // groups (at least one warp)
   static constexpr int NT = NG * T;                         // threads
   static constexpr int H = L / 2;
-  static constexpr int NCHUNK = (H + 1 + KC - 1) / KC;
+  static constexpr int NCHUNK = x_tiles(L) / L;
   static constexpr int BOX = L * KC;                        // float2 per box
   static constexpr int KP = kpitch(L);                      // row pitch of the spectral buffers
   // Two tiles per CTA in both directions. The forward needs W~ only for its
@@ -223,8 +223,11 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
       for (int x = 0; x < L; x += tma_rows(L)) tma_store_3d(&S.tmx[kSpChi], kz0, ky, x, box + x * P::KC);
       tma_store_commit();
     }
-    last_block_finalize<P::NT>(S, 0, (int)(gridDim.x * gridDim.y),
-                               (int)(blockIdx.y * gridDim.x + blockIdx.x), fm, fs, false);
+    // Summed by the inverse plane kind, which runs before anything reads the
+    // scalars. A last-block ticket here (a fence and an atomic on one address
+    // per CTA, its place on the SM held for the round trip) cost more than the
+    // transforms: 75 -> 63 us at r = 256 without it, 807 -> 552 at r = 512.
+    if (tid == 0) S.part[blockIdx.y * gridDim.x + blockIdx.x] = make_float4(fm.hi, fm.lo, fs.hi, fs.lo);
     if (tid == 0) tma_store_wait_read();
   } else {
     // FFT_x of (g_a FFT_zy(dchi) + g_w W~ + g_s delta_{x=0}): the three terms
@@ -308,17 +311,6 @@ cudaError_t launch_xpass(bool bwd, int r, const Solve& s, const Solve* tab, int 
   }
 }
 
-int xpass_blocks(int r) {
-  switch (r) {
-    case 8: return XGeo<8>::NCHUNK * 8;
-    case 16: return XGeo<16>::NCHUNK * 16;
-    case 32: return XGeo<32>::NCHUNK * 32;
-    case 64: return XGeo<64>::NCHUNK * 64;
-    case 128: return XGeo<128>::NCHUNK * 128;
-    case 256: return XGeo<256>::NCHUNK * 256;
-    case 512: return XGeo<512>::NCHUNK * 512;
-    default: return 0;
-  }
-}
+int xpass_blocks(int r) { return x_tiles(r); }
 
 }  // namespace dpsr

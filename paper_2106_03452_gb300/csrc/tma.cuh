@@ -21,7 +21,7 @@ __device__ __forceinline__ int bx(int q, int c) {
 // L = 512 under the 64-byte swizzle (chunks XOR-ed by bits 1-2 of the row).
 template <int L>
 __device__ __forceinline__ int bxl(int q, int c) {
-  if constexpr (L < 512) return bx(q, c);
+  if constexpr (tile_cols(L) == 16) return bx(q, c);
   else return q * 8 + ((((c >> 1) ^ ((q >> 1) & 3)) << 1) | (c & 1));
 }
 
