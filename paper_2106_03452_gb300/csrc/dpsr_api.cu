@@ -387,6 +387,14 @@ int make_tensor_maps(Solve& s, int r) {
       if (rc != CUDA_SUCCESS) return DPSR_ECUDA;
     }
   }
+  if (r <= 256) {
+    const cuuint32_t boxw[3] = {16, (cuuint32_t)r, 1};
+    for (int k = 0; k < kNSpec; ++k)
+      if (enc(&s.tmw[k], CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, (void*)s.spec[k], dims, strides, boxw, es,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return DPSR_ECUDA;
+  }
   if (r < 64) return DPSR_OK;  // kSkip: the parts of tiles below are not used
   const cuuint32_t boxb[3] = {cols, 16, 1}, boxc[3] = {cols, 1, (cuuint32_t)(r / kXChunks)};
   for (int k = 0; k < kNSpec + 4; ++k) {

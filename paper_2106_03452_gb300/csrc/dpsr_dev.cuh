@@ -206,12 +206,13 @@ template <> struct Shape<512> { static constexpr int R1 = 32, T = 16; };
 // 1024-byte boundary, so the 128-byte swizzle runs on unchanged).
 __host__ __device__ constexpr int tma_rows(int r) { return r < 256 ? r : 256; }
 // Columns (kz slots) of a tile of the x and y passes: 16, one 128-byte line a
-// row, up to r = 256; 8 at r = 512, where tiles of 16 (64 KB a box) leave one
-// CTA to an SM, whose load, transform and store phases then follow one another
+// row, up to r = 128; 8 above. At r = 512 tiles of 16 (64 KB a box) leave one CTA
+// to an SM, whose load, transform and store phases then follow one another
 // (three with 8 columns: forward y pass 789 -> 527 us, dchi's 285 -> 170, inverse
-// 237 -> 190; the x passes, bound by too few warps either way, 779 -> 807 and
-// 722 -> 633).
-__host__ __device__ constexpr int tile_cols(int r) { return r < 512 ? 16 : 8; }
+// 237 -> 190, backward x pass 722 -> 633). At r = 256 twice as many CTAs of half the
+// size mix their phases better (backward x pass 72 -> 62 us, forward y pass 65 ->
+// 61, inverse y pass 32 -> 30.5; the forward x pass stays at 63).
+__host__ __device__ constexpr int tile_cols(int r) { return r < 256 ? 16 : 8; }
 // Tiles (blocks, and partial sums) of the x pass.
 __host__ __device__ constexpr int x_tiles(int r) { return (r / 2 + tile_cols(r)) / tile_cols(r) * r; }
 
@@ -374,6 +375,7 @@ struct Solve {
   // of 16 kz x 16 ky x 1 x (a y-block), tmc boxes of 16 kz x 1 ky x r/8 x (an
   // x-chunk, forward buffers only)
   CUtensorMap tmb[kNSpec];
+  CUtensorMap tmw[kNSpec];  // as tmy, 16 columns at every r (the plane kernels)
   CUtensorMap tmc[4];
   int r;
   int N;

@@ -461,7 +461,7 @@ __device__ __forceinline__ bool yfwd_tile(const Solve& S, int X, int kz0, int ki
 }
 
 template <int L, bool BWD>
-__global__ void __launch_bounds__(ynt<L>(), BWD ? 4 : (L >= 256 ? 3 : 5)) k_yfwd(const __grid_constant__ Solve s0,
+__global__ void __launch_bounds__(ynt<L>(), L == 256 ? (BWD ? 8 : 6) : (BWD ? 4 : (L >= 256 ? 3 : 5))) k_yfwd(const __grid_constant__ Solve s0,
                                                    const Solve* __restrict__ tab) {
   using P = Pen<L>;
   constexpr int NT = ynt<L>();
@@ -619,7 +619,7 @@ __device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int pa
 }
 
 template <int L, int NCH>
-__global__ void __launch_bounds__(ynt<L>(), 4)
+__global__ void __launch_bounds__(ynt<L>(), L == 256 ? 8 : 4)
     k_yinv(const __grid_constant__ Solve s0, const Solve* __restrict__ tab) {
   using P = Pen<L>;
   constexpr int NT = ynt<L>();

@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(fwd_threads<L, C>(), 512 / fwd_threads<L, C>()
       __syncthreads();
       if (tid == 0) {
         for (int b = 0; b < F::NB; ++b)
-          tma_store_3d(&S.tmy[buf], c * SPC + 16 * b, 0, X, sbox + b * F::BOX);
+          tma_store_3d(&S.tmw[buf], c * SPC + 16 * b, 0, X, sbox + b * F::BOX);
         tma_store_commit();
         tma_store_wait_read();
       }
@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(kNT, plane_minb<L, C>(1))
   if (tid == 0) {
     mbar_init(&bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    chunk_load<L, C>(&S.tmy[kSpChi], sbox, c * P::SPC, X, &bar);
+    chunk_load<L, C>(&S.tmw[kSpChi], sbox, c * P::SPC, X, &bar);
   }
   // While the first tiles land, every CTA sums the x pass's partials into the
   // scalars of Eq. 4 for itself; the first one publishes them.
@@ -492,7 +492,7 @@ __global__ void __launch_bounds__(kNT, plane_minb<L, C>(1))
   bool alive = true;
   for (int cb = 0; cb < P::SPC && alive; cb += P::CHK) {
     const int s_first = c * P::SPC + cb;
-    if (tid == 0 && cb > 0) chunk_load<L, C>(&S.tmy[kSpChi], sbox, s_first, X, &bar);
+    if (tid == 0 && cb > 0) chunk_load<L, C>(&S.tmw[kSpChi], sbox, s_first, X, &bar);
     const bool head = (c == 0 && cb == 0);
     float2 nyq[P::R1];
     if (head && g == 0 && P::H >= 16) {
@@ -672,7 +672,7 @@ __global__ void __launch_bounds__(kNT, plane_minb<L, C>(2))
     fence_async_smem();
     __syncthreads();
     if (tid == 0) {
-      chunk_store<L, C>(&S.tmy[kSpD], sbox, s_first, X);
+      chunk_store<L, C>(&S.tmw[kSpD], sbox, s_first, X);
       tma_store_wait_read();
     }
     __syncthreads();
@@ -803,7 +803,7 @@ __global__ void __launch_bounds__(binv_threads<L, C>(), binv_smem<L, C>() <= 113
     for (int k = 0; k < 2; ++k) {
       mbar_expect_tx(&barL[k], B::NB * B::BOX * (uint32_t)sizeof(float2));
       for (int b = 0; b < B::NB; ++b)
-        tma_load_3d((k ? buf1 : buf0) + b * B::BOX, &S.tmy[k ? kSpD : kSpChi], s_first + 16 * b, 0, X, &barL[k]);
+        tma_load_3d((k ? buf1 : buf0) + b * B::BOX, &S.tmw[k ? kSpD : kSpChi], s_first + 16 * b, 0, X, &barL[k]);
     }
   }
   __syncthreads();
@@ -999,7 +999,7 @@ __global__ void __launch_bounds__(BinvChGeo<L>::NT, 3)
     mbar_init(&bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     mbar_expect_tx(&bar, B::NB * B::BOX * (uint32_t)sizeof(float2));
-    for (int b = 0; b < B::NB; ++b) tma_load_3d(buf + b * B::BOX, &S.tmy[sp], 16 * b, 0, X, &bar);
+    for (int b = 0; b < B::NB; ++b) tma_load_3d(buf + b * B::BOX, &S.tmw[sp], 16 * b, 0, X, &bar);
   }
   __syncthreads();
   TwTab<L> twr{twt, t};

@@ -59,7 +59,7 @@ constexpr size_t xpass_smem() {
 // one kz column along x in registers (the box column doubles as its exchange
 // buffer), and TMA stores the results.
 template <int L, bool BWD>
-__global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ? 2 : 3) : 5))
+__global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ? 5 : 6) : 5))
     k_xpass(const __grid_constant__ Solve s0, const Solve* __restrict__ tab) {
   using P = XGeo<L>;
   constexpr int NCH = P::template nch<BWD>();

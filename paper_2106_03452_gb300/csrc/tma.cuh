@@ -10,6 +10,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "dpsr_dev.cuh"
+
 namespace dpsr {
 
 // float2 index of complex c (0..15) of box row q under the 128-byte swizzle.
