@@ -346,6 +346,7 @@ struct Scalars {
   float g_a, g_s, g_w;    // backward: G^ = g_a * FFT(dchi) + g_s + g_w * W^
   float c_mu;             // backward: weight of the stored lookup gradient
   double loss;            // L_DPSR of Eq. 9 (mean squared error against a target grid)
+  int bparts;             // partial sums that the backward x pass has yet to turn into the above (0: done)
   // arrival counters of the last-block reductions: [1] backward plane pass,
   // [2] the L_DPSR loss (reset by the binning's scatter of every forward, and
   // each by its own last block)

@@ -97,10 +97,29 @@ __device__ __forceinline__ FwdScalars fwd_scalars(const Solve& S, double a, doub
   return q;
 }
 
+// Those of its adjoint: a = sum dchi, b = sum dchi * chi = alpha * sum dchi (chi' - mu);
+// with alpha = m / |s|: D = b / alpha = b |s| / m and
+// s_bar = -m sign(s) D / s^2 = -sign(s) D alpha^2 / m.
+struct BwdScalars {
+  double D, s_bar, mu_bar;
+  float g_a, g_s, g_w;
+};
+__device__ __forceinline__ BwdScalars bwd_scalars(const Solve& S, double a, double b) {
+  BwdScalars q;
+  const double inv_n = (double)__frcp_rn((float)S.r * (float)S.r * (float)S.r);
+  const double alpha = S.sc->alpha, s = S.sc->s;
+  q.D = alpha > 0 ? b * fabs(s) * (1.0 / (double)kM) : 0.0;
+  q.s_bar = -(s > 0 ? 1.0 : -1.0) * q.D * alpha * alpha * (1.0 / (double)kM);
+  q.mu_bar = -alpha * a - q.s_bar;
+  q.g_a = (float)(alpha * inv_n);
+  q.g_s = (float)(q.s_bar * inv_n);
+  q.g_w = (float)(q.mu_bar * inv_n * S.inv_N);
+  return q;
+}
+
 // Thread 0: the scalars from the reduced sums.
 __device__ inline void finalize_scalars(const Solve& S, double a, double b, bool bwd) {
   Scalars* sc = S.sc;
-  const double inv_n = (double)__frcp_rn((float)S.r * (float)S.r * (float)S.r);
   if (!bwd) {
     const FwdScalars q = fwd_scalars(S, a, b);
     sc->acc_mu = a;
@@ -112,22 +131,15 @@ __device__ inline void finalize_scalars(const Solve& S, double a, double b, bool
     sc->b_chi = q.b_chi;
     if (q.bad) atomicOr(S.status, kStDegenerate);
   } else {
-    // a = sum dchi, b = sum dchi * chi = alpha * sum dchi (chi' - mu);
-    // with alpha = m / |s|: D = b / alpha = b |s| / m and
-    // s_bar = -m sign(s) D / s^2 = -sign(s) D alpha^2 / m
-    const double alpha = sc->alpha, s = sc->s;
-    const double Ssum = a;
-    const double D = alpha > 0 ? b * fabs(s) * (1.0 / (double)kM) : 0.0;
-    const double s_bar = -(s > 0 ? 1.0 : -1.0) * D * alpha * alpha * (1.0 / (double)kM);
-    const double mu_bar = -alpha * Ssum - s_bar;
-    sc->S = Ssum;
-    sc->D = D;
-    sc->s_bar = s_bar;
-    sc->mu_bar = mu_bar;
-    sc->g_a = (float)(alpha * inv_n);
-    sc->g_s = (float)(s_bar * inv_n);
-    sc->g_w = (float)(mu_bar * inv_n * S.inv_N);
-    sc->c_mu = sc->g_w;
+    const BwdScalars q = bwd_scalars(S, a, b);
+    sc->S = a;
+    sc->D = q.D;
+    sc->s_bar = q.s_bar;
+    sc->mu_bar = q.mu_bar;
+    sc->g_a = q.g_a;
+    sc->g_s = q.g_s;
+    sc->g_w = q.g_w;
+    sc->c_mu = q.g_w;
   }
 }
 
@@ -171,6 +183,7 @@ __device__ inline void last_block_finalize(const Solve& S, int ticket, int nbloc
   if (tid == 0) {
     finalize_scalars(S, ff_to_double(x), ff_to_double(y), bwd);
     S.sc->ticket[ticket] = 0;
+    if (bwd) S.sc->bparts = 0;
   }
 }
 

@@ -677,11 +677,15 @@ __global__ void __launch_bounds__(kNT, plane_minb<L, C>(2))
     }
     __syncthreads();
   }
-  // block partial sums (float-float, fixed order); the last CTA of the solve
-  // turns them into the adjoint scalars
+  // block partial sums (float-float, fixed order), turned into the adjoint's
+  // scalars by the x pass while its tiles land (a ticket, and the last CTA
+  // summing alone behind all others, took about 2 us at the end of this pass)
   FF dS = {accS, 0.f}, dD = {accD, 0.f};
   block_sum_ff<kNT>(dS, dD);
-  last_block_finalize<kNT>(S, 1, (int)gridDim.x, (int)blockIdx.x, dS, dD, true);
+  if (tid == 0) {
+    S.part[blockIdx.x] = make_float4(dS.hi, dS.lo, dD.hi, dD.lo);
+    if (blockIdx.x == 0) S.sc->bparts = (int)gridDim.x;
+  }
   cl.sync();
 }
 

@@ -233,13 +233,30 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
     // FFT_x of (g_a FFT_zy(dchi) + g_w W~ + g_s delta_{x=0}): the three terms
     // of the adjoint spectrum combined before the transform (it is linear).
     const Scalars* sc = S.sc;
-    const float ga = sc->g_a, gs = sc->g_s, gw = sc->g_w;
+    const int np = sc->bparts;
+    __shared__ float coef[3];
+    if (np > 0) {  // the plane pass left its partial sums: every CTA adds them up, the first one publishes
+      FF x, y;
+      sum_partials<P::NT>(S, np, x, y);
+      if (tid == 0) {
+        const BwdScalars q = bwd_scalars(S, ff_to_double(x), ff_to_double(y));
+        coef[0] = q.g_a;
+        coef[1] = q.g_s;
+        coef[2] = q.g_w;
+        if (blockIdx.x == 0 && blockIdx.y == 0) finalize_scalars(S, ff_to_double(x), ff_to_double(y), true);
+      }
+    } else if (tid == 0) {
+      coef[0] = sc->g_a;
+      coef[1] = sc->g_s;
+      coef[2] = sc->g_w;
+    }
     box_wait(0);
     box_wait(1);
     if (!__syncthreads_and(ok)) {  // both tiles are needed from the start
       leave();
       return;
     }
+    const float ga = coef[0], gs = coef[1], gw = coef[2];
 #pragma unroll
     for (int j = 0; j < P::R1; ++j) {
       const int x = t + P::T * j;
