@@ -173,8 +173,9 @@ __device__ __forceinline__ void r2c_pair_st(int t, const Tw& tw, float* p, const
 // i < L, addresses the pair's storage (A's slots for i < H, B's for
 // i >= H); it is also the FFT exchange area and receives (a[z], b[z]) at
 // x(z), unnormalised.
-template <int L, class Tw, class Acc>
-__device__ __forceinline__ void c2r_acc(int t, const Tw& tw, Acc x) {
+// out(z, (a[z], b[z])) sees each value on its way there.
+template <int L, class Tw, class Acc, class Out>
+__device__ __forceinline__ void c2r_acc(int t, const Tw& tw, Acc x, Out out) {
   constexpr int R1 = Shape<L>::R1, T = Shape<L>::T, H = L / 2;
   float2 v[R1];
 #pragma unroll
@@ -194,7 +195,10 @@ __device__ __forceinline__ void c2r_acc(int t, const Tw& tw, Acc x) {
   group_sync<T>();
   fft_r<L, +1>(v, t, x, tw);
 #pragma unroll
-  for (int j = 0; j < R1; ++j) x(t + T * j) = v[j];
+  for (int j = 0; j < R1; ++j) {
+    x(t + T * j) = v[j];
+    out(t + T * j, v[j]);
+  }
 }
 
 // ===========================================================================
@@ -826,7 +830,23 @@ __device__ __forceinline__ bool zinv_tile(const Solve& S, int tile, float2* sb, 
   constexpr int NP = NCH * NR / 2;
   for (int p0 = 0; p0 < NP; p0 += G) {
     const int pi = p0 + g;
-    if (pi < NP) c2r_acc<L>(t, twr, pair(pi / (NR / 2), pi % (NR / 2)));  // whole groups
+    if (pi < NP) {  // whole groups
+      const int ch = pi / (NR / 2), p = pi % (NR / 2);
+      // chi (Eq. 4) straight from registers, the halo pair's rows excepted: read back
+      // from shared memory it went through a unit that ncu had at 79 % (34.9 -> 31.0
+      // us at r = 256, 245 -> 225 at r = 512)
+      if constexpr (NCH == 1) {
+        float* row = S.chi + ((size_t)X * L + y0 + 2 * p) * L;
+        const bool own = p < YB / 2;
+        c2r_acc<L>(t, twr, pair(ch, p), [&](int z, float2 v) {
+          if (!own) return;
+          row[z] = fmaf(a_chi, v.x, b_chi);
+          row[L + z] = fmaf(a_chi, v.y, b_chi);
+        });
+      } else {
+        c2r_acc<L>(t, twr, pair(ch, p), [](int, float2) {});
+      }
+    }
   }
   __syncthreads();
   // value of channel ch, tile row ly, column z
@@ -834,18 +854,6 @@ __device__ __forceinline__ bool zinv_tile(const Solve& S, int tile, float2* sb, 
     const float2 f = pair(ch, ly >> 1)(z);
     return (ly & 1) ? f.y : f.x;
   };
-  if constexpr (NCH == 1) {
-    float* chi = S.chi;
-    for (int i = tid; i < YB * L / 4; i += NT) {
-      const int ly = i / (L / 4), z4 = (i % (L / 4)) * 4;
-      float4 o;
-      o.x = fmaf(a_chi, val(0, ly, z4), b_chi);
-      o.y = fmaf(a_chi, val(0, ly, z4 + 1), b_chi);
-      o.z = fmaf(a_chi, val(0, ly, z4 + 2), b_chi);
-      o.w = fmaf(a_chi, val(0, ly, z4 + 3), b_chi);
-      reinterpret_cast<float4*>(chi + ((size_t)X * L + y0 + ly) * L)[z4 / 4] = o;
-    }
-  }
   for (int v = tid; v < nv; v += NT) {
     const int side = v < n0 ? 0 : 1;
     const int i = side ? r1.x + (v - n0) : r0.x + v;
