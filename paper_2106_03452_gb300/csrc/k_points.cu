@@ -306,6 +306,9 @@ __global__ void __launch_bounds__(256) k_grid_splat(float* __restrict__ grid, in
 // arrive writes sc->loss), deterministic. n = r^3 is a power of two, so 2/n
 // and 1/n are exact.
 // ---------------------------------------------------------------------------
+// float4 of each grid per thread. Every block costs a ticket (a fence and an
+// atomic on its instance's counter): a batch's two classes 45.4 us with 2, 40.9 with 8.
+constexpr int kMsePer = 8;
 __global__ void __launch_bounds__(256) k_mse_grad(const __grid_constant__ Solve s0,
                                                   const Solve* __restrict__ tab) {
   constexpr int NT = 256;
@@ -318,9 +321,10 @@ __global__ void __launch_bounds__(256) k_mse_grad(const __grid_constant__ Solve 
   const float4* tg = reinterpret_cast<const float4*>(S.target);
   float4* g = reinterpret_cast<float4*>(S.dchi_rw);
   // this instance's blocks (a batch launch sizes the grid for its largest r)
-  const int nblk = (int)min((int64_t)gridDim.x, max(n4 / (2 * NT), (int64_t)1));
+  const int nblk = (int)min((int64_t)gridDim.x, max(n4 / (kMsePer * NT), (int64_t)1));
   if ((int)blockIdx.x >= nblk) return;
   float acc = 0.f;
+#pragma unroll 4
   for (int64_t i = blockIdx.x * (int64_t)NT + threadIdx.x; i < n4; i += (int64_t)nblk * NT) {
     const float4 a = __ldcs(chi + i), b = __ldcs(tg + i);
     const float4 d = make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
@@ -350,11 +354,11 @@ __global__ void __launch_bounds__(256) k_mse_grad(const __grid_constant__ Solve 
   }
 }
 
-// Blocks of the loss pass for grid size r: two float4 per thread, at most
+// Blocks of the loss pass for grid size r: kMsePer float4 per thread, at most
 // the r * 16 block partials the workspace holds.
 int mse_blocks(int r) {
   const int64_t n4 = (int64_t)r * r * r / 4;
-  const int64_t b = n4 / (2 * 256);
+  const int64_t b = n4 / (kMsePer * 256);
   return (int)std::max<int64_t>(1, std::min<int64_t>(b, (int64_t)r * 16));
 }
 
