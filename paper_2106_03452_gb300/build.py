@@ -1,7 +1,10 @@
-"""Build libdpsr.so in-tree with nvcc for sm_103a (GB300).
+"""Build libdpsr.so in-tree with nvcc for sm_103a (GB300), and the PyTorch
+binding of its hot calls with g++.
 
 Each .cu translation unit is compiled in parallel, then linked into
-paper_2106_03452_gb300/_build/libdpsr.so. No torch, no cmake.
+paper_2106_03452_gb300/_build/libdpsr.so (no torch, no cmake);
+csrc/torch_bind.cpp becomes _build/_dpsr_torch.so next to it, against the
+headers of the installed PyTorch.
 """
 from __future__ import annotations
 
@@ -11,6 +14,7 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -21,6 +25,8 @@ LIB = os.path.join(BUILD, "libdpsr.so")
 # the debug build (bounds checks on data-dependent indices, DPSR_DEBUG_CHECKS)
 BUILD_DEBUG = os.path.join(HERE, "_build_debug")
 LIB_DEBUG = os.path.join(BUILD_DEBUG, "libdpsr.so")
+BIND = "torch_bind.cpp"
+BIND_NAME = "_dpsr_torch.so"
 SOURCES = ["dpsr_api.cu", "k_plane.cu", "k_xpass.cu", "k_points.cu", "k_pencil.cu", "dpsr_static.cu", "dpsr_batch.cu", "dpsr_serve.cu", "k_mesh.cu", "k_opt.cu", "k_chamfer.cu", "tune_cache.cu", "k_peak.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
@@ -34,6 +40,24 @@ def _nvcc() -> str:
     raise RuntimeError("nvcc not found: the CUDA toolkit is required to build libdpsr")
 
 
+def _torch():
+    import torch
+    return torch
+
+
+def _bind_flags():
+    """(compile, link) flags of the binding: PyTorch's headers and libraries."""
+    torch = os.path.dirname(_torch().__file__)
+    inc = [os.path.join(torch, "include"), os.path.join(torch, "include", "torch", "csrc", "api", "include"),
+           sysconfig.get_paths()["include"], os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include"),
+           INCLUDE]
+    abi = f"-D_GLIBCXX_USE_CXX11_ABI={int(_torch().compiled_with_cxx11_abi())}"
+    comp = ["-O2", "-std=c++17", "-fPIC", "-fvisibility=hidden", abi, *(f"-I{d}" for d in inc)]
+    link = [f"-L{os.path.join(torch, 'lib')}", "-lc10", "-lc10_cuda", "-ltorch", "-ltorch_cpu", "-ltorch_cuda",
+            "-ltorch_python", "-ldpsr", "-Wl,-rpath,$ORIGIN"]
+    return comp, link
+
+
 def _fingerprint(extra=()) -> str:
     h = hashlib.sha256()
     for d, names in ((CSRC, sorted(os.listdir(CSRC))), (INCLUDE, sorted(os.listdir(INCLUDE)))):
@@ -44,6 +68,7 @@ def _fingerprint(extra=()) -> str:
                 with open(p, "rb") as f:
                     h.update(f.read())
     h.update(" ".join(ARCH + FLAGS + list(extra)).encode())
+    h.update(f"{_torch().__version__} {sysconfig.get_paths()['include']}".encode())
     return h.hexdigest()
 
 
@@ -57,7 +82,7 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
     fp = _fingerprint(extra)
     if not force and os.path.exists(lib) and os.path.exists(stamp):
         with open(stamp) as f:
-            if f.read().strip() == fp:
+            if f.read().strip() == fp and os.path.exists(os.path.join(build_dir, BIND_NAME)):
                 return lib
     nvcc = _nvcc()
     objs = []
@@ -74,14 +99,28 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
             sys.stderr.write(res.stderr)
         return obj
 
-    with cf.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
+    comp, libs = _bind_flags()
+    bind_obj = os.path.join(build_dir, "torch_bind.o")
+
+    def run(cmd, what):
+        res = subprocess.run(cmd, capture_output=True, text=True)
+        if res.returncode != 0:
+            raise RuntimeError(f"{what} failed:\n{res.stderr[-6000:]}")
+
+    with cf.ThreadPoolExecutor(max_workers=len(SOURCES) + 1) as ex:
+        bind = ex.submit(run, ["g++", *comp, "-c", os.path.join(CSRC, BIND), "-o", bind_obj], f"g++ on {BIND}")
         objs = list(ex.map(compile_one, SOURCES))
+        bind.result()
     tmp = lib + f".tmp{os.getpid()}"
     cmd = [nvcc, *ARCH, "-shared", "-o", tmp, *objs, "-lcudart"]
     res = subprocess.run(cmd, capture_output=True, text=True)
     if res.returncode != 0:
         raise RuntimeError(f"link failed:\n{res.stderr[-4000:]}")
     os.replace(tmp, lib)
+    ext = os.path.join(build_dir, BIND_NAME)
+    tmp = ext + f".tmp{os.getpid()}"
+    run(["g++", "-shared", "-o", tmp, bind_obj, f"-L{build_dir}", *libs], "link of the PyTorch binding")
+    os.replace(tmp, ext)
     with open(stamp, "w") as f:
         f.write(fp)
     return lib

@@ -32,6 +32,7 @@ class Plan:
         self.r, self.sigma = int(r), float(sigma)
         self.box = None if box is None else tuple(float(v) for v in box)
         self.device = torch.device(device) if device is not None else torch.device("cuda", torch.cuda.current_device())
+        self._index = self.device.index if self.device.index is not None else torch.cuda.current_device()
         with torch.cuda.device(self.device):
             if self.box is None:
                 self.handle = L.dpsr_plan_create(self.r, self.sigma)
@@ -57,6 +58,10 @@ class Plan:
         L.dpsr_plan_set_stream(self.handle, torch.cuda.current_stream(self.device).cuda_stream)
 
     def forward(self, points: torch.Tensor, normals: torch.Tensor, chi_out=None) -> torch.Tensor:
+        if chi_out is None:
+            chi = L.binding().plan_forward(self, points, normals)
+            if chi is not None:
+                return chi
         points = _dev_f32(points, "points")
         normals = _dev_f32(normals, "normals", points.shape)
         if points.dim() != 2 or points.shape[1] != 3:
@@ -117,7 +122,14 @@ class Plan:
 
 
 class DPSRFunction(torch.autograd.Function):
-    """chi = DPSR(points, normals) with the library's adjoint as backward."""
+    """chi = DPSR(points, normals) with the library's adjoint as backward.
+    apply() runs plain CUDA tensors through the same function in C++
+    (csrc/torch_bind.cpp), everything else through the methods below."""
+
+    @classmethod
+    def apply(cls, points, normals, plan):
+        chi = L.binding().layer(points, normals, plan)
+        return super().apply(points, normals, plan) if chi is None else chi
 
     @staticmethod
     def forward(ctx, points, normals, plan: Plan):

@@ -16,8 +16,10 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 # (build.build(debug=True)) instead of the release one
 _DEBUG = os.environ.get("DPSR_DEBUG_CHECKS", "") == "1"
 LIB_PATH = os.path.join(_HERE, "_build_debug" if _DEBUG else "_build", "libdpsr.so")
+BIND_PATH = os.path.join(os.path.dirname(LIB_PATH), "_dpsr_torch.so")
 _lock = threading.Lock()
 _lib = None
+_bind = None
 
 DPSR_OK = 0
 DPSR_EINVAL = -1
@@ -128,6 +130,28 @@ def load():
                 f.argtypes = args
             _lib = lib
     return _lib
+
+
+def binding():
+    """The in-tree PyTorch binding (csrc/torch_bind.cpp): the hot calls on
+    plain CUDA tensors without Python on the way. Its entries return None for
+    anything else. Raises if it has not been built."""
+    global _bind
+    if _bind is None:
+        load()
+        with _lock:
+            if _bind is None:
+                if not os.path.exists(BIND_PATH):
+                    raise RuntimeError(f"the PyTorch binding is not built ({BIND_PATH} missing): run "
+                                       f"`python -m paper_2106_03452_gb300.build{' --debug' if _DEBUG else ''}`")
+                import importlib.util
+                import torch  # noqa: F401  (its libraries first)
+                spec = importlib.util.spec_from_file_location("_dpsr_torch", BIND_PATH)
+                mod = importlib.util.module_from_spec(spec)
+                spec.loader.exec_module(mod)
+                mod.init(DPSRError)
+                _bind = mod
+    return _bind
 
 
 def check(code: int, what: str) -> None:

@@ -20,7 +20,13 @@ from .dpsr import Plan, dpsr
 
 class GridSample(torch.autograd.Function):
     """chi(q): trilinear lookup of an r^3 grid at query points, with the
-    rasterization of the incoming gradient as its backward."""
+    rasterization of the incoming gradient as its backward. apply() as in
+    DPSRFunction."""
+
+    @classmethod
+    def apply(cls, chi, q):
+        v = L.binding().grid_sample(chi, q)
+        return super().apply(chi, q) if v is None else v
 
     @staticmethod
     def forward(ctx, chi, q):

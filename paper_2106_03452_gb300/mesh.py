@@ -18,6 +18,9 @@ from . import libdpsr as L
 
 def extract(chi: torch.Tensor, level: float = 0.0):
     """(tris T x 3 x 3, normals T x 3) of the set chi = level (CUDA tensors)."""
+    out = L.binding().extract(chi, level)
+    if out is not None:
+        return out
     if not chi.is_cuda:
         raise ValueError("chi must be a CUDA tensor (there is no CPU path)")
     chi = chi.contiguous().float()
@@ -39,6 +42,9 @@ def extract(chi: torch.Tensor, level: float = 0.0):
 def sample(tris: torch.Tensor, normals: torch.Tensor, M: int, seed: int = 0):
     """M points drawn uniformly by area on a triangle soup (dpsr_mesh_sample),
     with the normal of the triangle each falls in."""
+    out = L.binding().sample(tris, normals, M, int(seed) & (2 ** 64 - 1))
+    if out is not None:
+        return out
     T = tris.shape[0]
     ws = torch.empty(T + (T + 1023) // 1024 + 1, dtype=torch.float64, device=tris.device)
     p = torch.empty((M, 3), device=tris.device)
@@ -82,7 +88,13 @@ def largest_component(chi: torch.Tensor, level: float = 0.0):
 
 
 class MeshPoints(torch.autograd.Function):
-    """(points, normals) on the level set of chi; backward: Eq. 6."""
+    """(points, normals) on the level set of chi; backward: Eq. 6. apply() as
+    in DPSRFunction."""
+
+    @classmethod
+    def apply(cls, chi, level=0.0, samples=0, seed=0):
+        out = L.binding().mesh_points(chi, level, samples, int(seed) & (2 ** 64 - 1))
+        return super().apply(chi, level, samples, seed) if out is None else out
 
     @staticmethod
     def forward(ctx, chi, level=0.0, samples=0, seed=0):

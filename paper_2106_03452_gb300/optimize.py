@@ -31,7 +31,13 @@ PAPER_LEVELS = ((32, 2.0, 1000), (64, 2.0, 1000), (128, 3.0, 1000), (256, 3.0, 2
 
 class ChamferLoss(torch.autograd.Function):
     """Bi-directional L2 Chamfer distance between a (differentiable) and b
-    (dpsr_chamfer_tree: exact nearest neighbours in both directions)."""
+    (dpsr_chamfer_tree: exact nearest neighbours in both directions).
+    apply() as in DPSRFunction."""
+
+    @classmethod
+    def apply(cls, a, b):
+        loss = L.binding().chamfer(a, b)
+        return super().apply(a, b) if loss is None else loss
 
     @staticmethod
     def forward(ctx, a, b):
