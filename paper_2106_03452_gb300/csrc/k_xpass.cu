@@ -278,7 +278,12 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
 #pragma unroll
         for (int j = 0; j < P::R1; ++j) c0.put(j, a[j]);
       }
-      group_sync<P::T, IL>();
+      fence_async_smem();
+      __syncthreads();
+      if (tid == 0) {  // Q1 leaves while Q2 is transformed: 61.7 -> 60.4 us at r = 256, 635 -> 615 us at r = 512
+        for (int x = 0; x < L; x += tma_rows(L)) tma_store_3d(&S.tmx[kSpD], kz0, ky, x, box + x * P::KC);
+        tma_store_commit();
+      }
 #pragma unroll
       for (int j = 0; j < P::R1; ++j) a[j] = c1.get(j);
       fft_c<L, +1, IL>(a, c1, twr);
@@ -290,10 +295,8 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
     fence_async_smem();
     __syncthreads();
     if (tid == 0) {
-      for (int x = 0; x < L; x += tma_rows(L)) {
-        tma_store_3d(&S.tmx[kSpD], kz0, ky, x, box + x * P::KC);             // Q1
+      for (int x = 0; x < L; x += tma_rows(L))
         tma_store_3d(&S.tmx[kSpChi], kz0, ky, x, box + P::BOX + x * P::KC);  // Q2
-      }
       tma_store_commit();
       tma_store_wait_read();
     }
