@@ -932,14 +932,16 @@ int dpsr_solve_host(dpsr_plan p, const float* points, const float* normals, int6
   HostIo v = host_io_view(p, N);
   const size_t nb = sizeof(float) * 3 * N, gb = sizeof(float) * p->r * p->r * p->r;
   cudaStream_t st = p->stream, cs = p->copy_stream;
-  // copy stream: the upstream gradient goes up while the forward pass runs;
-  // the plan's stream (and the staging it reuses) is free of earlier work first
+  // The points go up first and alone: the forward pass waits for nothing else.
+  // The upstream gradient follows on the copy stream, behind them and behind
+  // earlier work on the plan's stream (whose staging it reuses), while the
+  // forward pass runs.
+  if (cudaMemcpyAsync(v.pts, points, nb, cudaMemcpyHostToDevice, st) != cudaSuccess ||
+      cudaMemcpyAsync(v.nrm, normals, nb, cudaMemcpyHostToDevice, st) != cudaSuccess)
+    return DPSR_ECUDA;
   if (cudaEventRecord(p->ev_fwd, st) != cudaSuccess || cudaStreamWaitEvent(cs, p->ev_fwd, 0) != cudaSuccess ||
       cudaMemcpyAsync(v.dchi, dchi, gb, cudaMemcpyHostToDevice, cs) != cudaSuccess ||
       cudaEventRecord(p->ev_dchi, cs) != cudaSuccess)
-    return DPSR_ECUDA;
-  if (cudaMemcpyAsync(v.pts, points, nb, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-      cudaMemcpyAsync(v.nrm, normals, nb, cudaMemcpyHostToDevice, st) != cudaSuccess)
     return DPSR_ECUDA;
   rc = dpsr_forward(p, v.pts, v.nrm, N, v.chi);
   if (rc != DPSR_OK) return rc;
