@@ -1179,7 +1179,8 @@ static cudaError_t launch_pencil_t(int kind, const Solve& s, const Solve* tab, i
       }
       e = launch_k(k_yinv<L, 1>, dim3(L * P::NKC + 1, 1, count), dim3(nt), a, st, 0, s, tab);
       if (e == cudaSuccess)
-        e = launch_k(k_zinv<L, 1>, dim3(nz, 1, count), dim3(ZiGeo<L, 1>::NT), b, st, 0, s, tab);
+        // from r = 256 on after the y pass: 39 -> 33 us at r = 256, 232 -> 228 at r = 512; below, the gap costs more
+        e = launch_at(L < 256, k_zinv<L, 1>, dim3(nz, 1, count), dim3(ZiGeo<L, 1>::NT), b, st, 0, s, tab);
       return e;
     }
     case 2: {
@@ -1205,7 +1206,7 @@ static cudaError_t launch_pencil_t(int kind, const Solve& s, const Solve* tab, i
           e = set_smem(k_yadj<L>, a);
           if (e != cudaSuccess) return e;
         }
-        e = launch_k(k_yadj<L>, dim3(L * YDir<L>::NKC, 2, count), dim3(ColDir<L>::NT), a, st, 0, s, tab);
+        e = launch_after(k_yadj<L>, dim3(L * YDir<L>::NKC, 2, count), dim3(ColDir<L>::NT), a, st, 0, s, tab);
       } else {
         constexpr size_t a = yinv_smem<L, 3>();
         if (!attr_set[3]) {
@@ -1221,7 +1222,8 @@ static cudaError_t launch_pencil_t(int kind, const Solve& s, const Solve* tab, i
         nz = persistent_ctas(k_zinv<L, 3>, ZiGeo<L, 3>::NT, b, L * P::NYB, 1);
         attr_set[3] = true;
       }
-      return launch_k(k_zinv<L, 3>, dim3(nz, 1, count), dim3(ZiGeo<L, 3>::NT), b, st, 0, s, tab);
+      // r = 512: 231 -> 222 us after the y pass; r = 256: 36 -> 34 us early
+      return launch_at(L < 512, k_zinv<L, 3>, dim3(nz, 1, count), dim3(ZiGeo<L, 3>::NT), b, st, 0, s, tab);
     }
   }
 }

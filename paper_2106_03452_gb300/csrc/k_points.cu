@@ -253,8 +253,8 @@ __global__ void __launch_bounds__(256) k_combine(const __grid_constant__ Solve s
 cudaError_t launch_combine(const Solve& s, const Solve* tab, int count, int nmax, bool split,
                            cudaStream_t st) {
   const int blocks = min(max((nmax + 255) / 256, 1), 1184);
-  return split ? launch_k(k_combine<true>, dim3(blocks, 1, count), dim3(256), 0, st, 0, s, tab)
-               : launch_k(k_combine<false>, dim3(blocks, 1, count), dim3(256), 0, st, 0, s, tab);
+  return split ? launch_after(k_combine<true>, dim3(blocks, 1, count), dim3(256), 0, st, 0, s, tab)
+               : launch_after(k_combine<false>, dim3(blocks, 1, count), dim3(256), 0, st, 0, s, tab);
 }
 
 // ---------------------------------------------------------------------------

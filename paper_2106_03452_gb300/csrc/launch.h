@@ -15,11 +15,12 @@ namespace dpsr {
 bool pdl_enabled();
 void pdl_suspend(bool off);
 
-// cudaLaunchKernelEx with an optional cluster size (x) and the programmatic
-// launch attribute.
+// cudaLaunchKernelEx with an optional cluster size (x). `early`: with the
+// programmatic launch attribute, so that the kernel's CTAs take their places
+// while the previous kernel drains and wait there (2 to 4 us a kernel).
 template <class... KArgs, class... Args>
-cudaError_t launch_k(void (*fn)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                     int cluster, Args&&... args) {
+cudaError_t launch_at(bool early, void (*fn)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                      int cluster, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -34,7 +35,7 @@ cudaError_t launch_k(void (*fn)(KArgs...), dim3 grid, dim3 block, size_t smem, c
     attr[n].val.clusterDim.z = 1;
     ++n;
   }
-  if (pdl_enabled()) {
+  if (early && pdl_enabled()) {
     attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[n].val.programmaticStreamSerializationAllowed = 1;
     ++n;
@@ -42,6 +43,22 @@ cudaError_t launch_k(void (*fn)(KArgs...), dim3 grid, dim3 block, size_t smem, c
   cfg.attrs = attr;
   cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, fn, std::forward<Args>(args)...);
+}
+template <class... KArgs, class... Args>
+cudaError_t launch_k(void (*fn)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cluster,
+                     Args&&... args) {
+  return launch_at(true, fn, grid, block, smem, st, cluster, std::forward<Args>(args)...);
+}
+// A kernel that starts when the previous one has left the SMs. For those that
+// lose more by an early start than the gap costs: a CTA placed early finds the
+// SM split as the previous kernel's shared memory asked for, and keeps it so.
+// Kernels that read through L1 then run with next to none of it (adjoint y
+// pass at r = 256: 57 us early, 44 after; combine 11 and 8), and persistent
+// CTAs may not all fit at once (inverse z pass of the forward: 39 and 33 us).
+template <class... KArgs, class... Args>
+cudaError_t launch_after(void (*fn)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cluster,
+                         Args&&... args) {
+  return launch_at(false, fn, grid, block, smem, st, cluster, std::forward<Args>(args)...);
 }
 
 // Plane kernels: kind 0 = forward splat/z/y, 1 = forward inverse y/z + lookup
