@@ -318,9 +318,14 @@ __global__ void __launch_bounds__(kScanNT) k_block_offsets(double* __restrict__ 
 }
 
 // A sample's triangle by two searches: the last block whose offset does not
-// exceed its draw (offsets in shared memory up to 2 048 blocks, two million
-// triangles), then the first triangle of the block whose sum does. No pass
-// adds the offsets to the sums first.
+// exceed its draw, then the first triangle of the block whose sum does. No pass
+// adds the offsets to the sums first. Up to 2 048 blocks (two million
+// triangles) every CTA adds the block totals up in shared memory itself;
+// beyond that k_block_offsets has. The second search takes three pivots a step:
+// five dependent reads of a 1 024-triangle block instead of ten. The searches
+// live in L1, and the grid is small: launched early it would crowd onto the SMs
+// that the scan leaves free, so it waits (20 000 points on 150 001 triangles,
+// both kernels: 40 us early with the offsets in a launch of their own, 22.5).
 constexpr int kOffShared = 2048;
 constexpr int kSampleNT = 64;  // 20 000 samples: 313 blocks, two per SM (the searches compare on the FP64 pipe)
 __global__ void __launch_bounds__(kSampleNT) k_sample(const float* __restrict__ tris, const float* __restrict__ nrm,
@@ -328,15 +333,44 @@ __global__ void __launch_bounds__(kSampleNT) k_sample(const float* __restrict__ 
                                                 const double* __restrict__ tot, int nblocks, int64_t M, uint64_t seed,
                                                 float* __restrict__ p, float* __restrict__ n) {
   __shared__ double sh[kOffShared];
+  __shared__ double wtot[kSampleNT / 32];
   pdl_trigger();
   pdl_wait();
-  const bool in_shared = nblocks <= kOffShared;
-  if (in_shared) {
-    for (int i = threadIdx.x; i < nblocks; i += blockDim.x) sh[i] = tot[i];
+  const double* off = tot;
+  double A;
+  if (nblocks <= kOffShared) {
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    for (int i = tid; i < nblocks; i += kSampleNT) sh[i] = tot[i];
     __syncthreads();
+    const int per = (nblocks + kSampleNT - 1) / kSampleNT;
+    const int b0 = std::min(tid * per, nblocks), b1 = std::min(b0 + per, nblocks);
+    double run = 0.0;
+    for (int b = b0; b < b1; ++b) run += sh[b];
+    double incl = run;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const double v = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= d) incl += v;
+    }
+    if (lane == 31) wtot[w] = incl;
+    double acc = __shfl_up_sync(0xffffffffu, incl, 1);
+    if (lane == 0) acc = 0.0;
+    __syncthreads();
+    A = 0.0;
+    for (int k = 0; k < kSampleNT / 32; ++k) {
+      if (k == w) acc += A;
+      A += wtot[k];
+    }
+    for (int b = b0; b < b1; ++b) {
+      const double v = sh[b];
+      sh[b] = acc;
+      acc += v;
+    }
+    __syncthreads();
+    off = sh;
+  } else {
+    A = tot[nblocks];
   }
-  const double* off = in_shared ? sh : tot;
-  const double A = tot[nblocks];
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < M; s += (int64_t)gridDim.x * blockDim.x) {
     const double x = u01(seed, 3 * s) * A;
     int b = 0, e = nblocks;  // off[b] <= x (off[0] = 0), off[e] > x or e the end
@@ -348,9 +382,18 @@ __global__ void __launch_bounds__(kSampleNT) k_sample(const float* __restrict__ 
     const double base = off[b];
     int64_t lo = (int64_t)b * kScanBlock, hi = std::min<int64_t>(lo + kScanBlock, T) - 1;
     while (lo < hi) {
-      const int64_t mid = (lo + hi) >> 1;
-      if (cum[mid] + base > x) hi = mid;
-      else lo = mid + 1;
+      const int len = (int)(hi - lo);
+      const int64_t m1 = lo + len / 4, m2 = lo + len / 2, m3 = lo + 3 * len / 4;  // lo <= m1 <= m2 <= m3 < hi
+      const double c1 = cum[m1], c2 = cum[m2], c3 = cum[m3];
+      if (c2 + base > x) {
+        hi = m2;
+        if (c1 + base > x) hi = m1;
+        else lo = m1 + 1;
+      } else {
+        lo = m2 + 1;
+        if (c3 + base > x) hi = m3;
+        else lo = m3 + 1;
+      }
     }
     double u = u01(seed, 3 * s + 1), v = u01(seed, 3 * s + 2);
     if (u + v > 1.0) {
@@ -415,10 +458,11 @@ int dpsr_mesh_sample(const float* tris, const float* normals, int64_t T, int64_t
   double* cum = ws;
   double* tot = ws + T;  // nblk + 1 entries
   cudaError_t e = dpsr::launch_k(dpsr::k_area_scan, dim3(nblk), dim3(dpsr::kScanNT), 0, st, 0, tris, T, cum, tot);
-  if (e == cudaSuccess) e = dpsr::launch_k(dpsr::k_block_offsets, dim3(1), dim3(dpsr::kScanNT), 0, st, 0, tot, nblk);
+  if (e == cudaSuccess && nblk > dpsr::kOffShared)
+    e = dpsr::launch_k(dpsr::k_block_offsets, dim3(1), dim3(dpsr::kScanNT), 0, st, 0, tot, nblk);
   const unsigned sb = (unsigned)std::min<int64_t>((M + dpsr::kSampleNT - 1) / dpsr::kSampleNT, 4736);
   if (e == cudaSuccess)
-    e = dpsr::launch_k(dpsr::k_sample, dim3(sb), dim3(dpsr::kSampleNT), 0, st, 0, tris, normals, T, (const double*)cum,
+    e = dpsr::launch_after(dpsr::k_sample, dim3(sb), dim3(dpsr::kSampleNT), 0, st, 0, tris, normals, T, (const double*)cum,
                        (const double*)tot, nblk, M, seed, points, pnormals);
   if (e != cudaSuccess) cudaGetLastError();
   return e == cudaSuccess ? DPSR_OK : DPSR_ECUDA;
