@@ -21,8 +21,10 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <complex>
 #include <mutex>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include <cudaTypedefs.h>
@@ -127,7 +129,7 @@ size_t pts_ws_bytes(int64_t n) {
 
 // Cluster size of a plane kernel: the smallest whose CTAs fit two per SM
 // (<= 113 KB of shared memory), else the smallest that fits at all, else 0:
-// the pencil passes (r = 512, where no cluster kernel is built).
+// the pencil passes (from r = 256 on, where no cluster kernel is built).
 int pick_cluster(int kind, int r) {
   const int cands[4] = {1, 2, 4, 8};
   for (int C : cands) {
@@ -161,7 +163,8 @@ int cuda_err(cudaError_t e) { return e == cudaErrorMemoryAllocation ? DPSR_ENOME
 // picked by timing every candidate that fits on the first solve of a given r
 // in this process. The plane kernels are idempotent (they rewrite the same
 // outputs from the same inputs), so the candidates run in place, one after
-// the other; the last run leaves the correct results. Results are cached per
+// the other; the last run leaves the correct results. From r = 256 on there is
+// one path, and nothing is timed. Results are cached per
 // (kernel, r) for the process, and with DPSR_TUNE_CACHE=<file> persisted
 // across processes (tune_cache.cu): a choice found there is used without
 // timing. DPSR_TUNE=0 in the environment switches the tuner off (the static
@@ -272,10 +275,10 @@ cudaError_t tune_plane(dpsr_plan p, int kind, const Solve& s, cudaStream_t st) {
 cudaError_t run_plane(dpsr_plan p, int kind, const Solve& s, cudaStream_t st) {
   const int forced = forced_path(kind, p->r);
   if (forced >= 0) {
-    p->C[kind] = forced;
+    p->C[kind] = p->r < 256 ? forced : 0;
     return dpsr::launch_plane(kind, p->r, forced, s, nullptr, 1, st);
   }
-  if (tuning_enabled() && p->r >= 64) {
+  if (tuning_enabled() && p->r >= 64 && p->r < 256) {  // from 256 on there is one path
     int tuned;
     {
       std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -387,7 +390,7 @@ int make_tensor_maps(Solve& s, int r) {
       if (rc != CUDA_SUCCESS) return DPSR_ECUDA;
     }
   }
-  if (r <= 256) {
+  if (r < 256) {
     const cuuint32_t boxw[3] = {16, (cuuint32_t)r, 1};
     for (int k = 0; k < kNSpec; ++k)
       if (enc(&s.tmw[k], CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, (void*)s.spec[k], dims, strides, boxw, es,
@@ -797,6 +800,46 @@ int dpsr_get_loss(dpsr_plan p, double* loss) {
   return DPSR_OK;
 }
 
+// W~ from the weight field as the passes keep it from r = 256 on: y-blocks out
+// of the points' reach are zero and not stored, column 0 packs DC + i Nyquist.
+static void finish_w(int r, const unsigned* occ, std::complex<float>* w) {
+  typedef std::complex<double> Cd;
+  const int h = r / 2, nyb = dpsr::nybins(r), yb = r / nyb;
+  std::vector<Cd> tw(r), a(r), b(r);
+  for (int k = 0; k < r; ++k) tw[k] = std::polar(1.0, -2.0 * M_PI * k / r);
+  auto fft = [&](std::vector<Cd>& v) {  // radix 2, in order
+    for (int i = 1, j = 0; i < r; ++i) {
+      int bit = r >> 1;
+      for (; j & bit; bit >>= 1) j ^= bit;
+      j ^= bit;
+      if (i < j) std::swap(v[i], v[j]);
+    }
+    for (int len = 2; len <= r; len <<= 1)
+      for (int i = 0; i < r; i += len)
+        for (int k = 0; k < len / 2; ++k) {
+          const Cd u = v[i + k], t = v[i + k + len / 2] * tw[k * (r / len)];
+          v[i + k] = u + t;
+          v[i + k + len / 2] = u - t;
+        }
+  };
+  for (int x = 0; x < r; ++x) {
+    std::complex<float>* plane = w + (size_t)x * r * (h + 1);
+    const unsigned rows = dpsr::reach_mask(occ[x] | occ[(x - 1) & (r - 1)], nyb);
+    for (int kz = 0; kz < h; ++kz) {
+      for (int y = 0; y < r; ++y)
+        a[y] = (rows >> (y / yb)) & 1u ? Cd(plane[(size_t)y * (h + 1) + kz]) : Cd(0.0);
+      if (kz == 0)
+        for (int y = 0; y < r; ++y) b[y] = a[y].imag(), a[y] = a[y].real();
+      fft(a);
+      if (kz == 0) fft(b);
+      for (int y = 0; y < r; ++y) {
+        plane[(size_t)y * (h + 1) + kz] = std::complex<float>(a[y]);
+        if (kz == 0) plane[(size_t)y * (h + 1) + h] = std::complex<float>(b[y]);
+      }
+    }
+  }
+}
+
 int dpsr_debug_read_spectrum(dpsr_plan p, int which, void* out_host) {
   if (!p || !out_host || which < 0 || which > 5) return DPSR_EINVAL;
   if (p->spectra != (which < 4 ? 1 : 2)) return DPSR_ESTATE;
@@ -805,12 +848,21 @@ int dpsr_debug_read_spectrum(dpsr_plan p, int which, void* out_host) {
   static const int buf[6] = {dpsr::kSpD, dpsr::kSpC, dpsr::kSpW, dpsr::kSpChi, dpsr::kSpD, dpsr::kSpChi};
   const int r = p->r;
   const size_t w = sizeof(float2) * (size_t)(r / 2 + 1);
+  const bool half = which == 2 && r >= 256;  // kHalfW: y is still to be transformed
   if (cudaMemcpy2D(out_host, w, p->s.spec[buf[which]], sizeof(float2) * (size_t)dpsr::kpitch(r), w,
                    (size_t)r * r, cudaMemcpyDeviceToHost) != cudaSuccess) {
     cudaGetLastError();
     return DPSR_ECUDA;
   }
-  if (which < 3 && r >= 64) {  // the splat's spectra are zero, and not stored, in x-chunks without points
+  if (half) {
+    std::vector<unsigned> occ(r);
+    if (cudaMemcpy(occ.data(), dpsr::occ_words(p->s.bins, r), sizeof(unsigned) * r, cudaMemcpyDeviceToHost) !=
+        cudaSuccess) {
+      cudaGetLastError();
+      return DPSR_ECUDA;
+    }
+    finish_w(r, occ.data(), (std::complex<float>*)out_host);
+  } else if (which < 3 && r >= 64) {  // the splat's spectra are zero, and not stored, in x-chunks without points
     unsigned chunks = 0;
     if (cudaMemcpy(&chunks, dpsr::occ_words(p->s.bins, r) + r, sizeof(unsigned), cudaMemcpyDeviceToHost) !=
         cudaSuccess) {

@@ -129,8 +129,8 @@ cudaError_t tune_kind(BatchClass& c, int kind, cudaStream_t st, cudaEvent_t e0, 
   const Solve dummy = {};
   const int n = (int)c.members.size();
   const int forced = dpsr_internal_forced(kind, c.r);
-  if (forced != -1) {
-    if (forced >= 0) c.C[kind] = forced;
+  if (forced != -1 || c.r >= 256) {  // from r = 256 on there is one path
+    if (forced >= 0 && c.r < 256) c.C[kind] = forced;
     c.tuned[kind] = true;
     return dpsr::launch_plane(kind, c.r, c.C[kind], dummy, c.dtab, n, st);
   }

@@ -358,7 +358,8 @@ struct Scalars {
 //   kSpD   forward D; backward FFT_zy(dchi), then Q1 = IFFT_x(F)
 //   kSpChi forward chi~ after the x-pass; backward Q2 = IFFT_x(-i u_x F)
 //   kSpC   forward C; adjoint (pencil) V_bar_x
-//   kSpW   W~, kept from the forward for every backward
+//   kSpW   W~ (from r = 256 on W(x, y, kz), see kHalfW), kept from the forward
+//          for every backward
 //   kSpYa  pencil: y-domain chi~; adjoint V_bar_y
 //   kSpYb  pencil: adjoint V_bar_z
 // The pencil forward holds v_y, i u_z v_z, v_x, w (y-domain) in buffers
@@ -500,6 +501,20 @@ constexpr int kXChunks = 8;
 // 234). A cloud that fills the domain pays a mask read per block for it.
 template <int L>
 constexpr bool kSkip = L >= 64;
+// From r = 256 on, where the passes move more than the L2 holds, the weight
+// field stays as the z pass leaves it, W(x, y, kz) with DC and Nyquist packed
+// in column 0: its inner product with chi~ is taken in the inverse y pass and
+// its share of the adjoint spectrum added in the backward y pass (both
+// Parseval along y), where only the y-blocks with points are read. The forward
+// y pass then transforms three columns instead of four and stores two, and the
+// x passes do not read W~. r = 256: forward y pass 61.4 -> 46.7 us, x passes 62.7
+// -> 52.4 and 61.6 -> 49.0, for inverse y 31.2 -> 39.5 and backward y 21.6 -> 31.0;
+// r = 512: 526 -> 400, 551 -> 487 and 613 -> 567, for 191 -> 256 and 170 -> 211. (W
+// straight from global memory instead of a second tile: 40.4 and 30.7, 270 and 228.)
+// Below, the cluster kernels finish a plane on chip and need the sums before.
+template <int L>
+constexpr bool kHalfW = L >= 256;
+constexpr int kMuSlots = 8;  // accumulators of that product, double2 (mu, chi'(0)) at the start of Solve::part
 
 __host__ __device__ __forceinline__ const unsigned* occ_words(const int* bins, int r) {
   return reinterpret_cast<const unsigned*>(bins + 3 * (size_t)nbins(r) + 1);
@@ -527,7 +542,7 @@ __device__ __forceinline__ unsigned tile_mask(const Solve& S, int r, int X) {
 }
 // y-blocks whose rows those stencils reach: a stencil's second row may be the
 // first of the next block.
-__device__ __forceinline__ unsigned reach_mask(unsigned m, int nyb) {
+__host__ __device__ __forceinline__ unsigned reach_mask(unsigned m, int nyb) {
   if (nyb == 1) return m;
   const unsigned full = nyb >= 32 ? 0xffffffffu : (1u << nyb) - 1u;
   return (m | (m << 1) | (m >> (nyb - 1))) & full;

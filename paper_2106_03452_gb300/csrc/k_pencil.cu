@@ -1,5 +1,5 @@
 // Pencil kernels: the (y, z) transforms of a plane split into a z pass over
-// blocks of YB y-rows and a y pass over chunks of 16 kz columns, with the
+// blocks of YB y-rows and a y pass over chunks of 16 (8) kz columns, with the
 // intermediate spectra in the spectral buffers (L2-resident up to r = 128).
 // Each CTA is independent (no cluster, no DSMEM), so thousands of small CTAs
 // keep every SM busy; the plane kernels of k_plane.cu instead keep a plane in
@@ -9,11 +9,14 @@
 //   forward   k_zfwd  splat (Eq. A2) of v_y, v_z, v_x, w into YB rows, R2C
 //                     along z (v_z times i u_z)   -> buffers 0..3 (y, kz)
 //             k_yfwd  FFT along y: D = FFT(i u_z v_z) + i u_y FFT(v_y) -> kSpD,
-//                     C -> kSpC, W~ -> kSpW         (ky, kz)
-//   inverse   k_yinv  IFFT along y of chi~ (kSpChi) -> kSpYa (y, kz)
+//                     C -> kSpC, W~ -> kSpW         (ky, kz); from r = 256
+//                     on W stays as it is (kHalfW)
+//   inverse   k_yinv  IFFT along y of chi~ (kSpChi) -> kSpYa (y, kz), with
+//                     kHalfW the sums of Eq. 4 against W
 //             k_zinv<1> C2R along z, chi = a y + b (Eq. 4), lookup gradient
 //   backward  k_zbfwd sums of Eq. 4's adjoint, R2C along z of dchi -> kSpD
-//             k_yfwd  FFT along y of kSpD in place
+//             k_yfwd  FFT along y of kSpD in place, with kHalfW of the whole
+//                     adjoint source
 //   adjoint   k_yinv  IFFT along y of Q2, -i u_y Q1, -i u_z Q1 -> kSpC, kSpYa,
 //                     kSpYb
 //             k_zinv<3> C2R along z of the three fields, adjoint of the splat
@@ -325,29 +328,27 @@ __global__ void __launch_bounds__(ZfGeo<L>::NT, ZfGeo<L>::MINB) k_zfwd(const __g
 // ===========================================================================
 // Forward y pass over 16 kz columns of plane X, by CTA kind (blockIdx.y):
 // 0: D = FFT(i u_z v_z) + i u_y FFT(v_y) from buffers 0 and 1 into kSpD;
-// 1: C = FFT(v_x) in place in kSpC, and from r = 256 on (yfwd_merge) also
-// W~ = FFT(w) in place in kSpW; 2 (below r = 256): W~. BWD: FFT of the
-// z-transformed dchi in place in kSpD. Merging C and W~ halves the CTAs of
-// the bandwidth-bound r = 256 pass; below, where the pass is bound by the
-// latency of each CTA, more and shorter CTAs win.
+// 1: C = FFT(v_x) in place in kSpC; 2 (not with kHalfW): W~ = FFT(w) in place
+// in kSpW. BWD: FFT of the z-transformed dchi in place in kSpD, with kHalfW of
+// g_a dchi + g_w W + g_s delta, the y and z transform of the whole adjoint source.
 // ===========================================================================
 template <int L>
 constexpr int ynt() {
   return Pen<L>::W * Shape<L>::T >= 32 ? Pen<L>::W * Shape<L>::T : 32;  // one group per column
 }
 
-template <int L>
-constexpr bool yfwd_merge() {
-  return L >= 256;
+template <int L, bool BWD>
+constexpr int yfwd_boxes() {
+  return BWD && !kHalfW<L> ? 1 : 2;
 }
 
 template <int L, bool BWD>
 constexpr size_t yfwd_smem() {
-  return box_align<L>() + sizeof(float2) * ((size_t)(BWD ? 1 : 2) * Pen<L>::BOX + L) + sizeof(float) * L;
+  return box_align<L>() + sizeof(float2) * ((size_t)yfwd_boxes<L, BWD>() * Pen<L>::BOX + L) + sizeof(float) * L;
 }
 
 // Input buffers of a y-pass tile of kind `kind` (see k_yfwd): box 0 holds
-// buf0 (input and output), box 1 (kinds 0 and merged 1) buf1.
+// buf0 (input and output), box 1 (kind 0, and the backward with kHalfW) buf1.
 struct YfwdBufs {
   int buf0, buf1;
   bool two;
@@ -356,8 +357,8 @@ template <int L, bool BWD>
 __device__ __forceinline__ YfwdBufs yfwd_bufs(int kind) {
   YfwdBufs b;
   b.buf0 = kind == 1 ? kSpC : (kind == 2 ? kSpW : kSpD);
-  b.buf1 = kind == 1 ? kSpW : 1;
-  b.two = !BWD && (kind == 0 || (kind == 1 && yfwd_merge<L>()));
+  b.buf1 = BWD ? kSpW : 1;
+  b.two = BWD ? kHalfW<L> : kind == 0;
   return b;
 }
 
@@ -378,17 +379,34 @@ __device__ __forceinline__ void yfwd_issue_rows(const Solve& S, int X, int kz0, 
   }
 }
 
-// Thread 0: the TMA tile loads of a y-pass tile, completion on `bar`.
+// Thread 0: the TMA tile loads of a whole y-pass tile, completion on `bar`,
+// which also awaits `more` bytes.
 template <int L, bool BWD>
 __device__ __forceinline__ void yfwd_issue(const Solve& S, int X, int kz0, int kind, float2* box,
-                                           uint64_t* bar) {
+                                           uint64_t* bar, uint32_t more = 0u) {
   using P = Pen<L>;
   const YfwdBufs b = yfwd_bufs<L, BWD>(kind);
-  mbar_expect_tx(bar, (b.two ? 2 : 1) * P::BOX * (uint32_t)sizeof(float2));
+  const bool two = !BWD && b.two;
+  mbar_expect_tx(bar, (two ? 2 : 1) * P::BOX * (uint32_t)sizeof(float2) + more);
   for (int y = 0; y < L; y += tma_rows(L)) {
     tma_load_3d(box + y * P::W, &S.tmy[b.buf0], kz0, y, X, bar);
-    if (b.two) tma_load_3d(box + P::BOX + y * P::W, &S.tmy[b.buf1], kz0, y, X, bar);
+    if (two) tma_load_3d(box + P::BOX + y * P::W, &S.tmy[b.buf1], kz0, y, X, bar);
   }
+}
+
+// W's y-blocks `rows` of a tile (kHalfW): their bytes, and their loads by the
+// lanes of warp 0 once thread 0 has announced them.
+template <int L>
+__device__ __forceinline__ uint32_t w_bytes(unsigned rows) {
+  return __popc(rows) * Pen<L>::W * Pen<L>::YB * (uint32_t)sizeof(float2);
+}
+template <int L>
+__device__ __forceinline__ void w_issue(const Solve& S, int X, int kz0, unsigned rows, float2* box, uint64_t* bar) {
+  using P = Pen<L>;
+  const int lane = threadIdx.x;
+  __syncwarp();
+  if (lane < P::NYB && ((rows >> lane) & 1u))
+    tma_load_3d(box + lane * P::YB * P::W, &S.tmb[kSpW], kz0, lane * P::YB, X, bar);
 }
 
 // All threads: wait for the tile (phase `phase` of `bar`), transform, store
@@ -401,11 +419,17 @@ __device__ __forceinline__ bool yfwd_tile(const Solve& S, int X, int kz0, int ki
   using P = Pen<L>;
   constexpr int H = P::H;
   const YfwdBufs bb = yfwd_bufs<L, BWD>(kind);
-  const int buf0 = bb.buf0, buf1 = bb.buf1;
-  const bool two = bb.two;
+  const int buf0 = bb.buf0;
+  const bool two = !BWD && bb.two;
   constexpr bool IL = P::T == 16;  // interleaved groups: conflict-free column accesses
   using LN = Lanes<P::T, IL>;
   const int tid = threadIdx.x, g = LN::group(tid), t = LN::lane(tid);
+  float ga = 1.f, gs = 0.f, gw = 0.f;
+  if constexpr (BWD && kHalfW<L>) {
+    ga = S.sc->g_a;
+    gs = S.sc->g_s;
+    gw = S.sc->g_w;
+  }
   const bool landed = __syncthreads_and(mbar_wait(bar, phase));
   if (!landed) {
     if (tid == 0) atomicOr(S.status, kStTimeout);
@@ -420,6 +444,18 @@ __device__ __forceinline__ bool yfwd_tile(const Solve& S, int X, int kz0, int ki
     auto has = [rows](int j) { return BWD || !kSkip<L> || ((rows >> (P::T * j / P::YB)) & 1u); };
 #pragma unroll
     for (int j = 0; j < P::R1; ++j) a[j] = has(j) ? c0.get(j) : czero();
+    if constexpr (BWD && kHalfW<L>) {
+      const Col<L> c1(box + P::BOX, t, g);
+#pragma unroll
+      for (int j = 0; j < P::R1; ++j) {
+        a[j] = cscale(a[j], ga);
+        if ((rows >> (P::T * j / P::YB)) & 1u) a[j] = cadd(a[j], cscale(c1.get(j), gw));
+      }
+      if (X == 0 && t == 0) {  // the delta at the origin is 1 in every kz, DC and Nyquist in one column
+        a[0].x += gs;
+        if (kz0 + g == 0) a[0].y += gs;
+      }
+    }
     fft_c<L, -1, IL>(a, c0, twr);
 #pragma unroll
     for (int j = 0; j < P::R1; ++j) c0.put(j, a[j]);
@@ -428,26 +464,20 @@ __device__ __forceinline__ bool yfwd_tile(const Solve& S, int X, int kz0, int ki
 #pragma unroll
       for (int j = 0; j < P::R1; ++j) a[j] = has(j) ? c1.get(j) : czero();
       fft_c<L, -1, IL>(a, c1, twr);
-      if (kind == 0) {  // D = FFT(i u_z v_z) + i u_y FFT(v_y); this lane wrote c0 above
+      // D = FFT(i u_z v_z) + i u_y FFT(v_y); this lane wrote c0 above
 #pragma unroll
-        for (int j = 0; j < P::R1; ++j) {
-          const int ky = t + P::T * j;
-          c0.put(j, cadd(a[j], cmul_iu(c0.get(j), iu[ky])));
-        }
-      } else {
-#pragma unroll
-        for (int j = 0; j < P::R1; ++j) c1.put(j, a[j]);
+      for (int j = 0; j < P::R1; ++j) {
+        const int ky = t + P::T * j;
+        c0.put(j, cadd(a[j], cmul_iu(c0.get(j), iu[ky])));
       }
     }
   }
   __syncthreads();
-  const int nsplit = kind == 1 && two ? 2 : 1;  // tiles whose column 0 packs DC and Nyquist
-  if (kz0 == 0 && g < nsplit) {
+  if (kz0 == 0 && g == 0) {
     // column 0 holds X0 + i Xn of the DC and Nyquist columns: split them
-    float2* bq = box + g * P::BOX;
-    float2* dst = S.spec[g == 0 ? buf0 : buf1];
-    split_dc_nyq<L, IL>(bq, t, [&](int ky, float2 w) {
-      if (H < 16) bq[bxl<L>(ky, H)] = w;
+    float2* dst = S.spec[buf0];
+    split_dc_nyq<L, IL>(box, t, [&](int ky, float2 w) {
+      if (H < 16) box[bxl<L>(ky, H)] = w;
       else dst[((size_t)X * L + ky) * P::KP + H] = w;
     });
   }
@@ -456,7 +486,6 @@ __device__ __forceinline__ bool yfwd_tile(const Solve& S, int X, int kz0, int ki
   if (tid == 0) {
     for (int y = 0; y < L; y += tma_rows(L)) {
       tma_store_3d(&S.tmy[buf0], kz0, y, X, box + y * P::W);
-      if (kind == 1 && two) tma_store_3d(&S.tmy[buf1], kz0, y, X, box + P::BOX + y * P::W);
     }
     tma_store_commit();
     tma_store_wait_read();
@@ -465,7 +494,7 @@ __device__ __forceinline__ bool yfwd_tile(const Solve& S, int X, int kz0, int ki
 }
 
 template <int L, bool BWD>
-__global__ void __launch_bounds__(ynt<L>(), L == 256 ? (BWD ? 8 : 6) : (BWD ? 4 : (L >= 256 ? 3 : 5))) k_yfwd(const __grid_constant__ Solve s0,
+__global__ void __launch_bounds__(ynt<L>(), L == 256 ? 6 : (L >= 256 ? 3 : (BWD ? 4 : 5))) k_yfwd(const __grid_constant__ Solve s0,
                                                    const Solve* __restrict__ tab) {
   using P = Pen<L>;
   constexpr int NT = ynt<L>();
@@ -477,7 +506,7 @@ __global__ void __launch_bounds__(ynt<L>(), L == 256 ? (BWD ? 8 : 6) : (BWD ? 4 
   constexpr uint32_t AL = box_align<L>();
   const uint32_t pad = (AL - (smem_u32(smem_raw) & (AL - 1u))) & (AL - 1u);
   float2* box = reinterpret_cast<float2*>(smem_raw + pad);  // 1 or 2 boxes
-  float2* twt = box + (BWD ? 1 : 2) * P::BOX;
+  float2* twt = box + yfwd_boxes<L, BWD>() * P::BOX;
   float* iu = reinterpret_cast<float*>(twt + L);
   __shared__ uint64_t bar;
   pdl_trigger();
@@ -494,6 +523,10 @@ __global__ void __launch_bounds__(ynt<L>(), L == 256 ? (BWD ? 8 : 6) : (BWD ? 4 
     // empty (the x pass does not load it), else stored as zeros
     if (rows == 0u && !((chunk_mask(S, L) >> (X / (L / kXChunks))) & 1u)) return;
     if (tid < 32) yfwd_issue_rows<L>(S, X, kz0, kind, rows, box, &bar);
+  } else if constexpr (BWD && kHalfW<L>) {
+    rows = reach_mask(tile_mask(S, L, X), P::NYB);
+    if (tid == 0) yfwd_issue<L, BWD>(S, X, kz0, kind, box, &bar, w_bytes<L>(rows));
+    if (tid < 32) w_issue<L>(S, X, kz0, rows, box + P::BOX, &bar);
   } else if (tid == 0) {
     yfwd_issue<L, BWD>(S, X, kz0, kind, box, &bar);
   }
@@ -516,20 +549,25 @@ __global__ void __launch_bounds__(ynt<L>(), L == 256 ? (BWD ? 8 : 6) : (BWD ? 4 
 // r = 256, bound by bandwidth, one CTA does all three.
 // ===========================================================================
 template <int L, int NCH>
+constexpr int yinv_boxes() {
+  return NCH == 1 && kHalfW<L> ? 2 : NCH;
+}
+
+template <int L, int NCH>
 constexpr size_t yinv_smem() {
-  return box_align<L>() + sizeof(float2) * ((size_t)NCH * Pen<L>::BOX + L) + sizeof(float) * L;
+  return box_align<L>() + sizeof(float2) * ((size_t)yinv_boxes<L, NCH>() * Pen<L>::BOX + L) + sizeof(float) * L;
 }
 
 // Thread 0: the TMA tile loads of an inverse y-pass tile (part: -1 all
 // fields, else the CTA kind of yinv_split), completion on `bar`.
 template <int L, int NCH>
 __device__ __forceinline__ void yinv_issue(const Solve& S, int X, int kz0, int part, float2* box,
-                                           uint64_t* bar) {
+                                           uint64_t* bar, uint32_t more = 0u) {
   using P = Pen<L>;
   // NCH = 1: box 0 <- chi~; NCH = 3: box 0 <- Q2, box 1 <- Q1 (split: only
   // the kind's own input)
   const bool do0 = part != 1, do1 = NCH == 3 && part != 0;
-  mbar_expect_tx(bar, ((do0 ? 1 : 0) + (do1 ? 1 : 0)) * P::BOX * (uint32_t)sizeof(float2));
+  mbar_expect_tx(bar, ((do0 ? 1 : 0) + (do1 ? 1 : 0)) * P::BOX * (uint32_t)sizeof(float2) + more);
   for (int y = 0; y < L; y += tma_rows(L)) {
     if (do0) tma_load_3d(box + y * P::W, &S.tmy[kSpChi], kz0, y, X, bar);
     if (do1) tma_load_3d(box + P::BOX + y * P::W, &S.tmy[kSpD], kz0, y, X, bar);
@@ -541,12 +579,13 @@ __device__ __forceinline__ void yinv_issue(const Solve& S, int X, int kz0, int p
 template <int L, int NCH>
 __device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int part, float2* box,
                                           const float2* twt, const float* iu, uint64_t* bar,
-                                          uint32_t phase) {
+                                          uint32_t phase, unsigned rows = 0u) {
   using P = Pen<L>;
   constexpr int H = P::H;
   constexpr bool IL = P::T == 16;  // interleaved groups: conflict-free column accesses
   using LN = Lanes<P::T, IL>;
   const int tid = threadIdx.x, g = LN::group(tid), t = LN::lane(tid);
+  float am = 0.f, as = 0.f;  // this thread's share of the sums of Eq. 4 (kHalfW)
   constexpr int NIN = NCH == 1 ? 1 : 2;
   const bool do0 = part != 1, do1 = NCH == 3 && part != 0;
   const bool landed = __syncthreads_and(mbar_wait(bar, phase));
@@ -580,6 +619,22 @@ __device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int pa
       fft_c<L, +1, IL>(v, c0, twr);
 #pragma unroll
       for (int j = 0; j < P::R1; ++j) c0.put(j, v[j]);
+      if constexpr (NCH == 1 && kHalfW<L>) {
+        // sum_ky conj(W~) chi~ = sum_y conj(W) P by Parseval along y; the half
+        // spectrum counts twice but for column 0, where DC and Nyquist are
+        // packed on both sides: Re(conj(W) P) is the sum of the two products
+        const Col<L> cw(box + P::BOX, t, g);
+        const float wz = sz == 0 ? 1.f : 2.f;  // exact
+#pragma unroll
+        for (int j = 0; j < P::R1; ++j) {
+          if ((rows >> (P::T * j / P::YB)) & 1u) {
+            const float2 w = cw.get(j);
+            am += w.x * v[j].x + w.y * v[j].y;
+          }
+        }
+        am *= wz;
+        if (X == 0 && t == 0) as = sz == 0 ? v[0].x + v[0].y : 2.f * v[0].x;  // chi'(0) = sum over kz at x = y = 0
+      }
     }
     if (do1) {
       const auto c1 = cref(1);
@@ -604,6 +659,23 @@ __device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int pa
   }
   fence_async_smem();
   __syncthreads();
+  if constexpr (NCH == 1 && kHalfW<L>) {
+    if (tid == 0) {
+      for (int y = 0; y < L; y += tma_rows(L)) tma_store_3d(&S.tmy[kSpYa], kz0, y, X, box + y * P::W);
+      tma_store_commit();
+    }
+    if (rows != 0u || X == 0) {  // the same for the whole block
+      FF fm = {am, 0.f}, fs = {as, 0.f};
+      block_sum_ff<ynt<L>()>(fm, fs);
+      if (tid == 0) {  // a few addresses, nothing waits for the additions
+        double2* slot = reinterpret_cast<double2*>(S.part) + blockIdx.x % kMuSlots;
+        atomicAdd(&slot->x, ff_to_double(fm));
+        if (X == 0) atomicAdd(&slot->y, ff_to_double(fs));
+      }
+    }
+    if (tid == 0) tma_store_wait_read();
+    return true;
+  }
   if (tid == 0) {
     for (int y = 0; y < L; y += tma_rows(L)) {
       if constexpr (NCH == 1) {
@@ -623,7 +695,7 @@ __device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int pa
 }
 
 template <int L, int NCH>
-__global__ void __launch_bounds__(ynt<L>(), L == 256 ? 8 : 4)
+__global__ void __launch_bounds__(ynt<L>(), L == 256 ? 6 : (L >= 512 ? 3 : 4))
     k_yinv(const __grid_constant__ Solve s0, const Solve* __restrict__ tab) {
   using P = Pen<L>;
   constexpr int NT = ynt<L>();
@@ -634,7 +706,7 @@ __global__ void __launch_bounds__(ynt<L>(), L == 256 ? 8 : 4)
   constexpr uint32_t AL = box_align<L>();
   const uint32_t pad = (AL - (smem_u32(smem_raw) & (AL - 1u))) & (AL - 1u);
   float2* box = reinterpret_cast<float2*>(smem_raw + pad);
-  float2* twt = box + NCH * P::BOX;
+  float2* twt = box + yinv_boxes<L, NCH>() * P::BOX;
   float* iu = reinterpret_cast<float*>(twt + L);
   __shared__ uint64_t bar;
   pdl_trigger();
@@ -644,20 +716,27 @@ __global__ void __launch_bounds__(ynt<L>(), L == 256 ? 8 : 4)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   pdl_wait();
-  if (NCH == 1 && blockIdx.x == L * P::NKC) {  // one more CTA: the scalars of Eq. 4, read by the z pass
+  if (NCH == 1 && !kHalfW<L> && blockIdx.x == L * P::NKC) {  // one more CTA: the scalars of Eq. 4, read by the z pass
     FF x, y;
     sum_partials<NT>(S, x_tiles(L), x, y);
     if (tid == 0) finalize_scalars(S, ff_to_double(x), ff_to_double(y), false);
     return;
   }
   const int part = NCH == 3 ? (int)blockIdx.y : -1;
-  if (tid == 0) yinv_issue<L, NCH>(S, X, kz0, part, box, &bar);
+  unsigned rows = 0u;
+  if constexpr (NCH == 1 && kHalfW<L>) {
+    rows = reach_mask(tile_mask(S, L, X), P::NYB);
+    if (tid == 0) yinv_issue<L, NCH>(S, X, kz0, part, box, &bar, w_bytes<L>(rows));
+    if (tid < 32) w_issue<L>(S, X, kz0, rows, box + P::BOX, &bar);
+  } else if (tid == 0) {
+    yinv_issue<L, NCH>(S, X, kz0, part, box, &bar);
+  }
   for (int i = tid; i < L; i += NT) {
     twt[i] = S.tw[i];
     iu[i] = S.iu[L + i];  // y axis
   }
   __syncthreads();
-  yinv_tile<L, NCH>(S, X, kz0, part, box, twt, iu, &bar, 0);
+  yinv_tile<L, NCH>(S, X, kz0, part, box, twt, iu, &bar, 0, rows);
 }
 
 // ===========================================================================
@@ -998,20 +1077,43 @@ __global__ void __launch_bounds__(ZiGeo<L, NCH>::NT, L >= 512 ? (NCH == 1 ? 2 : 
   pdl_wait();
   int ntiles = L * P::NYB;
   if constexpr (LIST) ntiles = list.build(S);
+  // the scalars of Eq. 4 from the y pass's sums, in every CTA while its first tile loads
+  constexpr bool MU = NCH == 1 && kHalfW<L>;
+  __shared__ float2 ab;
+  if constexpr (MU) {
+    if (tid == 0 && (int)blockIdx.x < ntiles) zinv_issue<L, NCH>(S, blockIdx.x, stg, &bar[0]);
+    if (tid == 32) {
+      const double2* slots = reinterpret_cast<const double2*>(S.part);
+      double2 v[kMuSlots];
+#pragma unroll
+      for (int q = 0; q < kMuSlots; ++q) v[q] = __ldcg(slots + q);
+#pragma unroll
+      for (int q = 1; q < kMuSlots; ++q) {
+        v[0].x += v[q].x;
+        v[0].y += v[q].y;
+      }
+      const FwdScalars f = fwd_scalars(S, v[0].x, v[0].y);
+      ab = make_float2(f.a_chi, f.b_chi);
+      if (blockIdx.x == 0) finalize_scalars(S, v[0].x, v[0].y, false);
+    }
+  }
   __syncthreads();
   auto at = [&](int k) {  // the k-th tile to do
     if constexpr (LIST) return list.tile(k);
     else return k;
   };
   float a_chi = 0.f, b_chi = 0.f;
-  if constexpr (NCH == 1) {
+  if constexpr (MU) {
+    a_chi = ab.x;
+    b_chi = ab.y;
+  } else if constexpr (NCH == 1) {
     a_chi = S.sc->a_chi;
     b_chi = S.sc->b_chi;
   }
   uint32_t ph = 0u;  // bit st: parity of stage st's next completion
   int k = blockIdx.x;
   int tile = k < ntiles ? at(k) : 0;
-  if (tid == 0 && k < ntiles) zinv_issue<L, NCH>(S, tile, stg, &bar[0]);
+  if (!MU && tid == 0 && k < ntiles) zinv_issue<L, NCH>(S, tile, stg, &bar[0]);
   for (int it = 0; k < ntiles; ++it, k += gridDim.x) {
     const int st = it & 1;
     const int next = k + gridDim.x;
@@ -1162,7 +1264,7 @@ static cudaError_t launch_pencil_t(int kind, const Solve& s, const Solve* tab, i
       }
       e = launch_k(k_zfwd<L>, dim3(4 / ZfGeo<L>::NCC * L * P::NYB, 1, count), dim3(ZfGeo<L>::NT), a, st, 0, s, tab);
       if (e == cudaSuccess)
-        e = launch_k(k_yfwd<L, false>, dim3(L * P::NKC, yfwd_merge<L>() ? 2 : 3, count), dim3(ynt<L>()),
+        e = launch_k(k_yfwd<L, false>, dim3(L * P::NKC, kHalfW<L> ? 2 : 3, count), dim3(ynt<L>()),
                      b, st, 0, s, tab);
       return e;
     }
@@ -1177,7 +1279,7 @@ static cudaError_t launch_pencil_t(int kind, const Solve& s, const Solve* tab, i
         nz = persistent_ctas(k_zinv<L, 1>, ZiGeo<L, 1>::NT, b, L * P::NYB, 1);
         attr_set[1] = true;
       }
-      e = launch_k(k_yinv<L, 1>, dim3(L * P::NKC + 1, 1, count), dim3(nt), a, st, 0, s, tab);
+      e = launch_k(k_yinv<L, 1>, dim3(L * P::NKC + (kHalfW<L> ? 0 : 1), 1, count), dim3(nt), a, st, 0, s, tab);
       if (e == cudaSuccess)
         // from r = 256 on after the y pass: 39 -> 33 us at r = 256, 232 -> 228 at r = 512; below, the gap costs more
         e = launch_at(L < 256, k_zinv<L, 1>, dim3(nz, 1, count), dim3(ZiGeo<L, 1>::NT), b, st, 0, s, tab);

@@ -42,17 +42,16 @@ struct PlaneGeo {
 };
 
 // Cluster sizes instantiated per grid size: one CTA per plane up to r = 64,
-// 1/2/4 CTAs at r = 128, 2/4/8 CTAs at r = 256 (r^2 complex values of one
-// plane do not fit one SM's shared memory there).
+// 1/2/4 CTAs at r = 128, none above.
 template <int L, int C>
 constexpr bool plane_inst() {
   // every CTA must own at least 16 slots (one TMA box of kz) so that box
   // stores never cover a neighbour's slots
-  return L <= 64 ? C == 1 : (L == 128 ? (C == 1 || C == 2 || C == 4) : (C == 2 || C == 4 || C == 8));
+  return L <= 64 ? C == 1 : (C == 1 || C == 2 || C == 4);
 }
 
 // The forward plane kernel transforms all slots of a CTA in one y pass, which
-// needs at least as many groups as slots (r = 256: C >= 4).
+// needs at least as many groups as slots (it has them at every size here).
 template <int L, int C>
 constexpr bool fwd_inst() {
   return plane_inst<L, C>() && (512 / Shape<L>::T) >= (L / 2) / C;
@@ -1159,7 +1158,6 @@ static cudaError_t launch_plane_L(int kind, int C, const Solve& s, const Solve* 
     case 1: if constexpr (plane_inst<L, 1>()) return launch_plane_t<L, 1>(kind, s, tab, count, st); break;
     case 2: if constexpr (plane_inst<L, 2>()) return launch_plane_t<L, 2>(kind, s, tab, count, st); break;
     case 4: if constexpr (plane_inst<L, 4>()) return launch_plane_t<L, 4>(kind, s, tab, count, st); break;
-    case 8: if constexpr (plane_inst<L, 8>()) return launch_plane_t<L, 8>(kind, s, tab, count, st); break;
     default: break;
   }
   return cudaErrorInvalidValue;
@@ -1167,7 +1165,10 @@ static cudaError_t launch_plane_L(int kind, int C, const Solve& s, const Solve* 
 
 cudaError_t launch_plane(int kind, int r, int C, const Solve& s, const Solve* tab, int count,
                          cudaStream_t st) {
-  if (C == 0) return launch_pencil(kind, r, s, tab, count, st);
+  // A plane of r = 256 would take 2 to 8 CTAs: timed against the pencil passes
+  // such clusters lost in every kind, and they need W~ whole (see kHalfW). The
+  // sizes stay accepted and run the pencil passes.
+  if (C == 0 || (r == 256 && (C == 2 || C == 4 || C == 8))) return launch_pencil(kind, r, s, tab, count, st);
   if (C == kPathSplit) {
     if (kind != 3) return cudaErrorInvalidValue;
     if (r == 64) return launch_binv_ch_t<64>(s, tab, count, st);
@@ -1180,7 +1181,6 @@ cudaError_t launch_plane(int kind, int r, int C, const Solve& s, const Solve* ta
     case 32: return launch_plane_L<32>(kind, C, s, tab, count, st);
     case 64: return launch_plane_L<64>(kind, C, s, tab, count, st);
     case 128: return launch_plane_L<128>(kind, C, s, tab, count, st);
-    case 256: return launch_plane_L<256>(kind, C, s, tab, count, st);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -1216,7 +1216,6 @@ size_t plane_smem_bytes(int kind, int r, int C) {
       case 1: return kind_smem<L, 1>(kind);
       case 2: return kind_smem<L, 2>(kind);
       case 4: return kind_smem<L, 4>(kind);
-      case 8: return kind_smem<L, 8>(kind);
       default: return 0;
     }
   };
@@ -1226,7 +1225,6 @@ size_t plane_smem_bytes(int kind, int r, int C) {
     case 32: return pick(std::integral_constant<int, 32>{});
     case 64: return pick(std::integral_constant<int, 64>{});
     case 128: return pick(std::integral_constant<int, 128>{});
-    case 256: return pick(std::integral_constant<int, 256>{});
     default: return 0;
   }
 }

@@ -1,13 +1,14 @@
 // x-axis pass: FFT along x of the partially transformed fields, the spectral
 // solve of Eq. 3 (forward) or its adjoint (backward), and the inverse FFT
-// along x, for a tile of 16 consecutive kz columns at one ky, moved between
+// along x, for a tile of 16 (8) consecutive kz columns at one ky, moved between
 // HBM and shared memory by TMA.
 //
 // Forward:  chi~ = G(k) (D + i u_x C),  G = g(u) / (-2 pi |u|^2),
 //           g = exp(-2 sigma^2 |u|^2 / r^2)                        (Eq. 3, A7)
 //           with the spectral sums for the mean and the value at x = 0 of
-//           Eq. 4 (Parseval over the half spectrum, and along x).
-// Backward: F = G(k) (g_a FFT(dchi) + g_s + g_w W~);  Q1 = IFFT_x(F),
+//           Eq. 4 (Parseval over the half spectrum, and along x) up to r = 128.
+// Backward: F = G(k) (g_a FFT(dchi) + g_s + g_w W~), the bracket formed here up
+//           to r = 128 and by the y pass above (kHalfW);  Q1 = IFFT_x(F),
 //           Q2 = IFFT_x(-i u_x F)  (the adjoint of Eq. 3, conj(H_a) = -H_a).
 // Three FFTs of length r per column in each direction.
 #include "col.cuh"
@@ -28,12 +29,11 @@ struct XGeo {
   static constexpr int NCHUNK = x_tiles(L) / L;
   static constexpr int BOX = L * KC;                        // float2 per box
   static constexpr int KP = kpitch(L);                      // row pitch of the spectral buffers
-  // Two tiles per CTA in both directions. The forward needs W~ only for its
-  // spectral sums, after the transforms of C: up to r = 128 it reads W~'s
-  // column straight from L2 (the spectra stay resident there); at r = 256 a
-  // TMA load brings W~'s tile into C's box once every group is done with C,
-  // overlapping the inverse transform.
-  static constexpr bool WL2 = L <= 128;
+  // Two tiles per CTA in both directions. Up to r = 128 the forward needs W~
+  // for its spectral sums, after the transforms of C: it reads W~'s column
+  // straight from L2 (the spectra stay resident there), and the backward reads
+  // W~'s tile. From r = 256 on W~ has no part in the x passes (kHalfW).
+  static constexpr bool HW = kHalfW<L>;
   template <bool BWD>
   static constexpr int nch() { return 2; }
 };
@@ -54,7 +54,7 @@ constexpr size_t xpass_smem() {
   return box_align<L>() + sizeof(float2) * ((size_t)NCH * P::BOX + L) + 3 * sizeof(float) * L;
 }
 
-// One CTA per (kz tile of 16, ky): TMA loads the tiles [x][16 kz] of the
+// One CTA per (kz tile, ky): TMA loads the tiles [x][16 or 8 kz] of the
 // input channels (128B-swizzled boxes), each group of T threads transforms
 // one kz column along x in registers (the box column doubles as its exchange
 // buffer), and TMA stores the results.
@@ -76,17 +76,22 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
   float* g1 = reinterpret_cast<float*>(tw + L);
   float* u2 = g1 + L;
   float* iu = u2 + L;
-  // One barrier per box: the forward transforms D while C and W~ still land.
+  // One barrier per box: the forward transforms D while C still lands.
   __shared__ uint64_t bar[NCH];
-  // inputs: forward D, C, W~; backward FFT_zy(dchi), W~
+  // inputs: forward D, C; backward FFT_zy(dchi) and, without kHalfW, W~
   const int src0 = kSpD, src1 = BWD ? kSpW : kSpC;
   pdl_trigger();
   pdl_wait();
   // the binning of this forward pass is done: its counters start the next one at zero
   if constexpr (!BWD) clear_bin_counters(S, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
+  if constexpr (!BWD && P::HW) {
+    if (blockIdx.x == 0 && blockIdx.y == 0 && tid < kMuSlots)
+      reinterpret_cast<double2*>(S.part)[tid] = make_double2(0.0, 0.0);
+  }
   // From r = 64 on the splat's spectra (D, C, W~) are only loaded for the
   // x-chunks that points touch, a lane of warp 0 per chunk; the rest is zero.
-  const unsigned chunks = kSkip<L> ? chunk_mask(S, L) : 0xffu;
+  constexpr bool TWO = !(BWD && P::HW);  // two input tiles
+  const unsigned chunks = kSkip<L> && TWO ? chunk_mask(S, L) : 0xffu;
   constexpr int XC = L / kXChunks;
   auto has = [chunks](int j) { return !kSkip<L> || ((chunks >> (P::T * j / XC)) & 1u); };  // x = t + T j, t < T
   auto load_chunks = [&](int buf, int c) {  // warp 0
@@ -109,7 +114,7 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
     if constexpr (kSkip<L>) {
       if (!BWD) load_chunks(src0, 0);
       else if (tid == 0) load_all(src0, 0);
-      load_chunks(src1, 1);
+      if constexpr (TWO) load_chunks(src1, 1);
     } else if (tid == 0) {
       load_all(src0, 0);
       load_all(src1, 1);
@@ -129,21 +134,18 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
   auto box_wait = [&](int c, uint32_t phase = 0u) {
     if (ok) ok = mbar_wait(&bar[c], phase);
   };
-  bool w_reload = false;  // r = 256 forward: W~ went into box 1 (its second phase)
   auto leave = [&]() {  // after a failed vote
     if (tid == 0) {
       atomicOr(S.status, kStTimeout);
 #pragma unroll
-      for (int c = 0; c < NCH; ++c) mbar_wait(&bar[c], 0);  // copies in flight: a last bounded chance
-      if (w_reload) mbar_wait(&bar[1], 1);
+      for (int c = 0; c < (TWO ? 2 : 1); ++c) mbar_wait(&bar[c], 0);  // copies in flight: a last bounded chance
     }
   };
   const int gc = g < P::KC ? g : P::KC - 1;  // extra groups (tiny r) shadow the last column
   const bool own = g < P::KC;
   const int kz = min(kz0 + gc, P::H);
   const bool valid = own && kz0 + g <= P::H;
-  // shared-memory twiddles and one live column array: at r = 256 three CTAs
-  // per SM forward (two backward, where three would spill), five below
+  // shared-memory twiddles and one live column array
   const TwTab<L> twr{tw, t};
   // u2 in shared memory is the x axis' table; the y and z axes' come from global memory
   const float gyz = g1[ky] * g1[kz], u2yz = __ldg(S.u2 + L + ky) + __ldg(S.u2 + 2 * L + kz);
@@ -175,50 +177,33 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
         a[j] = cscale(cadd(c0.get(j), cmul_iu(a[j], iu[kx])), G);
       }
     }
-    if constexpr (!P::WL2) {
-      // every group is done with box 1 (C and its exchange): W~'s tile goes
-      // there (the fence orders this thread's writes to it before the copy's)
-      fence_async_smem();
-      __syncthreads();
-      static_assert(kSkip<L>, "loaded by chunks");
-      if (tid < 32 && __all_sync(0xffffffffu, ok)) load_chunks(kSpW, 1);
-      w_reload = true;
-    }
     if (valid) {
       fft_c<L, +1, IL>(a, c0, twr);  // P = unnormalised IFFT_x(chi~)
-      // Spectral sums of Eq. 4, by Parseval along x against the x-domain W~
-      // (its tile, or up to r = 128 its column straight from L2):
-      // sum_kx conj(W~(kx)) chi~(kx) = sum_x conj(W~_x(x)) P(x),
-      // sum_kx chi~(kx) = P(x = 0).
-      if constexpr (!P::WL2) {
-        box_wait(1, 1u);
-#pragma unroll
-        for (int j = 0; j < P::R1; ++j) {
-          const float2 w = has(j) ? c1.get(j) : czero();
-          am += w.x * a[j].x + w.y * a[j].y;
-        }
-      } else {
+      if constexpr (!P::HW) {
+        // Spectral sums of Eq. 4, by Parseval along x against the x-domain W~
+        // (its column straight from L2):
+        // sum_kx conj(W~(kx)) chi~(kx) = sum_x conj(W~_x(x)) P(x),
+        // sum_kx chi~(kx) = P(x = 0).
         const float2* wc = S.spec[kSpW] + (size_t)ky * P::KP + kz;
 #pragma unroll
         for (int j = 0; j < P::R1; ++j) {
           const float2 w = has(j) ? __ldcg(wc + (size_t)(t + P::T * j) * L * P::KP) : czero();
           am += w.x * a[j].x + w.y * a[j].y;
         }
+        if (t == 0) as = a[0].x;
+        wz = (kz == 0 || kz == P::H) ? 1.f : 2.f;
       }
-      if (t == 0) as = a[0].x;
-      wz = (kz == 0 || kz == P::H) ? 1.f : 2.f;
       if (own) {
 #pragma unroll
         for (int j = 0; j < P::R1; ++j) c0.put(j, a[j]);
       }
     }
     FF fm = {am * wz, 0.f}, fs = {as * wz, 0.f};  // wz in {1, 2}: exact
-    if (!__syncthreads_and(ok)) {
+    fence_async_smem();
+    if (!__syncthreads_and(ok)) {  // the tile is complete
       leave();
       return;
     }
-    fence_async_smem();
-    block_sum_ff<P::NT>(fm, fs);  // synchronises the block: the tile is complete
     if (tid == 0) {
       for (int x = 0; x < L; x += tma_rows(L)) tma_store_3d(&S.tmx[kSpChi], kz0, ky, x, box + x * P::KC);
       tma_store_commit();
@@ -227,41 +212,52 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
     // scalars. A last-block ticket here (a fence and an atomic on one address
     // per CTA, its place on the SM held for the round trip) cost more than the
     // transforms: 75 -> 63 us at r = 256 without it, 807 -> 552 at r = 512.
-    if (tid == 0) S.part[blockIdx.y * gridDim.x + blockIdx.x] = make_float4(fm.hi, fm.lo, fs.hi, fs.lo);
+    if constexpr (!P::HW) {
+      block_sum_ff<P::NT>(fm, fs);
+      if (tid == 0) S.part[blockIdx.y * gridDim.x + blockIdx.x] = make_float4(fm.hi, fm.lo, fs.hi, fs.lo);
+    }
     if (tid == 0) tma_store_wait_read();
   } else {
     // FFT_x of (g_a FFT_zy(dchi) + g_w W~ + g_s delta_{x=0}): the three terms
-    // of the adjoint spectrum combined before the transform (it is linear).
-    const Scalars* sc = S.sc;
-    const int np = sc->bparts;
+    // of the adjoint spectrum combined before the transform (it is linear); from
+    // r = 256 on the y pass has combined them.
     __shared__ float coef[3];
-    if (np > 0) {  // the plane pass left its partial sums: every CTA adds them up, the first one publishes
-      FF x, y;
-      sum_partials<P::NT>(S, np, x, y);
-      if (tid == 0) {
-        const BwdScalars q = bwd_scalars(S, ff_to_double(x), ff_to_double(y));
-        coef[0] = q.g_a;
-        coef[1] = q.g_s;
-        coef[2] = q.g_w;
-        if (blockIdx.x == 0 && blockIdx.y == 0) finalize_scalars(S, ff_to_double(x), ff_to_double(y), true);
+    if constexpr (!P::HW) {
+      const Scalars* sc = S.sc;
+      const int np = sc->bparts;
+      if (np > 0) {  // the plane pass left its partial sums: every CTA adds them up, the first one publishes
+        FF x, y;
+        sum_partials<P::NT>(S, np, x, y);
+        if (tid == 0) {
+          const BwdScalars q = bwd_scalars(S, ff_to_double(x), ff_to_double(y));
+          coef[0] = q.g_a;
+          coef[1] = q.g_s;
+          coef[2] = q.g_w;
+          if (blockIdx.x == 0 && blockIdx.y == 0) finalize_scalars(S, ff_to_double(x), ff_to_double(y), true);
+        }
+      } else if (tid == 0) {
+        coef[0] = sc->g_a;
+        coef[1] = sc->g_s;
+        coef[2] = sc->g_w;
       }
-    } else if (tid == 0) {
-      coef[0] = sc->g_a;
-      coef[1] = sc->g_s;
-      coef[2] = sc->g_w;
     }
     box_wait(0);
-    box_wait(1);
+    if constexpr (TWO) box_wait(1);
     if (!__syncthreads_and(ok)) {  // both tiles are needed from the start
       leave();
       return;
     }
-    const float ga = coef[0], gs = coef[1], gw = coef[2];
+    if constexpr (P::HW) {
 #pragma unroll
-    for (int j = 0; j < P::R1; ++j) {
-      const int x = t + P::T * j;
-      a[j] = cadd(cscale(c0.get(j), ga), has(j) ? cscale(c1.get(j), gw) : czero());
-      if (x == 0) a[j].x += gs;
+      for (int j = 0; j < P::R1; ++j) a[j] = c0.get(j);
+    } else {
+      const float ga = coef[0], gs = coef[1], gw = coef[2];
+#pragma unroll
+      for (int j = 0; j < P::R1; ++j) {
+        const int x = t + P::T * j;
+        a[j] = cadd(cscale(c0.get(j), ga), has(j) ? cscale(c1.get(j), gw) : czero());
+        if (x == 0) a[j].x += gs;
+      }
     }
     fft_c<L, -1, IL>(a, c0, twr);
     {
