@@ -89,4 +89,75 @@ __device__ __forceinline__ void fft_c(float2 (&v)[Shape<L>::R1], const Col<L>& c
   }
 }
 
+// The same for a 512-point column of an 8-column tile by 32 threads of 16 values
+// instead of 16 of 32: half the registers a thread, twice the warps on an SM, which
+// the x pass has the shared memory for (three CTAs either way): forward 487 -> 431
+// us, backward 567 -> 434 (168 -> 80 registers). 512 = 16 x 2 x 16:
+// radix 16 in registers, the exchange, then each 32-point DFT by a pair of lanes,
+// which halve it by a decimation in frequency (lane b takes the outputs 2 q + b)
+// and trade eight values by shuffles. Two adjacent columns take two warps: thread
+// t of a column is lane (t >> 4) 16 + (t & 7) 2 + column of warp (t >> 3) & 1, so
+// that a half-warp reaches 8 rows of two columns, all 32 banks, and the two lanes
+// of a pair (t, t ^ 16) share a warp.
+struct Wide512 {
+  static constexpr int R1 = 16, T = 32, C = 8;
+  static constexpr int TWP = 33, TWN = 16 * TWP;  // twiddle W^(t k1) at k1 TWP + t
+  static __device__ __forceinline__ int group(int tid) { return 2 * (tid >> 6) + (tid & 1); }
+  static __device__ __forceinline__ int lane(int tid) {
+    return ((tid & 16) | ((tid >> 2) & 8)) + ((tid >> 1) & 7);
+  }
+  // the two warps of two columns
+  static __device__ __forceinline__ void sync() {
+    asm volatile("bar.sync %0, 64;" ::"r"(1 + (int)(threadIdx.x >> 6)) : "memory");
+  }
+};
+
+struct ColWide {
+  static constexpr int RB = 64;
+  uint32_t p, px;  // row t; exchange row (t & 15) 32 + (t & 16) / 2 + (t & 7)
+  __device__ __forceinline__ ColWide(const float2* box, int t, int c) {
+    p = smem_u32(box) + (uint32_t)bxl<512>(t, c) * 8u;
+    px = smem_u32(box) + (uint32_t)bxl<512>((t & 15) * 32 + ((t & 16) >> 1) + (t & 7), c) * 8u;
+  }
+  __device__ __forceinline__ float2 get(int j) const { return Col<512>::ld(p + j * (32 * RB)); }
+  __device__ __forceinline__ void put(int j, float2 v) const { Col<512>::st(p + j * (32 * RB), v); }
+  // exchange value (k1, n) at row k1 32 + (n ^ (k1 & 7))
+  __device__ __forceinline__ void xput(int k1, float2 v) const {
+    Col<512>::st((p ^ Col<512>::flip(k1 & 7)) + k1 * (32 * RB), v);
+  }
+  // value (t & 15, 8 (t >> 4) + i + 16 h)
+  __device__ __forceinline__ float2 xget(int i, int h) const {
+    return Col<512>::ld((px ^ Col<512>::flip(i)) + h * (16 * RB));
+  }
+};
+
+template <int DIR>
+__device__ __forceinline__ void fft_wide(float2 (&v)[16], const ColWide& col, const float2* tw, int t) {
+  Dft<16, DIR>::run(v);
+#pragma unroll
+  for (int k1 = 1; k1 < 16; ++k1) {
+    float2 w = tw[k1 * Wide512::TWP + t];
+    if (DIR > 0) w.y = -w.y;
+    v[k1] = cmul(v[k1], w);
+  }
+  Wide512::sync();  // both warps have read the column
+#pragma unroll
+  for (int k1 = 0; k1 < 16; ++k1) col.xput(k1, v[k1]);
+  Wide512::sync();
+  const bool b = t >= 16;
+  sfor<0, 8>([&](auto ic) {
+    constexpr int i = decltype(ic)::value;
+    const float2 y0 = col.xget(i, 0), y1 = col.xget(i, 1);
+    const float2 s = cadd(y0, y1);
+    float2 d = twc32<i, DIR>(csub(y0, y1));  // W32^i; the other lane's n = 8 + i takes W4 more
+    if (b) d = DIR < 0 ? make_float2(d.y, -d.x) : make_float2(-d.y, d.x);
+    const float2 give = b ? s : d, keep = b ? d : s;
+    const float2 got = make_float2(__shfl_xor_sync(0xffffffffu, give.x, 16), __shfl_xor_sync(0xffffffffu, give.y, 16));
+    v[i] = b ? got : keep;
+    v[8 + i] = b ? keep : got;
+  });
+  Dft<16, DIR>::run(v);
+  Wide512::sync();  // both warps have read the exchange
+}
+
 }  // namespace dpsr
