@@ -91,8 +91,9 @@ __device__ __forceinline__ void fft_c(float2 (&v)[Shape<L>::R1], const Col<L>& c
 
 // The same for a 512-point column of an 8-column tile by 32 threads of 16 values
 // instead of 16 of 32: half the registers a thread, twice the warps on an SM, which
-// the x pass has the shared memory for (three CTAs either way): forward 487 -> 431
-// us, backward 567 -> 434 (168 -> 80 registers). 512 = 16 x 2 x 16:
+// the column passes have the shared memory for (three CTAs either way). x pass:
+// forward 487 -> 431 us, backward 567 -> 434 (168 -> 80 registers); y passes:
+// forward 398 -> 382, inverse 257 -> 234, backward 211 either way. 512 = 16 x 2 x 16:
 // radix 16 in registers, the exchange, then each 32-point DFT by a pair of lanes,
 // which halve it by a decimation in frequency (lane b takes the outputs 2 q + b)
 // and trade eight values by shuffles. Two adjacent columns take two warps: thread
@@ -106,7 +107,7 @@ struct Wide512 {
   static __device__ __forceinline__ int lane(int tid) {
     return ((tid & 16) | ((tid >> 2) & 8)) + ((tid >> 1) & 7);
   }
-  // the two warps of two columns
+  // the two warps of two columns: all 64 threads
   static __device__ __forceinline__ void sync() {
     asm volatile("bar.sync %0, 64;" ::"r"(1 + (int)(threadIdx.x >> 6)) : "memory");
   }
@@ -159,5 +160,33 @@ __device__ __forceinline__ void fft_wide(float2 (&v)[16], const ColWide& col, co
   Dft<16, DIR>::run(v);
   Wide512::sync();  // both warps have read the exchange
 }
+
+// How a column of a tile is transformed, by size: its threads, their share of the
+// values (t + T j), its shared-memory view, and the place of entry i of Solve::tw.
+template <int L>
+struct ColFft {
+  static constexpr bool WIDE = false;
+  static constexpr int R1 = Shape<L>::R1, T = Shape<L>::T, TWN = L;
+  static constexpr bool IL = T == 16;  // interleaved groups: conflict-free column accesses
+  using LN = Lanes<T, IL>;
+  using CL = Col<L>;
+  static __device__ __forceinline__ int tw_at(int i) { return i; }
+  template <int DIR>
+  static __device__ __forceinline__ void run(float2 (&v)[R1], const CL& c, const float2* tw, int t) {
+    fft_c<L, DIR, IL>(v, c, TwTab<L>{tw, t});
+  }
+  static __device__ __forceinline__ void sync() { group_sync<T, IL>(); }
+};
+template <>
+struct ColFft<512> : Wide512 {
+  static constexpr bool WIDE = true;
+  using LN = Wide512;
+  using CL = ColWide;
+  static __device__ __forceinline__ int tw_at(int i) { return (i & 15) * TWP + (i >> 4); }  // W^(t k1) at 16 t + k1
+  template <int DIR>
+  static __device__ __forceinline__ void run(float2 (&v)[R1], const CL& c, const float2* tw, int t) {
+    fft_wide<DIR>(v, c, tw, t);
+  }
+};
 
 }  // namespace dpsr

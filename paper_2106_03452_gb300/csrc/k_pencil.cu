@@ -74,21 +74,27 @@ __device__ __forceinline__ float tri_w(int d, float t) { return d ? t : 1.f - t;
 
 // Column 0 of a box holds P = X0 + i Xn, the transforms of the DC and Nyquist
 // columns packed together. Split them in place (column 0 <- X0) and hand Xn
-// to nyq(ky, value). Run by the T threads of one group.
-template <int L, bool IL = false, class Nyq>
-__device__ __forceinline__ void split_dc_nyq(float2* b, int t, Nyq nyq) {
-  constexpr int R1 = Shape<L>::R1, T = Shape<L>::T;
+// to nyq(ky, value). Called by all threads, done by those of group g = 0.
+template <int L, class Nyq>
+__device__ __forceinline__ void split_dc_nyq(float2* b, int g, int t, Nyq nyq) {
+  using F = ColFft<L>;
+  constexpr int R1 = F::R1, T = F::T;
+  if (g > (F::WIDE ? 1 : 0)) return;  // the threads that share a barrier
   float2 x0[R1];
+  if (g == 0) {
 #pragma unroll
-  for (int j = 0; j < R1; ++j) {
-    const int ky = t + T * j;
-    float2 xn;
-    unpack_dc_nyq(b[bxl<L>(ky, 0)], b[bxl<L>((L - ky) & (L - 1), 0)], x0[j], xn);
-    nyq(ky, xn);  // never column 0
+    for (int j = 0; j < R1; ++j) {
+      const int ky = t + T * j;
+      float2 xn;
+      unpack_dc_nyq(b[bxl<L>(ky, 0)], b[bxl<L>((L - ky) & (L - 1), 0)], x0[j], xn);
+      nyq(ky, xn);  // never column 0
+    }
   }
-  group_sync<T, IL>();
+  F::sync();
+  if (g == 0) {
 #pragma unroll
-  for (int j = 0; j < R1; ++j) b[bxl<L>(t + T * j, 0)] = x0[j];
+    for (int j = 0; j < R1; ++j) b[bxl<L>(t + T * j, 0)] = x0[j];
+  }
 }
 
 // Sorted-point index range of point bin (x-cell xc, y-block yb): the points
@@ -334,7 +340,7 @@ __global__ void __launch_bounds__(ZfGeo<L>::NT, ZfGeo<L>::MINB) k_zfwd(const __g
 // ===========================================================================
 template <int L>
 constexpr int ynt() {
-  return Pen<L>::W * Shape<L>::T >= 32 ? Pen<L>::W * Shape<L>::T : 32;  // one group per column
+  return Pen<L>::W * ColFft<L>::T >= 32 ? Pen<L>::W * ColFft<L>::T : 32;  // one group per column
 }
 
 template <int L, bool BWD>
@@ -344,7 +350,7 @@ constexpr int yfwd_boxes() {
 
 template <int L, bool BWD>
 constexpr size_t yfwd_smem() {
-  return box_align<L>() + sizeof(float2) * ((size_t)yfwd_boxes<L, BWD>() * Pen<L>::BOX + L) + sizeof(float) * L;
+  return box_align<L>() + sizeof(float2) * ((size_t)yfwd_boxes<L, BWD>() * Pen<L>::BOX + ColFft<L>::TWN) + sizeof(float) * L;
 }
 
 // Input buffers of a y-pass tile of kind `kind` (see k_yfwd): box 0 holds
@@ -421,9 +427,8 @@ __device__ __forceinline__ bool yfwd_tile(const Solve& S, int X, int kz0, int ki
   const YfwdBufs bb = yfwd_bufs<L, BWD>(kind);
   const int buf0 = bb.buf0;
   const bool two = !BWD && bb.two;
-  constexpr bool IL = P::T == 16;  // interleaved groups: conflict-free column accesses
-  using LN = Lanes<P::T, IL>;
-  const int tid = threadIdx.x, g = LN::group(tid), t = LN::lane(tid);
+  using F = ColFft<L>;
+  const int tid = threadIdx.x, g = F::LN::group(tid), t = F::LN::lane(tid);
   float ga = 1.f, gs = 0.f, gw = 0.f;
   if constexpr (BWD && kHalfW<L>) {
     ga = S.sc->g_a;
@@ -436,47 +441,48 @@ __device__ __forceinline__ bool yfwd_tile(const Solve& S, int X, int kz0, int ki
     mbar_wait(bar, phase);  // a last bounded chance for copies in flight
     return false;
   }
-  TwTab<L> twr{twt, t};
   if (g < P::NCOL) {  // whole groups; one column array live at a time
-    const Col<L> c0(box, t, g);
-    float2 a[P::R1];
-    // rows of blocks that were not loaded are zero (T divides a block)
-    auto has = [rows](int j) { return BWD || !kSkip<L> || ((rows >> (P::T * j / P::YB)) & 1u); };
+    const typename F::CL c0(box, t, g);
+    float2 a[F::R1];
+    // rows of blocks that were not loaded are zero (T divides a block, or spans two: t >= 16 is in the second)
+    const unsigned mine = F::T > P::YB ? rows >> (t / P::YB) : rows;
+    auto held = [mine](int j) { return (mine >> (F::T * j / P::YB)) & 1u; };
+    auto has = [held](int j) { return BWD || !kSkip<L> || held(j); };
 #pragma unroll
-    for (int j = 0; j < P::R1; ++j) a[j] = has(j) ? c0.get(j) : czero();
+    for (int j = 0; j < F::R1; ++j) a[j] = has(j) ? c0.get(j) : czero();
     if constexpr (BWD && kHalfW<L>) {
-      const Col<L> c1(box + P::BOX, t, g);
+      const typename F::CL c1(box + P::BOX, t, g);
 #pragma unroll
-      for (int j = 0; j < P::R1; ++j) {
+      for (int j = 0; j < F::R1; ++j) {
         a[j] = cscale(a[j], ga);
-        if ((rows >> (P::T * j / P::YB)) & 1u) a[j] = cadd(a[j], cscale(c1.get(j), gw));
+        if (held(j)) a[j] = cadd(a[j], cscale(c1.get(j), gw));
       }
       if (X == 0 && t == 0) {  // the delta at the origin is 1 in every kz, DC and Nyquist in one column
         a[0].x += gs;
         if (kz0 + g == 0) a[0].y += gs;
       }
     }
-    fft_c<L, -1, IL>(a, c0, twr);
+    F::template run<-1>(a, c0, twt, t);
 #pragma unroll
-    for (int j = 0; j < P::R1; ++j) c0.put(j, a[j]);
+    for (int j = 0; j < F::R1; ++j) c0.put(j, a[j]);
     if (two) {
-      const Col<L> c1(box + P::BOX, t, g);
+      const typename F::CL c1(box + P::BOX, t, g);
 #pragma unroll
-      for (int j = 0; j < P::R1; ++j) a[j] = has(j) ? c1.get(j) : czero();
-      fft_c<L, -1, IL>(a, c1, twr);
+      for (int j = 0; j < F::R1; ++j) a[j] = has(j) ? c1.get(j) : czero();
+      F::template run<-1>(a, c1, twt, t);
       // D = FFT(i u_z v_z) + i u_y FFT(v_y); this lane wrote c0 above
 #pragma unroll
-      for (int j = 0; j < P::R1; ++j) {
-        const int ky = t + P::T * j;
+      for (int j = 0; j < F::R1; ++j) {
+        const int ky = t + F::T * j;
         c0.put(j, cadd(a[j], cmul_iu(c0.get(j), iu[ky])));
       }
     }
   }
   __syncthreads();
-  if (kz0 == 0 && g == 0) {
+  if (kz0 == 0) {
     // column 0 holds X0 + i Xn of the DC and Nyquist columns: split them
     float2* dst = S.spec[buf0];
-    split_dc_nyq<L, IL>(box, t, [&](int ky, float2 w) {
+    split_dc_nyq<L>(box, g, t, [&](int ky, float2 w) {
       if (H < 16) box[bxl<L>(ky, H)] = w;
       else dst[((size_t)X * L + ky) * P::KP + H] = w;
     });
@@ -507,7 +513,7 @@ __global__ void __launch_bounds__(ynt<L>(), L == 256 ? 6 : (L >= 256 ? 3 : (BWD 
   const uint32_t pad = (AL - (smem_u32(smem_raw) & (AL - 1u))) & (AL - 1u);
   float2* box = reinterpret_cast<float2*>(smem_raw + pad);  // 1 or 2 boxes
   float2* twt = box + yfwd_boxes<L, BWD>() * P::BOX;
-  float* iu = reinterpret_cast<float*>(twt + L);
+  float* iu = reinterpret_cast<float*>(twt + ColFft<L>::TWN);
   __shared__ uint64_t bar;
   pdl_trigger();
   // thread 0 issues the tile loads first; the tables load while they fly
@@ -531,7 +537,7 @@ __global__ void __launch_bounds__(ynt<L>(), L == 256 ? 6 : (L >= 256 ? 3 : (BWD 
     yfwd_issue<L, BWD>(S, X, kz0, kind, box, &bar);
   }
   for (int i = tid; i < L; i += NT) {
-    twt[i] = S.tw[i];
+    twt[ColFft<L>::tw_at(i)] = S.tw[i];
     iu[i] = S.iu[L + i];  // y axis
   }
   __syncthreads();
@@ -555,7 +561,7 @@ constexpr int yinv_boxes() {
 
 template <int L, int NCH>
 constexpr size_t yinv_smem() {
-  return box_align<L>() + sizeof(float2) * ((size_t)yinv_boxes<L, NCH>() * Pen<L>::BOX + L) + sizeof(float) * L;
+  return box_align<L>() + sizeof(float2) * ((size_t)yinv_boxes<L, NCH>() * Pen<L>::BOX + ColFft<L>::TWN) + sizeof(float) * L;
 }
 
 // Thread 0: the TMA tile loads of an inverse y-pass tile (part: -1 all
@@ -582,9 +588,8 @@ __device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int pa
                                           uint32_t phase, unsigned rows = 0u) {
   using P = Pen<L>;
   constexpr int H = P::H;
-  constexpr bool IL = P::T == 16;  // interleaved groups: conflict-free column accesses
-  using LN = Lanes<P::T, IL>;
-  const int tid = threadIdx.x, g = LN::group(tid), t = LN::lane(tid);
+  using F = ColFft<L>;
+  const int tid = threadIdx.x, g = F::LN::group(tid), t = F::LN::lane(tid);
   float am = 0.f, as = 0.f;  // this thread's share of the sums of Eq. 4 (kHalfW)
   constexpr int NIN = NCH == 1 ? 1 : 2;
   const bool do0 = part != 1, do1 = NCH == 3 && part != 0;
@@ -594,14 +599,13 @@ __device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int pa
     mbar_wait(bar, phase);
     return false;
   }
-  TwTab<L> twr{twt, t};
   if (kz0 == 0 && g < NIN && (g == 0 ? do0 : do1)) {
     // column 0 becomes X0 + i Xn (Xn: the Nyquist column); the same lanes
     // read these elements again below
     float2* b = box + g * P::BOX;
     const float2* nq = S.spec[g == 0 ? kSpChi : kSpD] + (size_t)X * L * P::KP + H;
-    for (int j = 0; j < P::R1; ++j) {
-      const int ky = t + P::T * j;
+    for (int j = 0; j < F::R1; ++j) {
+      const int ky = t + F::T * j;
       const float2 n = H >= 16 ? nq[(size_t)ky * P::KP] : b[bxl<L>(ky, H)];
       const float2 x0 = b[bxl<L>(ky, 0)];
       b[bxl<L>(ky, 0)] = make_float2(x0.x - n.y, x0.y + n.x);
@@ -610,24 +614,25 @@ __device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int pa
   __syncthreads();
   if (g < P::NCOL) {
     const int sz = kz0 + g;
-    auto cref = [&](int k) { return Col<L>(box + k * P::BOX, t, g); };
-    float2 v[P::R1];
+    auto cref = [&](int k) { return typename F::CL(box + k * P::BOX, t, g); };
+    float2 v[F::R1];
     const auto c0 = cref(0);
     if (do0) {
 #pragma unroll
-      for (int j = 0; j < P::R1; ++j) v[j] = c0.get(j);
-      fft_c<L, +1, IL>(v, c0, twr);
+      for (int j = 0; j < F::R1; ++j) v[j] = c0.get(j);
+      F::template run<+1>(v, c0, twt, t);
 #pragma unroll
-      for (int j = 0; j < P::R1; ++j) c0.put(j, v[j]);
+      for (int j = 0; j < F::R1; ++j) c0.put(j, v[j]);
       if constexpr (NCH == 1 && kHalfW<L>) {
         // sum_ky conj(W~) chi~ = sum_y conj(W) P by Parseval along y; the half
         // spectrum counts twice but for column 0, where DC and Nyquist are
         // packed on both sides: Re(conj(W) P) is the sum of the two products
-        const Col<L> cw(box + P::BOX, t, g);
+        const typename F::CL cw(box + P::BOX, t, g);
+        const unsigned mine = F::T > P::YB ? rows >> (t / P::YB) : rows;
         const float wz = sz == 0 ? 1.f : 2.f;  // exact
 #pragma unroll
-        for (int j = 0; j < P::R1; ++j) {
-          if ((rows >> (P::T * j / P::YB)) & 1u) {
+        for (int j = 0; j < F::R1; ++j) {
+          if ((mine >> (F::T * j / P::YB)) & 1u) {
             const float2 w = cw.get(j);
             am += w.x * v[j].x + w.y * v[j].y;
           }
@@ -640,21 +645,21 @@ __device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int pa
       const auto c1 = cref(1);
       const auto c2 = cref(2);
 #pragma unroll
-      for (int j = 0; j < P::R1; ++j) {
+      for (int j = 0; j < F::R1; ++j) {
         v[j] = c1.get(j);
         c2.put(j, v[j]);
-        v[j] = cmul_iu(v[j], -iu[t + P::T * j]);
+        v[j] = cmul_iu(v[j], -iu[t + F::T * j]);
       }
-      fft_c<L, +1, IL>(v, c1, twr);
+      F::template run<+1>(v, c1, twt, t);
 #pragma unroll
-      for (int j = 0; j < P::R1; ++j) c1.put(j, v[j]);
-      group_sync<P::T, IL>();
+      for (int j = 0; j < F::R1; ++j) c1.put(j, v[j]);
+      F::sync();
 #pragma unroll
-      for (int j = 0; j < P::R1; ++j) v[j] = c2.get(j);
-      fft_c<L, +1, IL>(v, c2, twr);
+      for (int j = 0; j < F::R1; ++j) v[j] = c2.get(j);
+      F::template run<+1>(v, c2, twt, t);
       const float ez = sz == 0 ? 0.f : -__ldg(S.iu + 2 * L + sz);  // z axis
 #pragma unroll
-      for (int j = 0; j < P::R1; ++j) c2.put(j, cmul_iu(v[j], ez));
+      for (int j = 0; j < F::R1; ++j) c2.put(j, cmul_iu(v[j], ez));
     }
   }
   fence_async_smem();
@@ -707,7 +712,7 @@ __global__ void __launch_bounds__(ynt<L>(), L == 256 ? 6 : (L >= 512 ? 3 : 4))
   const uint32_t pad = (AL - (smem_u32(smem_raw) & (AL - 1u))) & (AL - 1u);
   float2* box = reinterpret_cast<float2*>(smem_raw + pad);
   float2* twt = box + yinv_boxes<L, NCH>() * P::BOX;
-  float* iu = reinterpret_cast<float*>(twt + L);
+  float* iu = reinterpret_cast<float*>(twt + ColFft<L>::TWN);
   __shared__ uint64_t bar;
   pdl_trigger();
   // thread 0 issues the tile loads first; the tables load while they fly
@@ -732,7 +737,7 @@ __global__ void __launch_bounds__(ynt<L>(), L == 256 ? 6 : (L >= 512 ? 3 : 4))
     yinv_issue<L, NCH>(S, X, kz0, part, box, &bar);
   }
   for (int i = tid; i < L; i += NT) {
-    twt[i] = S.tw[i];
+    twt[ColFft<L>::tw_at(i)] = S.tw[i];
     iu[i] = S.iu[L + i];  // y axis
   }
   __syncthreads();

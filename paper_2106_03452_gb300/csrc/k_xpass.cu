@@ -11,8 +11,6 @@
 //           to r = 128 and by the y pass above (kHalfW);  Q1 = IFFT_x(F),
 //           Q2 = IFFT_x(-i u_x F)  (the adjoint of Eq. 3, conj(H_a) = -H_a).
 // Three FFTs of length r per column in each direction.
-#include <type_traits>
-
 #include "col.cuh"
 #include "dpsr_dev.cuh"
 #include "launch.h"
@@ -23,9 +21,8 @@ namespace dpsr {
 
 template <int L>
 struct XGeo {
-  static constexpr bool WIDE = L == 512;                    // 32 threads a column (Wide512)
-  static constexpr int R1 = WIDE ? Wide512::R1 : Shape<L>::R1, T = WIDE ? Wide512::T : Shape<L>::T;
-  static constexpr int TWN = WIDE ? Wide512::TWN : L;       // twiddle entries
+  using F = ColFft<L>;
+  static constexpr int R1 = F::R1, T = F::T;
   static constexpr int KC = tile_cols(L);                   // kz columns per CTA (one TMA box row)
   static constexpr int NG = KC * T >= 32 ? KC : 32 / T;     // groups (at least one warp)
   static constexpr int NT = NG * T;                         // threads
@@ -55,7 +52,7 @@ template <int L, bool BWD>
 constexpr size_t xpass_smem() {
   using P = XGeo<L>;
   constexpr int NCH = P::template nch<BWD>();
-  return box_align<L>() + sizeof(float2) * ((size_t)NCH * P::BOX + P::TWN) + 3 * sizeof(float) * L;
+  return box_align<L>() + sizeof(float2) * ((size_t)NCH * P::BOX + P::F::TWN) + 3 * sizeof(float) * L;
 }
 
 // One CTA per (kz tile, ky): TMA loads the tiles [x][16 or 8 kz] of the
@@ -69,15 +66,14 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
   constexpr int NCH = P::template nch<BWD>();
   const Solve& S = tab ? tab[blockIdx.z] : s0;
   const int kz0 = blockIdx.x * P::KC, ky = blockIdx.y;
-  constexpr bool IL = P::T == 16;  // interleaved groups: conflict-free column accesses
-  using LN = std::conditional_t<P::WIDE, Wide512, Lanes<P::T, IL>>;
-  const int tid = threadIdx.x, g = LN::group(tid), t = LN::lane(tid);
+  using F = ColFft<L>;
+  const int tid = threadIdx.x, g = F::LN::group(tid), t = F::LN::lane(tid);
   extern __shared__ unsigned char smem_raw[];
   constexpr uint32_t AL = box_align<L>();
   const uint32_t pad = (AL - (smem_u32(smem_raw) & (AL - 1u))) & (AL - 1u);
   float2* box = reinterpret_cast<float2*>(smem_raw + pad);  // NCH boxes
   float2* tw = box + NCH * P::BOX;
-  float* g1 = reinterpret_cast<float*>(tw + P::TWN);
+  float* g1 = reinterpret_cast<float*>(tw + P::F::TWN);
   float* u2 = g1 + L;
   float* iu = u2 + L;
   // One barrier per box: the forward transforms D while C still lands.
@@ -125,8 +121,7 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
     }
   }
   for (int i = tid; i < L; i += P::NT) {
-    if constexpr (P::WIDE) tw[(i & 15) * Wide512::TWP + (i >> 4)] = S.tw[i];  // W^(t k1) at 16 t + k1
-    else tw[i] = S.tw[i];
+    tw[F::tw_at(i)] = S.tw[i];
     g1[i] = S.g1[i];
     u2[i] = S.u2[i];  // x axis
     iu[i] = S.iu[i];
@@ -150,18 +145,11 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
   const bool own = g < P::KC;
   const int kz = min(kz0 + gc, P::H);
   // (a column next to a valid one is transformed with it: they share barriers)
-  const bool valid = own && kz0 + (P::WIDE ? g & ~1 : g) <= P::H;
+  const bool valid = own && kz0 + (F::WIDE ? g & ~1 : g) <= P::H;
   // shared-memory twiddles and one live column array
-  auto fft = [&](auto dir, float2(&v)[P::R1], const auto& c) {
-    if constexpr (P::WIDE) fft_wide<decltype(dir)::value>(v, c, tw, t);
-    else fft_c<L, decltype(dir)::value, IL>(v, c, TwTab<L>{tw, t});
-  };
-  constexpr std::integral_constant<int, -1> FWD{};
-  constexpr std::integral_constant<int, 1> INV{};
   // u2 in shared memory is the x axis' table; the y and z axes' come from global memory
   const float gyz = g1[ky] * g1[kz], u2yz = __ldg(S.u2 + L + ky) + __ldg(S.u2 + 2 * L + kz);
-  using CL = std::conditional_t<P::WIDE, ColWide, Col<L>>;
-  const CL c0(box, t, gc), c1(box + P::BOX, t, gc);
+  const typename F::CL c0(box, t, gc), c1(box + P::BOX, t, gc);
   float2 a[P::R1];
   if constexpr (!BWD) {
     // Columns past Nyquist (the last kz tile) hold zeros and are not stored:
@@ -173,7 +161,7 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
       box_wait(0);
 #pragma unroll
       for (int j = 0; j < P::R1; ++j) a[j] = has(j) ? c0.get(j) : czero();
-      fft(FWD, a, c0);
+      F::template run<-1>(a, c0, tw, t);
       if (own) {  // groups past the last column (tiny r) only shadow it
 #pragma unroll
         for (int j = 0; j < P::R1; ++j) c0.put(j, a[j]);
@@ -181,7 +169,7 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
       box_wait(1);
 #pragma unroll
       for (int j = 0; j < P::R1; ++j) a[j] = has(j) ? c1.get(j) : czero();
-      fft(FWD, a, c1);
+      F::template run<-1>(a, c1, tw, t);
 #pragma unroll
       for (int j = 0; j < P::R1; ++j) {
         const int kx = t + P::T * j;  // this lane wrote c0(kx) above
@@ -190,7 +178,7 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
       }
     }
     if (valid) {
-      fft(INV, a, c0);  // P = unnormalised IFFT_x(chi~)
+      F::template run<+1>(a, c0, tw, t);  // P = unnormalised IFFT_x(chi~)
       if constexpr (!P::HW) {
         // Spectral sums of Eq. 4, by Parseval along x against the x-domain W~
         // (its column straight from L2):
@@ -271,7 +259,7 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
         if (x == 0) a[j].x += gs;
       }
     }
-    fft(FWD, a, c0);
+    F::template run<-1>(a, c0, tw, t);
     {
       // F = G (.); Q2's input -i u_x F goes to the column of W~ (read above by
       // this group), Q1 = IFFT_x(F) is transformed from registers first
@@ -281,7 +269,7 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
         a[j] = cscale(a[j], spectral_G(kx, gyz, u2yz, g1, u2));
         if (own) c1.put(j, cmul_iu(a[j], -iu[kx]));
       }
-      fft(INV, a, c0);
+      F::template run<+1>(a, c0, tw, t);
       if (own) {
 #pragma unroll
         for (int j = 0; j < P::R1; ++j) c0.put(j, a[j]);
@@ -294,7 +282,7 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? (BWD ?
       }
 #pragma unroll
       for (int j = 0; j < P::R1; ++j) a[j] = c1.get(j);
-      fft(INV, a, c1);
+      F::template run<+1>(a, c1, tw, t);
       if (own) {
 #pragma unroll
         for (int j = 0; j < P::R1; ++j) c1.put(j, a[j]);
