@@ -93,7 +93,10 @@ __device__ __forceinline__ void fft_c(float2 (&v)[Shape<L>::R1], const Col<L>& c
 // instead of 16 of 32: half the registers a thread, twice the warps on an SM, which
 // the column passes have the shared memory for (three CTAs either way). x pass:
 // forward 487 -> 431 us, backward 567 -> 434 (168 -> 80 registers); y passes:
-// forward 398 -> 382, inverse 257 -> 234, backward 211 either way. 512 = 16 x 2 x 16:
+// forward 398 -> 382, inverse 257 -> 234, backward 211 either way. (Not below: at r =
+// 128 and 256 an SM has 20 and 24 warps already, and the shuffles cost more than
+// the rest gives: forward x pass of a training batch 71 -> 79 us, of r = 256 52 -> 60.)
+// 512 = 16 x 2 x 16:
 // radix 16 in registers, the exchange, then each 32-point DFT by a pair of lanes,
 // which halve it by a decimation in frequency (lane b takes the outputs 2 q + b)
 // and trade eight values by shuffles. Two adjacent columns take two warps: thread
@@ -101,7 +104,7 @@ __device__ __forceinline__ void fft_c(float2 (&v)[Shape<L>::R1], const Col<L>& c
 // that a half-warp reaches 8 rows of two columns, all 32 banks, and the two lanes
 // of a pair (t, t ^ 16) share a warp.
 struct Wide512 {
-  static constexpr int R1 = 16, T = 32, C = 8;
+  static constexpr int R1 = 16, T = 32;
   static constexpr int TWP = 33, TWN = 16 * TWP;  // twiddle W^(t k1) at k1 TWP + t
   static __device__ __forceinline__ int group(int tid) { return 2 * (tid >> 6) + (tid & 1); }
   static __device__ __forceinline__ int lane(int tid) {

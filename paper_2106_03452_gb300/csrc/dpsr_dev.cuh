@@ -377,7 +377,7 @@ struct Solve {
   // of 16 kz x 16 ky x 1 x (a y-block), tmc boxes of 16 kz x 1 ky x r/8 x (an
   // x-chunk, forward buffers only)
   CUtensorMap tmb[kNSpec];
-  CUtensorMap tmw[kNSpec];  // as tmy, 16 columns at every r (the plane kernels)
+  CUtensorMap tmw[kNSpec];  // as tmy, 16 columns (the plane kernels, below r = 256)
   CUtensorMap tmc[4];
   int r;
   int N;

@@ -1,5 +1,7 @@
-// Scalar finalisation of a solve, run by the last block to finish of the pass
-// that produces the block partials (forward x-pass, backward plane pass).
+// Scalar finalisation of a solve: the passes leave block sums and the pass that
+// needs the scalars adds them up (from r = 256 on the forward's are added to a few
+// FP64 accumulators instead, in no fixed order); the backward z pass ends with its
+// last block doing so.
 //
 // The sums run in float-float arithmetic: a value is an FP32 pair (hi, lo)
 // whose exact sum carries it, combined with error-free transformations
