@@ -300,7 +300,8 @@ DPSR_API int dpsr_plan_profile(dpsr_plan plan, int enable);
  * (DPSR_TUNE=0 keeps the static choice). The environment can fix them:
  * DPSR_PLANE_PATHS_<r>="a,b,c,d" for grid size r, or DPSR_PLANE_PATH=c for
  * every kind and size (c in 0, 1, 2, 4, 8). From r = 256 on only the pencil
- * passes exist: at r = 256 a cluster size of 2, 4 or 8 runs them. A path
+ * passes exist; at r = 256 a cluster size of 4 or 8 (2 for the second and
+ * third kind) runs them. A path
  * that does not exist for a kind and size makes the solve fail with
  * DPSR_ECUDA. */
 DPSR_API int dpsr_plan_clusters(dpsr_plan plan, int *C4);

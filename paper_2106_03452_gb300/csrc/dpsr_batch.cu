@@ -132,7 +132,7 @@ cudaError_t tune_kind(BatchClass& c, int kind, cudaStream_t st, cudaEvent_t e0, 
   if (forced != -1 || c.r >= 256) {  // from r = 256 on there is one path
     if (forced >= 0 && c.r < 256) c.C[kind] = forced;
     c.tuned[kind] = true;
-    return dpsr::launch_plane(kind, c.r, c.C[kind], dummy, c.dtab, n, st);
+    return dpsr::launch_plane(kind, c.r, forced >= 0 ? forced : c.C[kind], dummy, c.dtab, n, st);
   }
   {  // a choice persisted by an earlier process (DPSR_TUNE_CACHE)
     const int cached = dpsr_internal_tc_lookup(kind, c.r, n);

@@ -1167,8 +1167,9 @@ cudaError_t launch_plane(int kind, int r, int C, const Solve& s, const Solve* ta
                          cudaStream_t st) {
   // A plane of r = 256 would take 2 to 8 CTAs: timed against the pencil passes
   // such clusters lost in every kind, and they need W~ whole (see kHalfW). The
-  // sizes stay accepted and run the pencil passes.
-  if (C == 0 || (r == 256 && (C == 2 || C == 4 || C == 8))) return launch_pencil(kind, r, s, tab, count, st);
+  // sizes that fitted stay accepted and run the pencil passes.
+  const bool as_pencil = r == 256 && (C == 4 || C == 8 || (C == 2 && (kind == 1 || kind == 2)));
+  if (C == 0 || as_pencil) return launch_pencil(kind, r, s, tab, count, st);
   if (C == kPathSplit) {
     if (kind != 3) return cudaErrorInvalidValue;
     if (r == 64) return launch_binv_ch_t<64>(s, tab, count, st);
