@@ -1148,7 +1148,13 @@ static cudaError_t launch_plane_t(int kind, const Solve& s, const Solve* tab, in
     if (kind == 0) block = dim3(fwd_threads<L, C>());
   }
   if (kind == 3) block = dim3(binv_threads<L, C>());
-  return launch_k(fn, dim3(L * C, 1, count), block, smem, st, C, s, tab);
+  // The transforms from points and from dchi with fewer CTAs than the GPU has SMs
+  // (152) start when the previous kernel has left: launched early they crowd onto
+  // the SMs that empty first, two to one, while others stay idle. r = 32, 200 000
+  // points: the layer 1 074 us early, 950 after; 60 000: 362 and 319; forward of
+  // 3 000: 37.4 and 38.5. The inverse kinds gain nothing by it.
+  const bool crowds = kind % 2 == 0 && L * C * count < 152;
+  return launch_at(!crowds, fn, dim3(L * C, 1, count), block, smem, st, C, s, tab);
 }
 
 template <int L>
