@@ -9,6 +9,11 @@
 //
 // Why: with 20 to 130 us of kernels a call, the Python forward and backward
 // and their argument handling took longer than the GPU.
+//
+// The interpreter lock is held to look at the arguments and at the plan's
+// attributes, and let go for the calls themselves: a first solve is tuned, a
+// plan grows its workspace and an extraction reads its count back, and each of
+// these waits for everything queued on the stream.
 #include <ATen/cuda/CUDAContext.h>
 #include <c10/core/impl/LocalDispatchKeySet.h>
 #include <c10/core/impl/TorchDispatchModeTLS.h>
@@ -44,8 +49,8 @@ void check(int rc, const char* what) {
 // and the forward that it belongs to.
 struct LayerState : torch::CustomClassHolder {
   PyObject* plan;
-  int64_t generation, n, r;
-  LayerState(PyObject* p, int64_t g, int64_t n_, int64_t r_) : plan(p), generation(g), n(n_), r(r_) { Py_INCREF(plan); }
+  int64_t generation = 0, n, r;
+  LayerState(PyObject* p, int64_t n_, int64_t r_) : plan(p), n(n_), r(r_) { Py_INCREF(plan); }
   ~LayerState() override {
     if (!Py_IsInitialized()) return;
     py::gil_scoped_acquire gil;
@@ -88,6 +93,16 @@ Tensor dense(const Tensor& g) {
   return g.contiguous();
 }
 
+// The result of `fn` for Python; fn runs without the interpreter lock.
+template <class F>
+py::object unlocked(const F& fn) {
+  auto v = [&] {
+    py::gil_scoped_release free;
+    return fn();
+  }();
+  return py::cast(v);
+}
+
 // ---------------------------------------------------------------------------
 // chi = DPSR(points, normals)
 // ---------------------------------------------------------------------------
@@ -99,21 +114,29 @@ dpsr_plan handle_of(PyObject* plan) {  // with the interpreter lock; NULL after 
 // The tensor without its graph (a leaf has none).
 py::object bare(const Tensor& t) { return py::cast(t.is_leaf() ? t : t.variable_data()); }
 
+// chi of a forward pass; without the interpreter lock.
+Tensor solve(dpsr_plan h, const Tensor& points, const Tensor& normals, int64_t r) {
+  Tensor chi = at::empty({r, r, r}, points.options());
+  check(dpsr_plan_set_stream(h, stream(points)), "dpsr_plan_set_stream");
+  check(dpsr_forward(h, ro(points), ro(normals), points.size(0), rw(chi)), "dpsr_forward");
+  return chi;
+}
+
+// A forward pass has run: the backward reads its buffers, so the plan keeps
+// them alive, and the count of forwards tells a backward whether they are still
+// its own.
+int64_t keep(py::handle plan, py::object points, py::object normals, py::object chi) {
+  plan.attr("_saved") = py::make_tuple(std::move(points), std::move(normals), std::move(chi));
+  const int64_t gen = plan.attr("generation").cast<int64_t>() + 1;
+  plan.attr("generation") = gen;
+  return gen;
+}
+
 struct Layer : torch::autograd::Function<Layer> {
-  static Tensor forward(AutogradContext* ctx, const Tensor& points, const Tensor& normals, py::handle plan,
-                        int64_t r) {
-    Tensor chi = at::empty({r, r, r}, points.options());
-    dpsr_plan h = handle_of(plan.ptr());
-    check(dpsr_plan_set_stream(h, stream(points)), "dpsr_plan_set_stream");
-    check(dpsr_forward(h, ro(points), ro(normals), points.size(0), rw(chi)), "dpsr_forward");
-    // the backward reads these buffers: the plan keeps them alive, and the
-    // count of forwards tells a backward whether they are still its own
-    plan.attr("_saved") = py::make_tuple(bare(points), bare(normals), chi.variable_data());
-    const int64_t gen = plan.attr("generation").cast<int64_t>() + 1;
-    plan.attr("generation") = gen;
-    ctx->saved_data["state"] =
-        c10::IValue::make_capsule(c10::make_intrusive<LayerState>(plan.ptr(), gen, points.size(0), r));
-    return chi;
+  static Tensor forward(AutogradContext* ctx, const Tensor& points, const Tensor& normals,
+                        const c10::intrusive_ptr<LayerState>& st, dpsr_plan h) {
+    ctx->saved_data["state"] = c10::IValue::make_capsule(st);
+    return solve(h, points, normals, st->r);
   }
   static variable_list backward(AutogradContext* ctx, variable_list grads) {
     const auto held = ctx->saved_data["state"].toCapsule();
@@ -141,7 +164,16 @@ py::object layer(py::handle points, py::handle normals, py::handle plan) {
     return py::none();
   if (plan.attr("handle").is_none() || plan.attr("_index").cast<int64_t>() != p->get_device() || !here(*p))
     return py::none();
-  return py::cast(Layer::apply(*p, *n, plan, plan.attr("r").cast<int64_t>()));
+  const Tensor a = *p, b = *n;
+  const dpsr_plan h = handle_of(plan.ptr());
+  auto st = c10::make_intrusive<LayerState>(plan.ptr(), a.size(0), plan.attr("r").cast<int64_t>());
+  Tensor chi;
+  {
+    py::gil_scoped_release free;
+    chi = Layer::apply(a, b, st, h);
+  }
+  st->generation = keep(plan, bare(a), bare(b), py::cast(chi.variable_data()));
+  return py::cast(chi);
 }
 
 // Plan.forward into a new grid.
@@ -152,14 +184,17 @@ py::object plan_forward(py::handle plan, py::handle points, py::handle normals) 
     return py::none();
   if (plan.attr("handle").is_none() || plan.attr("_index").cast<int64_t>() != p->get_device() || !here(*p))
     return py::none();
+  const Tensor a = *p, b = *n;
+  const dpsr_plan h = handle_of(plan.ptr());
   const int64_t r = plan.attr("r").cast<int64_t>();
-  Tensor chi = at::empty({r, r, r}, p->options());
-  dpsr_plan h = handle_of(plan.ptr());
-  check(dpsr_plan_set_stream(h, stream(*p)), "dpsr_plan_set_stream");
-  check(dpsr_forward(h, ro(*p), ro(*n), p->size(0), rw(chi)), "dpsr_forward");
-  plan.attr("_saved") = py::make_tuple(points, normals, chi);
-  plan.attr("generation") = plan.attr("generation").cast<int64_t>() + 1;
-  return py::cast(chi);
+  Tensor chi;
+  {
+    py::gil_scoped_release free;
+    chi = solve(h, a, b, r);
+  }
+  py::object out = py::cast(chi);
+  keep(plan, py::reinterpret_borrow<py::object>(points), py::reinterpret_borrow<py::object>(normals), out);
+  return out;
 }
 
 // ---------------------------------------------------------------------------
@@ -187,7 +222,7 @@ py::object grid_sample(py::handle chi, py::handle q) {
   const Tensor *c = plain(chi), *p = plain(q);
   if (!c || !p || !cube(*c) || !points3(*p) || c->device() != p->device() || p->size(0) < 1 || !here(*c) || !quiet())
     return py::none();
-  return py::cast(Lookup::apply(*c, *p));
+  return unlocked([a = *c, b = *p] { return Lookup::apply(a, b); });
 }
 
 // ---------------------------------------------------------------------------
@@ -216,7 +251,7 @@ py::object chamfer(py::handle a, py::handle b) {
   if (!p || !q || !points3(*p) || !points3(*q) || p->device() != q->device() || p->size(0) < 1 || q->size(0) < 1 ||
       !here(*p) || !quiet())
     return py::none();
-  return py::cast(Chamfer::apply(*p, *q));
+  return unlocked([a = *p, b = *q] { return Chamfer::apply(a, b); });
 }
 
 // ---------------------------------------------------------------------------
@@ -272,15 +307,16 @@ struct MeshPoints : torch::autograd::Function<MeshPoints> {
 py::object mesh_points(py::handle chi, double level, int64_t samples, uint64_t seed) {
   const Tensor* c = plain(chi);
   if (!c || !cube(*c) || !here(*c) || samples < 0 || !quiet()) return py::none();
-  const variable_list v = MeshPoints::apply(*c, level, samples, seed);
-  return py::make_tuple(v[0], v[1]);
+  return unlocked([a = *c, level, samples, seed] {
+    const variable_list v = MeshPoints::apply(a, level, samples, seed);
+    return std::make_pair(v[0], v[1]);
+  });
 }
 
 py::object extract(py::handle chi, double level) {
   const Tensor* c = plain(chi);
   if (!c || !cube(*c) || !here(*c) || !quiet()) return py::none();
-  auto [t, n] = extract_raw(*c, level);
-  return py::make_tuple(t, n);
+  return unlocked([a = *c, level] { return extract_raw(a, level); });
 }
 
 py::object sample(py::handle tris, py::handle nrm, int64_t m, uint64_t seed) {
@@ -289,8 +325,7 @@ py::object sample(py::handle tris, py::handle nrm, int64_t m, uint64_t seed) {
       t->size(0) < 1 || m < 1 || t->device() != n->device() || !here(*t) ||
       !quiet())
     return py::none();
-  auto [p, q] = sample_raw(*t, *n, m, seed);
-  return py::make_tuple(p, q);
+  return unlocked([a = *t, b = *n, m, seed] { return sample_raw(a, b, m, seed); });
 }
 
 }  // namespace
