@@ -58,7 +58,7 @@ class Plan:
         L.dpsr_plan_set_stream(self.handle, torch.cuda.current_stream(self.device).cuda_stream)
 
     def forward(self, points: torch.Tensor, normals: torch.Tensor, chi_out=None) -> torch.Tensor:
-        if chi_out is None:
+        if chi_out is None and type(self) is Plan:
             chi = L.binding().plan_forward(self, points, normals)
             if chi is not None:
                 return chi
@@ -124,11 +124,13 @@ class Plan:
 class DPSRFunction(torch.autograd.Function):
     """chi = DPSR(points, normals) with the library's adjoint as backward.
     apply() runs plain CUDA tensors through the same function in C++
-    (csrc/torch_bind.cpp), everything else through the methods below."""
+    (csrc/torch_bind.cpp), everything else through the methods below: a
+    subclass of the function or of the plan too, whose methods may differ."""
 
     @classmethod
     def apply(cls, points, normals, plan):
-        chi = L.binding().layer(points, normals, plan)
+        own = cls is DPSRFunction and type(plan) is Plan
+        chi = L.binding().layer(points, normals, plan) if own else None
         return super().apply(points, normals, plan) if chi is None else chi
 
     @staticmethod

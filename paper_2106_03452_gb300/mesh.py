@@ -93,7 +93,8 @@ class MeshPoints(torch.autograd.Function):
 
     @classmethod
     def apply(cls, chi, level=0.0, samples=0, seed=0):
-        out = L.binding().mesh_points(chi, level, samples, int(seed) & (2 ** 64 - 1))
+        own = cls is MeshPoints
+        out = L.binding().mesh_points(chi, level, samples, int(seed) & (2 ** 64 - 1)) if own else None
         return super().apply(chi, level, samples, seed) if out is None else out
 
     @staticmethod

@@ -36,7 +36,7 @@ class ChamferLoss(torch.autograd.Function):
 
     @classmethod
     def apply(cls, a, b):
-        loss = L.binding().chamfer(a, b)
+        loss = L.binding().chamfer(a, b) if cls is ChamferLoss else None
         return super().apply(a, b) if loss is None else loss
 
     @staticmethod

@@ -1,5 +1,5 @@
 """How the C++ entries of the hot calls sit in a Python program: what other
-threads may do meanwhile."""
+threads may do meanwhile, subclasses of the classes that call them."""
 import threading
 import time
 
@@ -68,3 +68,54 @@ def test_other_threads_run_while_a_call_waits(call):
     if call in ("extract", "mesh_points"):
         assert took > 0.1  # the call did wait
     assert gap[0] <= 0.1, (took, gap[0])
+
+
+def test_subclasses_answer_for_themselves():
+    """A subclass of a function or of the plan keeps its own methods."""
+    import torch
+    from paper_2106_03452_gb300.dpsr import DPSRFunction, Plan, dpsr
+    from paper_2106_03452_gb300.loop import GridSample
+    from paper_2106_03452_gb300.mesh import MeshPoints
+    from paper_2106_03452_gb300.optimize import ChamferLoss
+    p, n = _cloud()
+    calls = []
+
+    class Own(Plan):
+        def forward(self, points, normals, chi_out=None):
+            calls.append("forward")
+            return super().forward(points, normals, chi_out)
+
+        def backward(self, dchi, dpoints=None, dnormals=None):
+            calls.append("backward")
+            return super().backward(dchi, dpoints, dnormals)
+
+        def _bind_stream(self):
+            calls.append("stream")
+            super()._bind_stream()
+
+    plan = Own(32, 2.0)
+    a = p.clone().requires_grad_(True)
+    dpsr(a, n, plan).sum().backward()
+    assert calls == ["forward", "stream", "backward", "stream"]
+    plan.close()
+
+    def zeros(base, k):
+        class Zero(base):
+            @staticmethod
+            def backward(ctx, *g):
+                return (torch.zeros_like(ctx.x),) + (None,) * k
+
+            @staticmethod
+            def forward(ctx, x, *rest):
+                ctx.x = x
+                return base.forward(ctx, x, *rest)
+        return Zero
+
+    plan, chi = Plan(32, 2.0), _ball()
+    for fn, k, x, rest in ((DPSRFunction, 2, p, (n, plan)), (GridSample, 1, chi, (p,)), (ChamferLoss, 1, p, (p + 0.1,)),
+                           (MeshPoints, 3, chi, (0.0, 0, 0))):
+        x = x.clone().requires_grad_(True)
+        out = zeros(fn, k).apply(x, *rest)
+        (g,) = torch.autograd.grad((out[0] if isinstance(out, tuple) else out).sum(), x)
+        assert not g.any(), fn
+    plan.close()
