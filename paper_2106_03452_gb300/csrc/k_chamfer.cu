@@ -1,17 +1,32 @@
 // Bi-directional L2 Chamfer distance with exact nearest neighbours from a
 // shallow box tree, for callers that bring a workspace (dpsr_chamfer_tree).
 //
-// Per set: a counting sort along a Morton curve of 2^B cells per axis over the
-// set's bounding box, leaves of 32 consecutive points with their boxes, and
-// boxes over 32 leaves each. A query only scans the leaves whose box is not
-// farther than its best point so far. Box distances are computed with the
-// point distance's operations in the same order, and rounding is monotonic, so
-// a pruned leaf never holds a point that the brute force search would have
-// returned: indices (ties to the lowest) and distances are bit for bit its.
+// Per set: a counting sort along a Morton curve of 2^B slabs per axis, leaves
+// of 32 consecutive points with their boxes, and boxes over 32 leaves each. A
+// query only scans the leaves whose box is not farther than its best point so
+// far. Box distances are computed with the point distance's operations in the
+// same order, and rounding is monotonic, so a pruned leaf never holds a point
+// that the brute force search would have returned: indices (ties to the lowest)
+// and distances are bit for bit its.
+//
+// The slabs have equal widths over the range of a sample of 512 points, unless
+// that leaves the cells crowded (a far outlier in the sample, a cluster in a
+// large box): a query would open nearly every leaf of a cell that holds most
+// points in no order. The sort then starts again with slabs that hold equally
+// many points of the sample, narrow wherever the points are dense. 20 000 x
+// 20 000, with equal widths over the whole set's box before and now (brute force
+// 618 us): a surface 56.5 and 56.4 us, the same with one point 10^6 away 1 074 and
+// 60, a cluster in a box a thousand times its size 850 and 69, scales from 10^-4
+// to 10^3 1 059 and 79, all points of a set equal 1 407 and 129.
 //
 // Bound: 2 na nb distances by brute force (577 us for 20 000 x 20 000, one
-// thread per query and 79 blocks on 152 SMs) against a few hundred per query
-// here; what is left is the latency of the sort's phases and of the descent.
+// thread per query and 79 blocks on 152 SMs). Here a query on points of a
+// surface scans four leaves, and what is left is the latency of the sort's
+// phases and of the descent. A cell of c points costs its queries c / 32 leaves
+// each; where coordinates differ a cell of the second kind holds about a
+// slab's points (n / 16) at most, and in that worst case the scans cost half
+// the brute force.
+#include <limits.h>
 #include <math.h>
 #include <stdint.h>
 
@@ -31,7 +46,7 @@ constexpr int kQNT = 128;      // threads of a query block
 constexpr int kQW = 4;         // consecutive sorted queries of a warp
 constexpr int kQB = kQW * kQNT / 32;  // and of a block
 
-// Cells per axis 2^B: 16 up to 32 768 points (about 13 a cell on a surface),
+// Slabs per axis 2^B: 16 up to 32 768 points (about 13 a cell on a surface),
 // 32 above, where 16 would leave several leaves to a cell.
 __host__ __device__ constexpr int cell_bits(int64_t n) { return n <= 32768 ? 4 : 5; }
 
@@ -39,10 +54,10 @@ struct NnSet {
   const float* p;     // n x 3
   int n, nl1, nl2;    // points, leaves, boxes of 32 leaves
   float4* sorted;     // nl1 * 32: x, y, z, original index (padding: NaN)
-  float4* box1;       // nl1 x (lo, hi)
+  float4* box1;       // nl1 x (lo, hi); lo.w: the lowest index inside
   float4* box2;       // nl2 x (lo, hi)
   int* start;         // first sorted position of each cell
-  float* grid;        // lo[3], cells per unit length[3] of the cell grid
+  float* slab;        // 3 x 32: lower bounds of an axis' slabs 1 .. 2^B - 1
 };
 struct NnPair {
   NnSet s[2];
@@ -63,13 +78,25 @@ __device__ __forceinline__ unsigned morton3(unsigned x, unsigned y, unsigned z) 
   return spread(x) | (spread(y) << 1) | (spread(z) << 2);
 }
 
-// Cell of a point on a set's grid. Coordinates off the grid, infinite or NaN
-// go to an edge cell: the order of the points only decides how tight the
-// boxes are.
-__device__ __forceinline__ unsigned cell_of(const float* g, float x, float y, float z, int bits) {
-  const int m = (1 << bits) - 1;
-  auto q = [m](float v) { return (unsigned)min(max((int)v, 0), m); };
-  return morton3(q((x - g[0]) * g[3]), q((y - g[1]) * g[4]), q((z - g[2]) * g[5]));
+// Slab of a coordinate: the number of bounds that do not exceed it (they
+// ascend): first of those between the quarters, which every point is compared
+// with, then of the few in its quarter, read together. A NaN is in the first
+// slab: the order of the points only decides how tight the boxes are.
+template <int BITS>
+__device__ __forceinline__ unsigned slab_of(const float* bound, float v) {
+  constexpr unsigned Q = 1u << (BITS - 2);
+  const unsigned k = (v >= bound[Q - 1]) + (v >= bound[2 * Q - 1]) + (v >= bound[3 * Q - 1]);
+  unsigned n = k * Q;
+#pragma unroll
+  for (unsigned j = 0; j < Q; j += 4) {
+    const float4 b = *reinterpret_cast<const float4*>(bound + k * Q + j);
+    n += (v >= b.x) + (v >= b.y) + (v >= b.z) + (j + 4 < Q ? v >= b.w : 0);
+  }
+  return n;
+}
+template <int BITS>
+__device__ __forceinline__ unsigned cell_of(const float (&bound)[3][32], float x, float y, float z) {
+  return morton3(slab_of<BITS>(bound[0], x), slab_of<BITS>(bound[1], y), slab_of<BITS>(bound[2], z));
 }
 
 __device__ __forceinline__ float warp_min(float v) {
@@ -83,108 +110,184 @@ __device__ __forceinline__ float warp_max(float v) {
   return v;
 }
 
-// Box of the 32 points (or boxes) of a warp's lanes: lo in the low values.
-__device__ __forceinline__ void warp_box(float3 lo, float3 hi, float4* out, int lane) {
+// Box of the 32 points (or boxes) of a warp's lanes; `low` (their lowest index) goes along.
+__device__ __forceinline__ void warp_box(float3 lo, float3 hi, int low, float4* out, int lane) {
   lo.x = warp_min(lo.x);
   lo.y = warp_min(lo.y);
   lo.z = warp_min(lo.z);
   hi.x = warp_max(hi.x);
   hi.y = warp_max(hi.y);
   hi.z = warp_max(hi.z);
+  low = __reduce_min_sync(0xffffffffu, low);
   if (lane == 0) {
-    out[0] = make_float4(lo.x, lo.y, lo.z, 0.f);
+    out[0] = make_float4(lo.x, lo.y, lo.z, __int_as_float(low));
     out[1] = make_float4(hi.x, hi.y, hi.z, 0.f);
   }
 }
 
-// One cluster of 8 CTAs per set sorts it and builds its boxes: bounding box,
+// A point of the sample that places the slabs: one from each 512th of the set, at
+// a hashed place in it, so that no regularity of the input's order meets the
+// step. Every CTA of the cluster takes the same ones.
+__device__ __forceinline__ int64_t sample_index(int n) {
+  const int64_t i0 = (int64_t)threadIdx.x * n / kSortNT, i1 = (int64_t)(threadIdx.x + 1) * n / kSortNT;
+  return i0 + (int64_t)(((uint64_t)(threadIdx.x * 2654435769u) * (uint64_t)(i1 - i0)) >> 32);
+}
+
+// Bounds of slabs that hold equally many points of the sample: a bitonic sort
+// along each axis, an element a thread (45 steps, the ten that cross warps
+// through shared memory), the finite ones split evenly.
+__device__ void even_slabs(const float (&p)[3], int bits, float (&bound)[3][32]) {
+  __shared__ float sh[2][3][kSortNT];
+  const int tid = threadIdx.x;
+  float v[3];
+  int finite[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    finite[d] = __syncthreads_count(isfinite(p[d]));
+    v[d] = isfinite(p[d]) ? p[d] : INFINITY;  // behind the others
+  }
+  int turn = 0;
+#pragma unroll
+  for (int k = 2; k <= kSortNT; k <<= 1) {
+#pragma unroll
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      const bool low = ((tid & k) == 0) == ((tid & j) == 0);
+      if (j >= 32) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) sh[turn][d][tid] = v[d];
+        __syncthreads();
+      }
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const float o = j >= 32 ? sh[turn][d][tid ^ j] : __shfl_xor_sync(0xffffffffu, v[d], j);
+        v[d] = low ? fminf(v[d], o) : fmaxf(v[d], o);
+      }
+      if (j >= 32) turn ^= 1;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int d = 0; d < 3; ++d) sh[0][d][tid] = v[d];
+  __syncthreads();
+  if (tid < 32) {
+    const int q = tid + 1;  // the last entries stay infinite
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+      bound[d][tid] = q < (1 << bits) && finite[d] > 0 ? sh[0][d][q * finite[d] >> bits] : INFINITY;
+  }
+}
+
+// One cluster of 8 CTAs per set sorts it and builds its boxes: the slabs,
 // per-CTA histograms in shared memory, exclusive offsets per cell and CTA
 // through distributed shared memory (each CTA owns an eighth of the cells),
 // scatter, boxes. The phases are separated by cluster barriers, so one launch
 // does what would take five; 20 000 points are five per thread. Cluster 0 also
 // clears the gradient and the arrival counter of the query kernel.
 template <int BITS>
-__device__ void nn_sort(const NnSet& S, int* hist) {
+__device__ void nn_sort(const NnSet& S, int* hist, float (&bound)[3][32]) {
   constexpr int NC = 1 << (3 * BITS), SL = NC / kCs, PT = SL / kSortNT;  // cells, per CTA, per thread
   static_assert(PT >= 1, "a cell per thread at least");
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank(), tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   __shared__ float red[6][kSortNT / 32];
-  __shared__ float bb[6];      // this CTA's bounding box: lo, -hi
-  __shared__ float g[6];
+  __shared__ float g[6];  // equal slabs: lower end[3], slabs per unit length[3]
   __shared__ int wsum[kSortNT / 32];
+  __shared__ float wsq[kSortNT / 32];
   __shared__ int slice_total;
+  __shared__ float slice_sq;
   const int n = S.n, first = rank * kSortNT + tid;
   constexpr int STEP = kCs * kSortNT;
-  // bounding box of the finite coordinates (hi negated: minima throughout)
-  float m[6];
+  float p[3];
+  {
+    const int64_t i = sample_index(n);
 #pragma unroll
-  for (int k = 0; k < 6; ++k) m[k] = INFINITY;
-#pragma unroll 4
-  for (int64_t i = first; i < n; i += STEP) {
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const float v = S.p[3 * i + d];
-      if (isfinite(v)) {
-        m[d] = fminf(m[d], v);
-        m[3 + d] = fminf(m[3 + d], -v);
-      }
-    }
+    for (int d = 0; d < 3; ++d) p[d] = S.p[3 * i + d];
   }
+  // its range (upper ends negated: minima throughout)
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
-    m[k] = warp_min(m[k]);
-    if (lane == 0) red[k][w] = m[k];
+    const float v = warp_min(isfinite(p[k % 3]) ? (k < 3 ? p[k] : -p[k - 3]) : INFINITY);
+    if (lane == 0) red[k][w] = v;
   }
-  for (int i = tid; i < NC; i += kSortNT) hist[i] = 0;
   __syncthreads();
-  if (w < 6) {
-    const float v = warp_min(lane < kSortNT / 32 ? red[w][lane] : INFINITY);
-    if (lane == 0) bb[w] = v;
-  }
-  cl.sync();
-  if (tid < 6) {
-    float v = INFINITY;
-    for (int r = 0; r < kCs; ++r) v = fminf(v, cl.map_shared_rank(bb, r)[tid]);
-    const float lo = __shfl_sync(0x3fu, v, tid % 3), hi = -__shfl_sync(0x3fu, v, tid % 3 + 3);
+  if (w < 3) {
+    const float lo = warp_min(lane < kSortNT / 32 ? red[w][lane] : INFINITY);
+    const float hi = -warp_min(lane < kSortNT / 32 ? red[w + 3][lane] : INFINITY);
     const float sc = (float)(1 << BITS) / (hi - lo);
     const bool ok = hi > lo && isfinite(sc);
-    g[tid] = tid < 3 ? (isfinite(lo) ? lo : 0.f) : (ok ? sc : 0.f);
-    if (rank == 0) S.grid[tid] = g[tid];
+    if (lane == 0) {
+      g[w] = isfinite(lo) ? lo : 0.f;
+      g[w + 3] = ok ? sc : 0.f;
+    }
+    bound[w][lane] = ok && lane + 1 < (1 << BITS) ? lo + (float)(lane + 1) * ((hi - lo) / (float)(1 << BITS)) : INFINITY;
   }
-  __syncthreads();
-#pragma unroll 4
-  for (int64_t i = first; i < n; i += STEP)
-    atomicAdd(&hist[cell_of(g, S.p[3 * i], S.p[3 * i + 1], S.p[3 * i + 2], BITS)], 1);
-  cl.sync();
-  // this CTA's cells: counts over the CTAs, their exclusive scan, then every
-  // CTA's first position of each cell written back to its histogram
+  bool even = false;
+  // Points off the range, infinite or NaN go to an edge cell: the order of the
+  // points only decides how tight the boxes are.
+  auto cell = [&](float x, float y, float z) {
+    if (even) return cell_of<BITS>(bound, x, y, z);
+    auto q = [](float v) { return (unsigned)min(max((int)v, 0), (1 << BITS) - 1); };
+    return morton3(q((x - g[0]) * g[3]), q((y - g[1]) * g[4]), q((z - g[2]) * g[5]));
+  };
   const int c0 = rank * SL + tid * PT;
-  int run = 0, tot[PT];
+  int pos, tot[PT];
+  for (;;) {
+    for (int i = tid; i < NC; i += kSortNT) hist[i] = 0;
+    __syncthreads();
+#pragma unroll 4
+    for (int64_t i = first; i < n; i += STEP) atomicAdd(&hist[cell(S.p[3 * i], S.p[3 * i + 1], S.p[3 * i + 2])], 1);
+    cl.sync();
+    // this CTA's cells: counts over the CTAs, their exclusive scan and their squares
+    int run = 0;
+    float sq = 0.f;
 #pragma unroll
-  for (int j = 0; j < PT; ++j) {
-    tot[j] = 0;
+    for (int j = 0; j < PT; ++j) {
+      tot[j] = 0;
 #pragma unroll
-    for (int r = 0; r < kCs; ++r) tot[j] += cl.map_shared_rank(hist, r)[c0 + j];
-    run += tot[j];
+      for (int r = 0; r < kCs; ++r) tot[j] += cl.map_shared_rank(hist, r)[c0 + j];
+      run += tot[j];
+      sq = fmaf((float)tot[j], (float)tot[j], sq);
+    }
+    int incl = run;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= d) incl += v;
+      sq += __shfl_xor_sync(0xffffffffu, sq, d);
+    }
+    if (lane == 31) {
+      wsum[w] = incl;
+      wsq[w] = sq;
+    }
+    __syncthreads();
+    pos = incl - run;
+    int total = 0;
+    sq = 0.f;
+#pragma unroll
+    for (int k = 0; k < kSortNT / 32; ++k) {
+      pos += k < w ? wsum[k] : 0;
+      total += wsum[k];
+      sq += wsq[k];
+    }
+    if (tid == 0) {
+      slice_total = total;
+      slice_sq = sq;
+    }
+    cl.sync();
+    if (even) break;
+    // Crowded: a point shares its cell with more than four times as many as in a
+    // plane across the cells (on a sphere it is a sixth of the plane's). The same
+    // sum, and answer, in every CTA.
+    sq = 0.f;
+#pragma unroll
+    for (int r = 0; r < kCs; ++r) sq += *cl.map_shared_rank(&slice_sq, r);
+    if (sq <= (float)n * (64.f + (float)n * (4.f / (float)(1 << (2 * BITS))))) break;
+    even = true;
+    even_slabs(p, BITS, bound);
   }
-  int incl = run;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const int v = __shfl_up_sync(0xffffffffu, incl, d);
-    if (lane >= d) incl += v;
-  }
-  if (lane == 31) wsum[w] = incl;
-  __syncthreads();
-  int pos = incl - run, total = 0;
-#pragma unroll
-  for (int k = 0; k < kSortNT / 32; ++k) {
-    pos += k < w ? wsum[k] : 0;
-    total += wsum[k];
-  }
-  if (tid == 0) slice_total = total;
-  cl.sync();
+  if (rank == 0 && tid < 3 * 32) S.slab[tid] = bound[tid >> 5][tid & 31];
   for (int r = 0; r < rank; ++r) pos += *cl.map_shared_rank(&slice_total, r);
+  // every CTA's first position of each cell, written back to its histogram
 #pragma unroll
   for (int j = 0; j < PT; ++j) {
     S.start[c0 + j] = pos;
@@ -200,7 +303,7 @@ __device__ void nn_sort(const NnSet& S, int* hist) {
 #pragma unroll 4
   for (int64_t i = first; i < n; i += STEP) {
     const float x = S.p[3 * i], y = S.p[3 * i + 1], z = S.p[3 * i + 2];
-    const int at = atomicAdd(&hist[cell_of(g, x, y, z, BITS)], 1);
+    const int at = atomicAdd(&hist[cell(x, y, z)], 1);
     S.sorted[at] = make_float4(x, y, z, __int_as_float((int)i));
   }
   const float nan = __int_as_float(0x7fffffff);
@@ -214,19 +317,43 @@ __device__ void nn_sort(const NnSet& S, int* hist) {
     const bool bad = isnan(p.x) || isnan(p.y) || isnan(p.z);  // never anybody's neighbour
     const float3 v = make_float3(p.x, p.y, p.z);
     const float inf = INFINITY;
-    warp_box(bad ? make_float3(inf, inf, inf) : v, bad ? make_float3(-inf, -inf, -inf) : v, S.box1 + 2 * (int64_t)l, lane);
+    warp_box(bad ? make_float3(inf, inf, inf) : v, bad ? make_float3(-inf, -inf, -inf) : v,
+             bad ? INT_MAX : __float_as_int(p.w), S.box1 + 2 * (int64_t)l, lane);
   }
   __threadfence();
   cl.sync();
   for (int l = rank * (kSortNT / 32) + w; l < S.nl2; l += NW) {
-    const int64_t c = min((int64_t)l * 32 + lane, (int64_t)S.nl1 - 1);
-    const float4 lo = __ldcg(S.box1 + 2 * c), hi = __ldcg(S.box1 + 2 * c + 1);
-    warp_box(make_float3(lo.x, lo.y, lo.z), make_float3(hi.x, hi.y, hi.z), S.box2 + 2 * (int64_t)l, lane);
+    const int64_t own = (int64_t)l * 32 + lane, c = min(own, (int64_t)S.nl1 - 1);
+    float4 lo = __ldcg(S.box1 + 2 * c), hi = __ldcg(S.box1 + 2 * c + 1);
+    // Of leaves whose points are all equal, and equal to one another's, the one
+    // with the lowest index answers for all: the others' boxes are closed.
+    // Otherwise each of them is as far as the best point, and is opened.
+    const bool one = own < S.nl1 && lo.x == hi.x && lo.y == hi.y && lo.z == hi.z;
+    const unsigned ones = __ballot_sync(0xffffffffu, one);
+    if (ones & (ones - 1u)) {
+      bool closed = false;
+      for (unsigned m = ones; m; m &= m - 1u) {
+        const int src = __ffs(m) - 1;
+        const float x = __shfl_sync(0xffffffffu, lo.x, src), y = __shfl_sync(0xffffffffu, lo.y, src),
+                    z = __shfl_sync(0xffffffffu, lo.z, src);
+        const int low = __shfl_sync(0xffffffffu, __float_as_int(lo.w), src);
+        closed = closed || (one && x == lo.x && y == lo.y && z == lo.z && low < __float_as_int(lo.w));
+      }
+      if (closed) {
+        const float inf = INFINITY;
+        lo = make_float4(inf, inf, inf, lo.w);
+        hi = make_float4(-inf, -inf, -inf, 0.f);
+        S.box1[2 * own] = lo;
+        S.box1[2 * own + 1] = hi;
+      }
+    }
+    warp_box(make_float3(lo.x, lo.y, lo.z), make_float3(hi.x, hi.y, hi.z), 0, S.box2 + 2 * (int64_t)l, lane);
   }
 }
 
 __global__ void __launch_bounds__(kSortNT) k_nn_sort(const __grid_constant__ NnPair P) {
   extern __shared__ int hist[];
+  __shared__ __align__(16) float bound[3][32];
   const int set = blockIdx.x / kCs;
   pdl_trigger();
   pdl_wait();
@@ -235,8 +362,8 @@ __global__ void __launch_bounds__(kSortNT) k_nn_sort(const __grid_constant__ NnP
     if (blockIdx.x == 0 && threadIdx.x == 0) *P.ticket = 0u;
   }
   const NnSet& S = P.s[set];
-  if (cell_bits(S.n) == 4) nn_sort<4>(S, hist);
-  else nn_sort<5>(S, hist);
+  if (cell_bits(S.n) == 4) nn_sort<4>(S, hist, bound);
+  else nn_sort<5>(S, hist, bound);
 }
 
 // Squared distance between a query and a box: the operations of the point
@@ -301,7 +428,10 @@ __global__ void __launch_bounds__(kQNT) k_nn_query(const __grid_constant__ NnPai
       }
       if (bi < 0) {  // the leaf at the query's own cell
         best = INFINITY;
-        seed = min(T.start[cell_of(T.grid, q.x, q.y, q.z, cell_bits(T.n))] / kLeaf, T.nl1 - 1);
+        // slabs of the query, a lane per bound (those past the last are infinite, as q is not)
+        auto slab = [&](int d, float v) { return (unsigned)__popc(__ballot_sync(ALL, v >= T.slab[32 * d + lane])); };
+        const unsigned cell = morton3(slab(0, q.x), slab(1, q.y), slab(2, q.z));
+        seed = min(T.start[cell] / kLeaf, T.nl1 - 1);
         scan(seed);
       }
       // the lane with the smallest distance among `mask`
@@ -388,7 +518,7 @@ static size_t nn_layout(NnPair& P, int64_t na, int64_t nb, char* base) {
     S.box1 = (float4*)take(sizeof(float4) * 2 * nl1);
     S.box2 = (float4*)take(sizeof(float4) * 2 * nl2);
     S.start = (int*)take(sizeof(int) << (3 * cell_bits(n)));
-    S.grid = (float*)take(sizeof(float) * 6);
+    S.slab = (float*)take(sizeof(float) * 3 * 32);
     blocks += (n + kQB - 1) / kQB;
   }
   P.part = (float4*)take(sizeof(float4) * blocks);

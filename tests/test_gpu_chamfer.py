@@ -94,3 +94,69 @@ def test_workspace_is_checked():
     lib = L.load()
     for ws, nb in ((256, n - 1), (264, n), (0, n)):  # too small, misaligned, NULL: refused before any launch
         assert lib.dpsr_chamfer_tree(256, 10, 256, 10, ws or None, nb, 256, 256, None, None) == L.DPSR_EINVAL
+
+
+def _hard(kind, n=20000):
+    """Sets that a grid of equal cells over the bounding box cannot split."""
+    rng = synth.Rng(len(kind))
+    a, b = (synth.sphere_cloud(rng, n, jitter=0.01)[0] for _ in range(2))
+    if kind == "outlier":
+        a[7] = 1e6
+    elif kind == "outliers in both":
+        a[7], b[n - 9] = 1e6, -1e6
+    elif kind == "cluster in a large box":
+        box = rng.uniform(n // 4, 3) * 1000
+        a[::4], b[::4] = box, box + 0.5
+    elif kind == "one place":
+        b[:] = 0.25
+    elif kind == "two places":
+        a[:], b[:] = 0.75, 0.25
+    elif kind == "half in one place":
+        a[::2], b[1::2] = 0.5, 0.5
+    elif kind == "far apart":
+        b += 1e6
+    elif kind == "scales":
+        s = 10.0 ** np.floor(rng.uniform(n, 1) * 8 - 4)
+        a, b = rng.normal(n, 3) * s, rng.normal(n, 3) * s
+    elif kind == "axes":
+        k, (u, v) = np.arange(n) % 3, rng.uniform(2, n)
+        a, b = np.zeros((n, 3)), np.zeros((n, 3))
+        a[np.arange(n), k], b[np.arange(n), k] = u, v
+    return np.ascontiguousarray(a, np.float32), np.ascontiguousarray(b, np.float32)
+
+
+@pytest.mark.parametrize("kind", ["outlier", "outliers in both", "cluster in a large box", "one place", "two places",
+                                  "half in one place", "far apart", "scales", "axes"])
+def test_hard_sets_equal_bruteforce_and_cost_no_more(kind):
+    import torch
+    from paper_2106_03452_gb300 import libdpsr as L
+    a, b = (torch.from_numpy(x).cuda() for x in _hard(kind))
+    n, st = a.shape[0], torch.cuda.current_stream().cuda_stream
+    ws = torch.empty(L.dpsr_chamfer_ws_bytes(n, n), dtype=torch.uint8, device="cuda")
+    idx, d2 = torch.empty(2 * n, dtype=torch.int32, device="cuda"), torch.empty(2 * n, device="cuda")
+    out = []
+    for tree in (True, False):
+        g, loss = torch.empty_like(a), torch.empty(1, dtype=torch.float64, device="cuda")
+
+        def call():
+            if tree:
+                L.dpsr_chamfer_tree(a.data_ptr(), n, b.data_ptr(), n, ws.data_ptr(), ws.numel(), g.data_ptr(),
+                                    loss.data_ptr(), 0, st)
+            else:
+                L.dpsr_chamfer(a.data_ptr(), n, b.data_ptr(), n, idx.data_ptr(), d2.data_ptr(), g.data_ptr(),
+                               loss.data_ptr(), st)
+        call()
+        ms = []
+        for _ in range(5):
+            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            e[0].record()
+            call()
+            e[1].record()
+            e[1].synchronize()
+            ms.append(e[0].elapsed_time(e[1]))
+        out.append((loss.item(), g.cpu().double(), sorted(ms)[2]))
+    (l1, g1, t1), (l0, g0, t0) = out
+    # the same neighbours: sums of the same terms in another order
+    assert abs(l1 - l0) <= 1e-6 * abs(l0)
+    assert float((g1 - g0).abs().max()) <= 1e-5 * float(g0.abs().max())
+    assert t1 <= t0, (t1, t0)
