@@ -130,9 +130,12 @@ cudaError_t tune_kind(BatchClass& c, int kind, cudaStream_t st, cudaEvent_t e0, 
   const int n = (int)c.members.size();
   const int forced = dpsr_internal_forced(kind, c.r);
   if (forced != -1 || c.r >= 256) {  // from r = 256 on there is one path
-    if (forced >= 0 && c.r < 256) c.C[kind] = forced;
+    const int C = forced >= 0 ? forced : c.C[kind];
+    const cudaError_t e = dpsr::launch_plane(kind, c.r, C, dummy, c.dtab, n, st);
+    if (e != cudaSuccess) return e;  // a path that does not exist: not kept
+    if (c.r < 256) c.C[kind] = C;
     c.tuned[kind] = true;
-    return dpsr::launch_plane(kind, c.r, forced >= 0 ? forced : c.C[kind], dummy, c.dtab, n, st);
+    return e;
   }
   {  // a choice persisted by an earlier process (DPSR_TUNE_CACHE)
     const int cached = dpsr_internal_tc_lookup(kind, c.r, n);
@@ -178,6 +181,24 @@ cudaError_t tune_kind(BatchClass& c, int kind, cudaStream_t st, cudaEvent_t e0, 
   cudaError_t e = dpsr::launch_plane(kind, c.r, bestC, dummy, c.dtab, n, st);
   if (e == cudaSuccess && best < 1e30f) dpsr_internal_tc_store(kind, c.r, n, bestC, best);
   return e;
+}
+
+// After a run that failed on its way: the x pass may not have cleared the bin
+// counters that its binning counted into, and the next run needs them at zero
+// (offsets from counts of two runs would lie past the sorted points). A run that
+// was only being captured has counted nothing.
+int failed(dpsr_batch b) {
+  cudaGetLastError();
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(b->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return DPSR_ECUDA;
+  }
+  for (auto& c : b->classes) cudaStreamSynchronize(c.st);
+  for (const Solve& s : b->host) cudaMemsetAsync(s.bins, 0, sizeof(int) * dpsr::bins_ints(s.r), b->stream);
+  b->have_fwd = false;
+  cudaGetLastError();
+  return DPSR_ECUDA;
 }
 
 // One eager forward (and backward) of every class on the batch stream, tuning
@@ -336,10 +357,7 @@ int dpsr_batch_forward(dpsr_batch b) {
   int rc = upload(b);
   if (rc != DPSR_OK) return rc;
   const bool tune = needs_tuning(b, false);
-  if ((tune ? tune_batch(b, false) : launch_fwd(b)) != cudaSuccess) {
-    cudaGetLastError();
-    return DPSR_ECUDA;
-  }
+  if ((tune ? tune_batch(b, false) : launch_fwd(b)) != cudaSuccess) return failed(b);
   b->have_fwd = true;
   return DPSR_OK;
 }
@@ -354,7 +372,8 @@ int dpsr_batch_backward(dpsr_batch b) {
   if (rc != DPSR_OK) return rc;
   // tuning the backward kinds runs the forward again first (it is idempotent)
   const bool tune = needs_tuning(b, true);
-  if ((tune ? tune_batch(b, true) : launch_bwd(b)) != cudaSuccess) {
+  if (tune) return tune_batch(b, true) == cudaSuccess ? DPSR_OK : failed(b);
+  if (launch_bwd(b) != cudaSuccess) {
     cudaGetLastError();
     return DPSR_ECUDA;
   }
@@ -378,10 +397,7 @@ static int graph_launch(dpsr_batch b, int mode) {
     drop_graph(b);
     if (b->stream == nullptr) return DPSR_EINVAL;  // capture needs a non-default stream
     if (needs_tuning(b, with_bwd)) {  // picks the paths the graph will hold
-      if (tune_batch(b, with_bwd) != cudaSuccess) {
-        cudaGetLastError();
-        return DPSR_ECUDA;
-      }
+      if (tune_batch(b, with_bwd) != cudaSuccess) return failed(b);
     }
     cudaGraph_t g = nullptr;
     if (cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
@@ -479,10 +495,7 @@ int dpsr_internal_batch_run(dpsr_batch b, int k, int with_bwd) {
   int rc = upload(b);
   if (rc != DPSR_OK) return rc;
   if (needs_tuning(b, with_bwd != 0)) {  // once, on the whole class (all bound)
-    if (tune_batch(b, with_bwd != 0) != cudaSuccess) {
-      cudaGetLastError();
-      return DPSR_ECUDA;
-    }
+    if (tune_batch(b, with_bwd != 0) != cudaSuccess) return failed(b);
     return DPSR_OK;
   }
   cudaStream_t st = b->stream;
@@ -496,10 +509,7 @@ int dpsr_internal_batch_run(dpsr_batch b, int k, int with_bwd) {
     if (e == cudaSuccess) e = dpsr::launch_plane(3, c.r, c.C[3], dummy, c.dtab, k, st);
     if (e == cudaSuccess) e = dpsr::launch_combine(dummy, c.dtab, k, c.nmax, c.C[3] == dpsr::kPathSplit, st);
   }
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return DPSR_ECUDA;
-  }
+  if (e != cudaSuccess) return failed(b);
   b->have_fwd = true;
   return DPSR_OK;
 }
