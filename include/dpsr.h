@@ -228,17 +228,18 @@ DPSR_API int dpsr_mesh_surrogate_splat(float *dchi, int r, const float *points, 
  * (nearest neighbours by brute force, ties to the lowest index), written to
  * *loss (one double), and its gradient with respect to a into grad_a
  * (na x 3, overwritten; float atomics). ws_idx: na + nb ints, ws_d2: na + nb
- * floats of caller-owned scratch. */
+ * floats of caller-owned scratch. A point with a coordinate that is not finite
+ * has no neighbour: the loss is then not finite, and such a point of a gets a
+ * NaN gradient. */
 DPSR_API int dpsr_chamfer(const float *a, int64_t na, const float *b, int64_t nb, int *ws_idx, float *ws_d2,
                           float *grad_a, double *loss, void *stream);
 /* The same loss and gradient with a workspace that holds a spatial tree over
  * each set: the same nearest neighbours (ties to the lowest index) without
  * looking at every pair. ws: ws_bytes >= dpsr_chamfer_ws_bytes(na, nb) device
  * bytes on a 16-byte boundary, scratch of this call. loss32 (may be NULL)
- * receives the loss rounded to float. A point with a coordinate that is not
- * finite has no neighbour: the loss is then not finite, and such a point of a
- * gets a NaN gradient. DPSR_EINVAL as dpsr_chamfer, and for a workspace that
- * is too small or misaligned; dpsr_chamfer_ws_bytes returns 0 for sizes out
+ * receives the loss rounded to float. Points that are not finite as in
+ * dpsr_chamfer. DPSR_EINVAL as dpsr_chamfer, and for a workspace that is too
+ * small or misaligned; dpsr_chamfer_ws_bytes returns 0 for sizes out
  * of range (below 1, or above INT32_MAX). */
 DPSR_API size_t dpsr_chamfer_ws_bytes(int64_t na, int64_t nb);
 DPSR_API int dpsr_chamfer_tree(const float *a, int64_t na, const float *b, int64_t nb, void *ws, size_t ws_bytes,

@@ -59,7 +59,9 @@ __global__ void __launch_bounds__(256) k_nearest(const float* __restrict__ q, in
 }
 
 // dL/da for L = mean_a min_b |a-b|^2 + mean_b min_a |a-b|^2 with respect to
-// the points a (the second term scatters: each b pulls its nearest a).
+// the points a (the second term scatters: each b pulls its nearest a). A point
+// without a neighbour (index -1: no finite distance) pulls nobody, and one of a
+// gets a NaN gradient.
 __global__ void __launch_bounds__(256) k_chamfer_grad(const float* __restrict__ a, int64_t na,
                                                       const float* __restrict__ b, int64_t nb,
                                                       const int* __restrict__ ab, const int* __restrict__ ba,
@@ -70,10 +72,12 @@ __global__ void __launch_bounds__(256) k_chamfer_grad(const float* __restrict__ 
     if (i < na) {
       const int j = ab[i];
 #pragma unroll
-      for (int d = 0; d < 3; ++d) atomicAdd(&ga[3 * i + d], ca * (a[3 * i + d] - b[3 * (int64_t)j + d]));
+      for (int d = 0; d < 3; ++d)
+        atomicAdd(&ga[3 * i + d], j >= 0 ? ca * (a[3 * i + d] - b[3 * (int64_t)j + d]) : __int_as_float(0x7fffffff));
     } else {
       const int64_t k = i - na;
       const int j = ba[k];
+      if (j < 0) continue;
 #pragma unroll
       for (int d = 0; d < 3; ++d) atomicAdd(&ga[3 * (int64_t)j + d], cb * (a[3 * (int64_t)j + d] - b[3 * k + d]));
     }

@@ -160,3 +160,30 @@ def test_hard_sets_equal_bruteforce_and_cost_no_more(kind):
     assert abs(l1 - l0) <= 1e-6 * abs(l0)
     assert float((g1 - g0).abs().max()) <= 1e-5 * float(g0.abs().max())
     assert t1 <= t0, (t1, t0)
+
+
+def test_bruteforce_with_points_that_are_not_finite():
+    """dpsr_chamfer's points without a neighbour are nobody's, as the tree's
+    (their index is -1; buffers with guards around them stay as they are)."""
+    import torch
+    from paper_2106_03452_gb300 import libdpsr as L
+    rng = synth.Rng(6)
+    a, b = (torch.from_numpy(rng.uniform(n, 3).astype(np.float32)).cuda() for n in (500, 600))
+    a[0, 1], a[7, 0], a[20] = np.nan, np.inf, 3e38
+    b[0], b[5, 2] = np.nan, -np.inf
+    st = torch.cuda.current_stream().cuda_stream
+    g = torch.full((500 + 20, 3), 7.0, device="cuda")
+    loss = torch.empty(1, dtype=torch.float64, device="cuda")
+    idx, d2 = torch.empty(1100, dtype=torch.int32, device="cuda"), torch.empty(1100, device="cuda")
+    L.dpsr_chamfer(a.data_ptr(), 500, b.data_ptr(), 600, idx.data_ptr(), d2.data_ptr(), g[10:].data_ptr(),
+                   loss.data_ptr(), st)
+    assert bool((g[:10] == 7).all()) and bool((g[510:] == 7).all())
+    ws = torch.empty(L.dpsr_chamfer_ws_bytes(500, 600), dtype=torch.uint8, device="cuda")
+    t = torch.empty_like(a)
+    L.dpsr_chamfer_tree(a.data_ptr(), 500, b.data_ptr(), 600, ws.data_ptr(), ws.numel(), t.data_ptr(), loss.data_ptr(),
+                        0, st)
+    g = g[10:510]
+    bad = torch.isnan(g)
+    assert torch.equal(bad, torch.isnan(t)) and bool(bad[[0, 7, 20]].all()) and int(bad.any(1).sum()) == 3
+    assert float((g - t)[~bad].abs().max()) <= 1e-5 * float(t[~bad].abs().max())
+    assert not np.isfinite(loss.item())
