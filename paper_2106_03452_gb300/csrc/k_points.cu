@@ -302,9 +302,9 @@ __global__ void __launch_bounds__(256) k_grid_splat(float* __restrict__ grid, in
 // mean squared error between the solved indicator grid chi and a target grid
 // (the solve of a dense ground-truth sampling), and its gradient, in one pass:
 //   loss = (1/n) sum_j (chi_j - target_j)^2,   dchi_j = (2/n) (chi_j - target_j).
-// Per-thread FP32 sums, float-float block and grid sums (the last block to
-// arrive writes sc->loss), deterministic. n = r^3 is a power of two, so 2/n
-// and 1/n are exact.
+// Eight squares are summed in FP32, everything beyond in float-float (the last
+// block to arrive writes sc->loss), deterministic. n = r^3 is a power of two, so
+// 2/n and 1/n are exact.
 // ---------------------------------------------------------------------------
 // float4 of each grid per thread. Every block costs a ticket (a fence and an
 // atomic on its instance's counter): a batch's two classes 45.4 us with 2, 40.9 with 8.
@@ -323,19 +323,23 @@ __global__ void __launch_bounds__(256) k_mse_grad(const __grid_constant__ Solve 
   // this instance's blocks (a batch launch sizes the grid for its largest r)
   const int nblk = (int)min((int64_t)gridDim.x, max(n4 / (kMsePer * NT), (int64_t)1));
   if ((int)blockIdx.x >= nblk) return;
-  float acc = 0.f;
-#pragma unroll 4
-  for (int64_t i = blockIdx.x * (int64_t)NT + threadIdx.x; i < n4; i += (int64_t)nblk * NT) {
+  FF acc = {0.f, 0.f}, z = acc;
+  auto squares = [&](int64_t i) {
     const float4 a = __ldcs(chi + i), b = __ldcs(tg + i);
     const float4 d = make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
     __stcs(g + i, make_float4(two_n * d.x, two_n * d.y, two_n * d.z, two_n * d.w));
-    acc += (d.x * d.x + d.y * d.y) + (d.z * d.z + d.w * d.w);
+    return (d.x * d.x + d.y * d.y) + (d.z * d.z + d.w * d.w);
+  };
+  const int64_t step = (int64_t)nblk * NT;
+#pragma unroll 2
+  for (int64_t i = blockIdx.x * (int64_t)NT + threadIdx.x; i < n4; i += 2 * step) {
+    const float one = squares(i);
+    acc = ff_add(acc, i + step < n4 ? one + squares(i + step) : one);
   }
-  FF a = {acc, 0.f}, z = {0.f, 0.f};
-  block_sum_ff<NT>(a, z);
+  block_sum_ff<NT>(acc, z);
   __shared__ unsigned last;
   if (threadIdx.x == 0) {
-    S.part[blockIdx.x] = make_float4(a.hi, a.lo, 0.f, 0.f);
+    S.part[blockIdx.x] = make_float4(acc.hi, acc.lo, 0.f, 0.f);
     __threadfence();
     last = atomicAdd(&S.sc->ticket[2], 1u) == (unsigned)nblk - 1u ? 1u : 0u;
     if (last) __threadfence();
