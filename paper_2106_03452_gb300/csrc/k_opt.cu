@@ -193,18 +193,6 @@ __device__ __forceinline__ double u01(uint64_t seed, uint64_t i) {
 constexpr int kScanBlock = 1024;  // triangles per block of the scan
 constexpr int kScanNT = 256;      // its threads, four consecutive triangles each
 
-// Square root by Newton's iteration in FP64 from an FP32 reciprocal root: r
-// is corrected twice by half the residual over r (2^-22, 2^-44, rounding).
-// Six operations on the narrow FP64 pipe.
-__device__ __forceinline__ double newton_sqrt(double s) {
-  if (!(s > 1e-30 && s < 1e30)) return sqrt(s);  // off the FP32 seed's range
-  const float y = rsqrtf((float)s);
-  const double h = (double)(0.5f * y);
-  double r = s * (double)y;
-  r = fma(fma(-r, r, s), h, r);
-  return fma(fma(-r, r, s), h, r);
-}
-
 // b - a in FP32, and whether that is exact and a normal number or zero (TwoSum's
 // error term; close coordinates, the usual case, leave none; NaN is not).
 __device__ __forceinline__ float diff32(float b, float a, bool& ok) {
@@ -240,11 +228,12 @@ __device__ __forceinline__ double cross2(const float* c) {
 
 // Areas and their prefix sums within blocks of 1 024 triangles, in FP64. The
 // bound is the FP64 pipe (a warp instruction per 15 SM cycles): exact FP32
-// differences instead of FP64 ones, a Newton root instead of the library's and
-// a scan of thread totals (four triangles a thread) instead of ten rounds over
-// every triangle. The triangles pass through shared memory: whole lines from
-// HBM, and nine conflict-free 16-byte reads a thread. 150 001 triangles: 12.2
-// -> 10.9 us, of which the FP64 operations are about 7.
+// differences instead of FP64 ones, and a scan of thread totals (four triangles
+// a thread) instead of ten rounds over every triangle. The triangles pass
+// through shared memory: whole lines from HBM, and nine conflict-free 16-byte
+// reads a thread. (A Newton root from an FP32 seed in place of sqrt() had the
+// last bit wrong in one area of some 2^14, and sampling 20 000 points on 150 001
+// triangles took 22.5 us with it, 20.5 with sqrt().)
 __global__ void __launch_bounds__(kScanNT) k_area_scan(const float* __restrict__ tris, int64_t T,
                                                        double* __restrict__ cum, double* __restrict__ block_tot) {
   constexpr int PT = kScanBlock / kScanNT;
@@ -272,7 +261,7 @@ __global__ void __launch_bounds__(kScanNT) k_area_scan(const float* __restrict__
   double a[PT];
 #pragma unroll
   for (int q = 0; q < PT; ++q) {
-    a[q] = fma(0.5, newton_sqrt(cross2(t + 9 * q)), q ? a[q - 1] : 0.0);
+    a[q] = fma(0.5, sqrt(cross2(t + 9 * q)), q ? a[q - 1] : 0.0);
   }
   double incl = a[PT - 1];
 #pragma unroll
@@ -329,7 +318,7 @@ __global__ void __launch_bounds__(kScanNT) k_block_offsets(double* __restrict__ 
 // five dependent reads of a 1 024-triangle block instead of ten. The searches
 // live in L1, and the grid is small: launched early it would crowd onto the SMs
 // that the scan leaves free, so it waits (20 000 points on 150 001 triangles,
-// both kernels: 40 us early with the offsets in a launch of their own, 22.5).
+// both kernels: 40 us early with the offsets in a launch of their own, 20.5).
 constexpr int kOffShared = 2048;
 constexpr int kSampleNT = 64;  // 20 000 samples: 313 blocks, two per SM (the searches compare on the FP64 pipe)
 __global__ void __launch_bounds__(kSampleNT) k_sample(const float* __restrict__ tris, const float* __restrict__ nrm,

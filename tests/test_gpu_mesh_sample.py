@@ -57,3 +57,39 @@ def test_sample_matches_fp64(T, offset):
     # FP32 edge vectors and one rounding of the point: 3 x 2^-24 of coordinates below 1
     assert np.max(np.abs(P - want)[clear]) <= 3e-7
     assert np.array_equal(N[clear], nrm.astype(np.float64)[k][clear])
+
+
+def _hard_roots(count):
+    """Pairs of whole numbers whose y^2 + z^2 (exact in FP64) has a root within
+    2^-13 of the middle between two doubles."""
+    rng = np.random.default_rng(7)
+    y, z = (rng.integers(2 ** 22, 2 ** 24, 4_000_000).astype(np.float64) for _ in range(2))
+    s = y * y + z * z
+    r = np.sqrt(s)
+    c = r * 134217729.0  # Veltkamp's split: r * r = p + e exactly
+    hi = c - (c - r)
+    lo = r - hi
+    p = r * r
+    e = ((hi * hi - p) + 2 * hi * lo) + lo * lo
+    off = np.abs((s - p) - e) / (2 * r) / np.spacing(r)  # distance of the root from its rounding, in ulps
+    k = np.argsort(np.abs(off - 0.5))[:count]
+    return y[k].astype(np.float32), z[k].astype(np.float32), s[k]
+
+
+def test_areas_are_correctly_rounded():
+    """Areas 0.5 sqrt(y^2 + z^2) at the hardest roots, bit for bit: the sums in
+    the workspace start at each block of 1 024 triangles, here one with an area."""
+    import torch
+    from paper_2106_03452_gb300 import libdpsr as L
+    y, z, s = _hard_roots(1000)
+    T = 1024 * len(y)
+    tris = torch.zeros((len(y), 1024, 3, 3), device="cuda")
+    tris[:, 0, 1, 0] = 1.0  # edges (1, 0, 0) and (0, y, z): cross (0, -z, y)
+    tris[:, 0, 2, 1:] = torch.from_numpy(np.stack([y, z], 1)).cuda()
+    ws = torch.empty(T + len(y) + 1, dtype=torch.float64, device="cuda")
+    out = torch.empty((2, 8, 3), device="cuda")
+    nrm = torch.zeros((T, 3), device="cuda")
+    L.dpsr_mesh_sample(tris.data_ptr(), nrm.data_ptr(), T, 8, 1, ws.data_ptr(), out[0].data_ptr(), out[1].data_ptr(),
+                       torch.cuda.current_stream().cuda_stream)
+    got = ws[:T].view(-1, 1024)[:, 0].cpu().numpy()
+    assert np.array_equal(got, 0.5 * np.sqrt(s))
