@@ -369,8 +369,8 @@ __global__ void __launch_bounds__(kSampleNT) k_sample(const float* __restrict__ 
     int b = 0, e = nblocks;  // off[b] <= x (off[0] = 0), off[e] > x or e the end
     while (e - b > 1) {
       const int mid = (b + e) >> 1;
-      if (off[mid] <= x) b = mid;
-      else e = mid;
+      if (off[mid] > x) e = mid;
+      else b = mid;  // NaN areas too: the last triangle answers, as in the second search
     }
     const double base = off[b];
     int64_t lo = (int64_t)b * kScanBlock, hi = std::min<int64_t>(lo + kScanBlock, T) - 1;

@@ -93,3 +93,17 @@ def test_areas_are_correctly_rounded():
                        torch.cuda.current_stream().cuda_stream)
     got = ws[:T].view(-1, 1024)[:, 0].cpu().numpy()
     assert np.array_equal(got, 0.5 * np.sqrt(s))
+
+
+@pytest.mark.parametrize("T", [1000, 3000, 2048 * 1024 + 5])
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_areas_that_are_not_finite(T, bad):
+    """Without a total area there is nothing to search for: every sample falls
+    on the last triangle, however many scan blocks there are."""
+    import torch
+    from paper_2106_03452_gb300.mesh import sample
+    tris = torch.rand((T, 3, 3), device="cuda")
+    tris[10, 1, 2] = bad
+    nrm = torch.arange(T, device="cuda", dtype=torch.float32)[:, None].expand(T, 3).contiguous()
+    _, n = sample(tris, nrm, 500, 3)
+    assert torch.equal(n, nrm[-1].expand(500, 3))
