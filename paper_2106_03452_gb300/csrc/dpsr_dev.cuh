@@ -514,7 +514,9 @@ constexpr bool kSkip = L >= 64;
 // Below, the cluster kernels finish a plane on chip and need the sums before.
 template <int L>
 constexpr bool kHalfW = L >= 256;
-constexpr int kMuSlots = 8;  // accumulators of that product, double2 (mu, chi'(0)) at the start of Solve::part
+// Accumulators of that product, double2 (mu, chi'(0)) at the start of Solve::part
+// (see add_exact); four copies, so that the additions do not queue.
+constexpr int kMuBins = 7, kMuCopies = 4;
 
 __host__ __device__ __forceinline__ const unsigned* occ_words(const int* bins, int r) {
   return reinterpret_cast<const unsigned*>(bins + 3 * (size_t)nbins(r) + 1);

@@ -1,7 +1,7 @@
 // Scalar finalisation of a solve: the passes leave block sums and the pass that
-// needs the scalars adds them up (from r = 256 on the forward's are added to a few
-// FP64 accumulators instead, in no fixed order); the backward z pass ends with its
-// last block doing so.
+// needs the scalars adds them up in a fixed order (from r = 256 on the forward's go
+// to FP64 accumulators instead, whose additions are exact); the backward z pass ends
+// with its last block doing so.
 //
 // The sums run in float-float arithmetic: a value is an FP32 pair (hi, lo)
 // whose exact sum carries it, combined with error-free transformations
@@ -76,6 +76,46 @@ __device__ __forceinline__ void block_sum_ff(FF& a, FF& b) {
       b = ff_add(b, red[1][w]);
     }
   }
+}
+
+// Sums in no fixed order with one result: lane 0's v in pieces, a lane of the warp
+// and a bin for each: the bits of v from a bin's unit 2^(90 - 40 b) up to the next
+// bin's. Less than 2^40 units each, so that 2^13 pieces add up exactly in FP64, in
+// any order. Float pairs are multiples of 2^-149 below 2^130: seven bins hold all of
+// v. A value that is not finite goes to bin 0 as it is. `slot`: the first bin, the
+// others two doubles apart. (The inverse y pass at r = 512: 240 us with plain
+// additions, 242 so; 252 with the pieces taken off one after the other.)
+__device__ __forceinline__ void add_exact(double* slot, double v, int lane) {
+  v = __shfl_sync(0xffffffffu, v, 0);
+  auto above = [v](int unit) {  // v without the bits below 2^unit
+    const long long bits = __double_as_longlong(v);
+    const int keep = (int)((bits >> 52) & 0x7ff) - 1023 - unit;  // of the 52 behind the leading one
+    return keep < 0 ? 0.0 : (keep >= 52 ? v : __longlong_as_double(bits & (-1ll << (52 - keep))));
+  };
+  const bool finite = isfinite(v);
+  if (lane >= kMuBins || (!finite && lane > 0)) return;
+  const int unit = 90 - 40 * lane;
+  const double p = finite ? above(unit) - (lane > 0 ? above(unit + 40) : 0.0) : v;
+  if (p != 0.0) atomicAdd(slot + 2 * lane, p);
+}
+
+// A warp: the sums of the bins, in lane 0 (copies, then bins from the smallest, in
+// that order).
+__device__ __forceinline__ double2 sum_bins(const double2* slots, int lane) {
+  const double2 own = lane < kMuCopies * kMuBins ? __ldcg(slots + lane) : make_double2(0.0, 0.0);
+  double2 v = own;
+#pragma unroll
+  for (int c = 1; c < kMuCopies; ++c) {
+    v.x += __shfl_down_sync(0xffffffffu, own.x, c * kMuBins);
+    v.y += __shfl_down_sync(0xffffffffu, own.y, c * kMuBins);
+  }
+  double2 s = make_double2(0.0, 0.0);
+#pragma unroll
+  for (int b = kMuBins - 1; b >= 0; --b) {
+    s.x += __shfl_sync(0xffffffffu, v.x, b);
+    s.y += __shfl_sync(0xffffffffu, v.y, b);
+  }
+  return s;
 }
 
 // The scalars of Eq. 4 from the forward's reduced sums:

@@ -672,10 +672,10 @@ __device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int pa
     if (rows != 0u || X == 0) {  // the same for the whole block
       FF fm = {am, 0.f}, fs = {as, 0.f};
       block_sum_ff<ynt<L>()>(fm, fs);
-      if (tid == 0) {  // a few addresses, nothing waits for the additions
-        double2* slot = reinterpret_cast<double2*>(S.part) + blockIdx.x % kMuSlots;
-        atomicAdd(&slot->x, ff_to_double(fm));
-        if (X == 0) atomicAdd(&slot->y, ff_to_double(fs));
+      if (tid < 32) {  // a few addresses, nothing waits for the additions
+        double2* slot = reinterpret_cast<double2*>(S.part) + blockIdx.x % kMuCopies * kMuBins;
+        add_exact(&slot->x, ff_to_double(fm), tid);
+        if (X == 0) add_exact(&slot->y, ff_to_double(fs), tid);
       }
     }
     if (tid == 0) tma_store_wait_read();
@@ -1087,19 +1087,13 @@ __global__ void __launch_bounds__(ZiGeo<L, NCH>::NT, L >= 512 ? (NCH == 1 ? 2 : 
   __shared__ float2 ab;
   if constexpr (MU) {
     if (tid == 0 && (int)blockIdx.x < ntiles) zinv_issue<L, NCH>(S, blockIdx.x, stg, &bar[0]);
-    if (tid == 32) {
-      const double2* slots = reinterpret_cast<const double2*>(S.part);
-      double2 v[kMuSlots];
-#pragma unroll
-      for (int q = 0; q < kMuSlots; ++q) v[q] = __ldcg(slots + q);
-#pragma unroll
-      for (int q = 1; q < kMuSlots; ++q) {
-        v[0].x += v[q].x;
-        v[0].y += v[q].y;
+    if (tid / 32 == 1) {
+      const double2 v = sum_bins(reinterpret_cast<const double2*>(S.part), tid & 31);
+      if (tid == 32) {
+        const FwdScalars f = fwd_scalars(S, v.x, v.y);
+        ab = make_float2(f.a_chi, f.b_chi);
+        if (blockIdx.x == 0) finalize_scalars(S, v.x, v.y, false);
       }
-      const FwdScalars f = fwd_scalars(S, v[0].x, v[0].y);
-      ab = make_float2(f.a_chi, f.b_chi);
-      if (blockIdx.x == 0) finalize_scalars(S, v[0].x, v[0].y, false);
     }
   }
   __syncthreads();

@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? 6 : 5)
   // the binning of this forward pass is done: its counters start the next one at zero
   if constexpr (!BWD) clear_bin_counters(S, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
   if constexpr (!BWD && P::HW) {
-    if (blockIdx.x == 0 && blockIdx.y == 0 && tid < kMuSlots)
+    if (blockIdx.x == 0 && blockIdx.y == 0 && tid < kMuCopies * kMuBins)
       reinterpret_cast<double2*>(S.part)[tid] = make_double2(0.0, 0.0);
   }
   // From r = 64 on the splat's spectra (D, C, W~) are only loaded for the
