@@ -370,45 +370,42 @@ bool pdl_enabled() {
 void pdl_suspend(bool off) { t_pdl_off = off; }
 
 // Spectral buffer k: complex (8-byte) elements [x][ky][kz], kz < r/2+1 valid
-// out of a row pitch of r/2+2. tmx: boxes of 16 kz x 1 ky x r x; tmy: boxes
-// of 16 kz x r ky x 1 x. Out-of-range kz reads as zero and is not written.
-int make_tensor_maps(Solve& s, int r) {
+// out of a row pitch of r/2+2; the boxes are listed with Solve. Out-of-range kz
+// reads as zero and is not written. forward_planes: only the maps that a forward
+// pass on the plane path (one CTA a plane) uses, for a caller that makes them
+// anew on every call (7 of 28: 0.5 us, all of them 1.6).
+int make_tensor_maps(Solve& s, int r, bool forward_planes) {
   auto enc = tensor_map_encoder();
   if (!enc) return DPSR_ECUDA;
   const cuuint64_t dims[3] = {(cuuint64_t)(r / 2 + 1), (cuuint64_t)r, (cuuint64_t)r};
   const cuuint64_t strides[2] = {(cuuint64_t)kpitch(r) * 8, (cuuint64_t)r * kpitch(r) * 8};
-  const cuuint32_t cols = (cuuint32_t)tile_cols(r);
-  const cuuint32_t boxx[3] = {cols, 1, (cuuint32_t)tma_rows(r)}, boxy[3] = {cols, (cuuint32_t)tma_rows(r), 1};
-  const CUtensorMapSwizzle swz = cols == 16 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
   const cuuint32_t es[3] = {1, 1, 1};
+  bool ok = true;
+  auto map = [&](CUtensorMap* m, int k, int cols, int ky, int x) {  // map k of m, boxes of cols kz x ky x x
+    const cuuint32_t box[3] = {(cuuint32_t)cols, (cuuint32_t)ky, (cuuint32_t)x};
+    ok = ok && enc(m + k, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, (void*)s.spec[k], dims, strides, box, es,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE,
+                   cols == 16 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  };
+  const int cols = tile_cols(r), rows = tma_rows(r);
+  const bool parts = r >= 64;  // kSkip
+  if (forward_planes) {
+    for (int k : {kSpD, kSpC, kSpW, kSpChi}) map(s.tmw, k, 16, r, 1);
+    for (int k : {kSpD, kSpC})
+      if (parts) map(s.tmc, k, cols, 1, r / kXChunks);
+      else map(s.tmx, k, cols, 1, rows);
+    map(s.tmx, kSpChi, cols, 1, rows);
+    return ok ? DPSR_OK : DPSR_ECUDA;
+  }
   for (int k = 0; k < kNSpec; ++k) {
-    for (int w = 0; w < 2; ++w) {
-      CUresult rc = enc(w == 0 ? &s.tmx[k] : &s.tmy[k], CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3,
-                        (void*)s.spec[k], dims, strides, w == 0 ? boxx : boxy, es,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
-                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-      if (rc != CUDA_SUCCESS) return DPSR_ECUDA;
-    }
+    map(s.tmx, k, cols, 1, rows);
+    map(s.tmy, k, cols, rows, 1);
+    if (r < 256) map(s.tmw, k, 16, r, 1);
+    if (parts) map(s.tmb, k, cols, 16, 1);
+    if (parts && k < 4) map(s.tmc, k, cols, 1, r / kXChunks);
   }
-  if (r < 256) {
-    const cuuint32_t boxw[3] = {16, (cuuint32_t)r, 1};
-    for (int k = 0; k < kNSpec; ++k)
-      if (enc(&s.tmw[k], CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, (void*)s.spec[k], dims, strides, boxw, es,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return DPSR_ECUDA;
-  }
-  if (r < 64) return DPSR_OK;  // kSkip: the parts of tiles below are not used
-  const cuuint32_t boxb[3] = {cols, 16, 1}, boxc[3] = {cols, 1, (cuuint32_t)(r / kXChunks)};
-  for (int k = 0; k < kNSpec + 4; ++k) {
-    const bool b = k < kNSpec;
-    CUresult rc = enc(b ? &s.tmb[k] : &s.tmc[k - kNSpec], CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3,
-                      (void*)s.spec[b ? k : k - kNSpec], dims, strides, b ? boxb : boxc, es,
-                      CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
-                      CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (rc != CUDA_SUCCESS) return DPSR_ECUDA;
-  }
-  return DPSR_OK;
+  return ok ? DPSR_OK : DPSR_ECUDA;
 }
 }  // namespace dpsr
 

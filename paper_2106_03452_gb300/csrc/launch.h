@@ -97,9 +97,9 @@ cudaError_t launch_xpass(bool bwd, int r, const Solve& s, const Solve* tab, int 
                          cudaStream_t st);
 int xpass_blocks(int r);
 
-// TMA descriptors of the four spectral buffers of `s` (s.spec must be set).
-// Returns 0 on success.
-int make_tensor_maps(Solve& s, int r);
+// TMA descriptors of the spectral buffers of `s` (s.spec must be set), all or
+// those of a forward pass on the plane path alone. Returns 0 on success.
+int make_tensor_maps(Solve& s, int r, bool forward_planes = false);
 // Points: x-plane bucketing (count, scan, scatter) and the backward combine.
 cudaError_t launch_bin(const Solve& s, const Solve* tab, int count, int nmax, int r, cudaStream_t st);
 // split: the adjoint kind ran on path kPathSplit (per-channel slots).
