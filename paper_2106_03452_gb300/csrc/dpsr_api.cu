@@ -730,7 +730,7 @@ int dpsr_backward(dpsr_plan p, const float* dchi, float* dpoints, float* dnormal
   run(DPSR_K_PLANE_BFWD, [&] { return run_plane(p, 2, s, st); });
   run(DPSR_K_XPASS_BWD, [&] { return dpsr::launch_xpass(true, r, s, nullptr, 1, st); });
   run(DPSR_K_PLANE_BINV, [&] { return run_plane(p, 3, s, st); });
-  run(DPSR_K_COMBINE, [&] { return dpsr::launch_combine(s, nullptr, 1, s.N, p->C[3] == dpsr::kPathSplit, st); });
+  run(DPSR_K_COMBINE, [&] { return dpsr::launch_combine(s, nullptr, 1, s.N, r, p->C[3] == dpsr::kPathSplit, st); });
   if (e != cudaSuccess) {
     cudaGetLastError();
     return cuda_err(e);

@@ -110,7 +110,7 @@ cudaError_t launch_bwd(dpsr_batch b) {
     cudaError_t e = dpsr::launch_plane(2, c.r, c.C[2], dummy, c.dtab, n, st);
     if (e == cudaSuccess) e = dpsr::launch_xpass(true, c.r, dummy, c.dtab, n, st);
     if (e == cudaSuccess) e = dpsr::launch_plane(3, c.r, c.C[3], dummy, c.dtab, n, st);
-    if (e == cudaSuccess) e = dpsr::launch_combine(dummy, c.dtab, n, c.nmax, c.C[3] == dpsr::kPathSplit, st);
+    if (e == cudaSuccess) e = dpsr::launch_combine(dummy, c.dtab, n, c.nmax, c.r, c.C[3] == dpsr::kPathSplit, st);
     return e;
   });
 }
@@ -223,7 +223,7 @@ cudaError_t tune_batch(dpsr_batch b, bool with_bwd) {
       if (e == cudaSuccess) e = plane(2);
       if (e == cudaSuccess) e = dpsr::launch_xpass(true, c.r, dummy, c.dtab, n, st);
       if (e == cudaSuccess) e = plane(3);
-      if (e == cudaSuccess) e = dpsr::launch_combine(dummy, c.dtab, n, c.nmax, c.C[3] == dpsr::kPathSplit, st);
+      if (e == cudaSuccess) e = dpsr::launch_combine(dummy, c.dtab, n, c.nmax, c.r, c.C[3] == dpsr::kPathSplit, st);
     }
   }
   if (e0) cudaEventDestroy(e0);
@@ -507,7 +507,7 @@ int dpsr_internal_batch_run(dpsr_batch b, int k, int with_bwd) {
     if (e == cudaSuccess) e = dpsr::launch_plane(2, c.r, c.C[2], dummy, c.dtab, k, st);
     if (e == cudaSuccess) e = dpsr::launch_xpass(true, c.r, dummy, c.dtab, k, st);
     if (e == cudaSuccess) e = dpsr::launch_plane(3, c.r, c.C[3], dummy, c.dtab, k, st);
-    if (e == cudaSuccess) e = dpsr::launch_combine(dummy, c.dtab, k, c.nmax, c.C[3] == dpsr::kPathSplit, st);
+    if (e == cudaSuccess) e = dpsr::launch_combine(dummy, c.dtab, k, c.nmax, c.r, c.C[3] == dpsr::kPathSplit, st);
   }
   if (e != cudaSuccess) return failed(b);
   b->have_fwd = true;

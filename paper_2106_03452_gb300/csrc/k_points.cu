@@ -250,11 +250,17 @@ __global__ void __launch_bounds__(256) k_combine(const __grid_constant__ Solve s
   }
 }
 
-cudaError_t launch_combine(const Solve& s, const Solve* tab, int count, int nmax, bool split,
+cudaError_t launch_combine(const Solve& s, const Solve* tab, int count, int nmax, int r, bool split,
                            cudaStream_t st) {
+  // Early for single solves below r = 128, where the points' reads through L1 are
+  // few and the gap costs more: layer of 1 000 points at r = 8 58.9 us early, 60.5
+  // after; 3 000 at r = 16 66.7 and 67.9 (alone 77.5 and 80.0); 20 000 at r = 32
+  // 120.0 and 121.6. From r = 128 on after: 20 000 points 112.4 early, 108.4 after;
+  // and in batches: four of r = 32 with 3 000 points 77.5 early, 75.7 after.
+  const bool early = r < 128 && !tab;
   const int blocks = min(max((nmax + 255) / 256, 1), 1184);
-  return split ? launch_after(k_combine<true>, dim3(blocks, 1, count), dim3(256), 0, st, 0, s, tab)
-               : launch_after(k_combine<false>, dim3(blocks, 1, count), dim3(256), 0, st, 0, s, tab);
+  return split ? launch_at(early, k_combine<true>, dim3(blocks, 1, count), dim3(256), 0, st, 0, s, tab)
+               : launch_at(early, k_combine<false>, dim3(blocks, 1, count), dim3(256), 0, st, 0, s, tab);
 }
 
 // ---------------------------------------------------------------------------

@@ -103,7 +103,7 @@ int make_tensor_maps(Solve& s, int r, bool forward_planes = false);
 // Points: x-plane bucketing (count, scan, scatter) and the backward combine.
 cudaError_t launch_bin(const Solve& s, const Solve* tab, int count, int nmax, int r, cudaStream_t st);
 // split: the adjoint kind ran on path kPathSplit (per-channel slots).
-cudaError_t launch_combine(const Solve& s, const Solve* tab, int count, int nmax, bool split,
+cudaError_t launch_combine(const Solve& s, const Solve* tab, int count, int nmax, int r, bool split,
                            cudaStream_t st);
 
 // Trilinear lookup of a grid at query points and its adjoint (atomic adds).
