@@ -1149,11 +1149,19 @@ static cudaError_t launch_plane_t(int kind, const Solve& s, const Solve* tab, in
   }
   if (kind == 3) block = dim3(binv_threads<L, C>());
   // The transforms from points and from dchi with fewer CTAs than the GPU has SMs
-  // (152) start when the previous kernel has left: launched early they crowd onto
-  // the SMs that empty first, two to one, while others stay idle. r = 32, 200 000
-  // points: the layer 1 074 us early, 950 after; 60 000: 362 and 319; forward of
-  // 3 000: 37.4 and 38.5. The inverse kinds gain nothing by it.
-  const bool crowds = kind % 2 == 0 && L * C * count < 152;
+  // (152) crowd onto the SMs that empty first, two to one, when they are launched
+  // early, while others stay idle. That of dchi, behind a pass that fills the GPU,
+  // starts when the previous kernel has left (layer of 20 000 points at r = 64: 83.5
+  // us early, 73.6 after; 3 000: 65.4 and 60.2). That from points follows the
+  // binning, which leaves SMs free, and starts late only where a plane's points
+  // take longer than the gap: forward at r = 32, in a row and alone, 3 000 points
+  // 36.8 and 46.4 us early, 38.3 and 49.6 after; 20 000: 81.3 and 90.0, 82.2 and
+  // 93.4; 60 000: 202.5 and 206.1, 196.2 and 207.3; 200 000: 630 and 660, 587 and
+  // 600. (At r = 128 with a CTA a plane early at any number: 200 000 points 176.6
+  // and 187.9, 178.9 and 190.0; in a batch, whose kernels know no N, the two are
+  // equal.) The inverse kinds gain nothing by a late start.
+  const bool few = L * C * count < 152;
+  const bool crowds = few && (kind == 2 || (kind == 0 && L <= 64 && s.N >= 30000));
   return launch_at(!crowds, fn, dim3(L * C, 1, count), block, smem, st, C, s, tab);
 }
 
