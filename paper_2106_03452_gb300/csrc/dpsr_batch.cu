@@ -133,7 +133,7 @@ cudaError_t tune_kind(BatchClass& c, int kind, cudaStream_t st, cudaEvent_t e0, 
     const int C = forced >= 0 ? forced : c.C[kind];
     const cudaError_t e = dpsr::launch_plane(kind, c.r, C, dummy, c.dtab, n, st);
     if (e != cudaSuccess) return e;  // a path that does not exist: not kept
-    if (c.r < 256) c.C[kind] = C;
+    c.C[kind] = c.r < 256 ? C : 0;  // the pencil passes, whichever accepted size asked for them
     c.tuned[kind] = true;
     return e;
   }

@@ -1,4 +1,4 @@
-"""Batches whose launches are refused."""
+"""Batches of large grids against solo solves, and batches whose launches are refused."""
 import numpy as np
 import pytest
 
@@ -68,4 +68,27 @@ def test_a_refused_run_leaves_the_batch_usable(monkeypatch):
         b.run(graph=graph)
         assert b.sync() == 0
         _agree(io, rs)
+    b.close()
+
+
+@pytest.mark.parametrize("path", [None, "4"])
+def test_large_grids_in_a_batch(monkeypatch, path):
+    """r = 256 and 512 in one batch, their Solve read from the device table: the
+    solo solves' results by plain launches, capture and replay, the paths and
+    launches that ran (the pencil passes, asked for by a cluster size or not)."""
+    if path:
+        monkeypatch.setenv("DPSR_PLANE_PATH", path)
+    else:
+        monkeypatch.delenv("DPSR_PLANE_PATH", raising=False)
+    rs = [256, 512, 256] if path is None else [256, 256]  # no cluster size is accepted at r = 512
+    b, io = _batch(rs, [20000, 30000, 700][:len(rs)], seed=1)
+    for graph in (False, True, True):
+        for t in io:
+            for x in t[3:]:
+                x.fill_(float("nan"))
+        b.run(graph=graph)
+        assert b.sync() == 0
+        _agree(io, rs)
+    assert all(list(b.paths(r)) == [0] * 4 for r in set(rs))
+    assert b.launches(False) == len(set(rs)) * 7 and b.launches() == len(set(rs)) * 13
     b.close()
