@@ -10,6 +10,7 @@ from __future__ import annotations
 import ctypes
 import os
 import threading
+import warnings
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 # DPSR_DEBUG_CHECKS=1 in the environment loads the bounds-checking build
@@ -132,25 +133,46 @@ def load():
     return _lib
 
 
+class _NoBinding:
+    """Stands in for the binding: every entry leaves the call to the Python classes."""
+
+    def __getattr__(self, name):
+        return lambda *args: None
+
+
+def _load_binding():
+    import importlib.util
+    import torch
+    if not os.path.exists(BIND_PATH):
+        raise ImportError(f"{BIND_PATH} is missing")
+    stamp = BIND_PATH + ".stamp"
+    built = open(stamp).readline().strip() if os.path.exists(stamp) else "another version"
+    if built != torch.__version__:
+        raise ImportError(f"{BIND_PATH} was built for PyTorch {built}, this is {torch.__version__}")
+    spec = importlib.util.spec_from_file_location("_dpsr_torch", BIND_PATH)
+    mod = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(mod)
+    mod.init(DPSRError)
+    return mod
+
+
 def binding():
     """The in-tree PyTorch binding (csrc/torch_bind.cpp): the hot calls on
     plain CUDA tensors without Python on the way. Its entries return None for
-    anything else. Raises if it has not been built."""
+    anything else. Where it is missing, or was built for another PyTorch, the
+    Python classes answer every call, after one warning."""
     global _bind
     if _bind is None:
         load()
         with _lock:
             if _bind is None:
-                if not os.path.exists(BIND_PATH):
-                    raise RuntimeError(f"the PyTorch binding is not built ({BIND_PATH} missing): run "
-                                       f"`python -m paper_2106_03452_gb300.build{' --debug' if _DEBUG else ''}`")
-                import importlib.util
-                import torch  # noqa: F401  (its libraries first)
-                spec = importlib.util.spec_from_file_location("_dpsr_torch", BIND_PATH)
-                mod = importlib.util.module_from_spec(spec)
-                spec.loader.exec_module(mod)
-                mod.init(DPSRError)
-                _bind = mod
+                try:
+                    _bind = _load_binding()
+                except ImportError as e:
+                    warnings.warn(f"no PyTorch binding, calls go through Python: {e}; run "
+                                  f"`python -m paper_2106_03452_gb300.build{' --debug' if _DEBUG else ''}`",
+                                  RuntimeWarning, stacklevel=3)
+                    _bind = _NoBinding()
     return _bind
 
 
