@@ -802,9 +802,9 @@ int dpsr_get_loss(dpsr_plan p, double* loss) {
 static void finish_w(int r, const unsigned* occ, std::complex<float>* w) {
   typedef std::complex<double> Cd;
   const int h = r / 2, nyb = dpsr::nybins(r), yb = r / nyb;
-  std::vector<Cd> tw(r), a(r), b(r);
+  Cd tw[512], a[512], b[512];  // no allocation: nothing to throw across the C entry
   for (int k = 0; k < r; ++k) tw[k] = std::polar(1.0, -2.0 * M_PI * k / r);
-  auto fft = [&](std::vector<Cd>& v) {  // radix 2, in order
+  auto fft = [&](Cd* v) {  // radix 2, in order
     for (int i = 1, j = 0; i < r; ++i) {
       int bit = r >> 1;
       for (; j & bit; bit >>= 1) j ^= bit;
@@ -852,13 +852,13 @@ int dpsr_debug_read_spectrum(dpsr_plan p, int which, void* out_host) {
     return DPSR_ECUDA;
   }
   if (half) {
-    std::vector<unsigned> occ(r);
-    if (cudaMemcpy(occ.data(), dpsr::occ_words(p->s.bins, r), sizeof(unsigned) * r, cudaMemcpyDeviceToHost) !=
+    unsigned occ[512];
+    if (cudaMemcpy(occ, dpsr::occ_words(p->s.bins, r), sizeof(unsigned) * r, cudaMemcpyDeviceToHost) !=
         cudaSuccess) {
       cudaGetLastError();
       return DPSR_ECUDA;
     }
-    finish_w(r, occ.data(), (std::complex<float>*)out_host);
+    finish_w(r, occ, (std::complex<float>*)out_host);
   } else if (which < 3 && r >= 64) {  // the splat's spectra are zero, and not stored, in x-chunks without points
     unsigned chunks = 0;
     if (cudaMemcpy(&chunks, dpsr::occ_words(p->s.bins, r) + r, sizeof(unsigned), cudaMemcpyDeviceToHost) !=
