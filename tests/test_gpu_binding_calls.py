@@ -1,5 +1,5 @@
 """How the C++ entries of the hot calls sit in a Python program: what other
-threads may do meanwhile, subclasses of the classes that call them."""
+threads may do meanwhile, subclasses of the classes that call them, streams."""
 import threading
 import time
 
@@ -118,4 +118,62 @@ def test_subclasses_answer_for_themselves():
         out = zeros(fn, k).apply(x, *rest)
         (g,) = torch.autograd.grad((out[0] if isinstance(out, tuple) else out).sum(), x)
         assert not g.any(), fn
+    plan.close()
+
+
+@pytest.mark.parametrize("r", [32, 64, 256])
+def test_a_side_stream_waits_for_its_own_inputs(r):
+    """The inputs are written on a side stream, behind a long kernel, right before
+    the call: work on any other stream would read what was there before. The
+    upstream gradient is random: the layer is well conditioned then, and two solves
+    of one cloud differ by some 5e-7 of the largest value (their splats' sums run
+    in no fixed order), where chi.square().sum() turns the same rounding into 1e-4."""
+    import torch
+    from paper_2106_03452_gb300.dpsr import Plan, dpsr
+    from paper_2106_03452_gb300.optimize import chamfer
+    (p, n), (p0, n0) = _cloud(3000, 1), _cloud(3000, 2)
+    w = torch.randn((r, r, r), device="cuda", generator=torch.Generator("cuda").manual_seed(r))
+    plan = Plan(r, 2.0)
+
+    def step(a, b, g, q):
+        chi = dpsr(a, b, plan)
+        return [chi.detach(), *torch.autograd.grad(chi, (a, b), g), *torch.autograd.grad(chamfer(a, q), a)]
+
+    def inputs(p, n, w, q):
+        return p.clone().requires_grad_(True), n.clone().requires_grad_(True), w.clone(), q.clone()
+
+    want = step(*inputs(p, n, w, p0))
+    late = inputs(p0, n0, torch.zeros_like(w), p)
+    other = step(*inputs(p0, n0, w, p))
+    st = torch.cuda.Stream()
+    st.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(st):
+        torch.cuda._sleep(100_000_000)  # some 50 ms
+        with torch.no_grad():
+            for x, y in zip(late, (p, n, w, p0)):
+                x.copy_(y)
+        got = step(*late)
+    torch.cuda.current_stream().wait_stream(st)
+    for x, y, z in zip(got, want, other):
+        scale = float(y.abs().max())
+        assert float((x - y).abs().max()) <= 1e-5 * scale
+        assert float((z - y).abs().max()) >= 1e-2 * scale  # the inputs before would have shown
+    plan.close()
+
+
+def test_a_plan_without_a_name_answers_as_another():
+    """The graph keeps a plan that went out of scope; with a random upstream
+    gradient (see above)."""
+    import gc
+    import torch
+    from paper_2106_03452_gb300.dpsr import Plan, dpsr
+    p, n = _cloud()
+    w = torch.randn((32, 32, 32), device="cuda")
+    a = p.clone().requires_grad_(True)
+    plan = Plan(32, 2.0)
+    (want,) = torch.autograd.grad(dpsr(a, n, plan), a, w)
+    chi = dpsr(a, n, Plan(32, 2.0))
+    gc.collect()
+    (got,) = torch.autograd.grad(chi, a, w)
+    assert float((got - want).abs().max()) <= 1e-5 * float(want.abs().max())
     plan.close()
