@@ -347,10 +347,10 @@ struct Scalars {
   float c_mu;             // backward: weight of the stored lookup gradient
   double loss;            // L_DPSR of Eq. 9 (mean squared error against a target grid)
   int bparts;             // partial sums that the backward x pass has yet to turn into the above (0: done)
-  // arrival counters of the last-block reductions: [1] backward plane pass,
-  // [2] the L_DPSR loss (reset by the binning's scatter of every forward, and
-  // each by its own last block)
-  unsigned ticket[3];
+  // arrival counters of the last-block reductions: [0] backward z pass, [1] the
+  // L_DPSR loss (reset by the binning's scatter of every forward, and each by
+  // its own last block)
+  unsigned ticket[2];
 };
 
 // Spectral buffers of a solve (Solve::spec) and what they hold between the
@@ -368,13 +368,14 @@ constexpr int kSpD = 0, kSpChi = 1, kSpC = 2, kSpW = 3, kSpYa = 4, kSpYb = 5;
 constexpr int kNSpec = 6;
 
 struct Solve {
-  // TMA descriptors of the spectral buffers (dims kz = r/2+1, ky, x): tmx
-  // boxes are 16 kz x 1 ky x r x (x-pass tiles), tmy boxes 16 kz x r ky x
-  // 1 x (plane tiles). 128-byte swizzle.
+  // TMA descriptors of the spectral buffers (dims kz = r/2+1, ky, x), with
+  // c = tile_cols(r) columns of kz: tmx boxes are c kz x 1 ky x r x (x-pass
+  // tiles), tmy boxes c kz x r ky x 1 x (y-pass tiles; both 256 rows at r =
+  // 512). Swizzle of 128 bytes for 16 columns, 64 for 8.
   CUtensorMap tmx[kNSpec];
   CUtensorMap tmy[kNSpec];
   // and in parts, for tiles that hold no points in places (kSkip): tmb boxes
-  // of 16 kz x 16 ky x 1 x (a y-block), tmc boxes of 16 kz x 1 ky x r/8 x (an
+  // of c kz x 16 ky x 1 x (a y-block), tmc boxes of c kz x 1 ky x r/8 x (an
   // x-chunk, forward buffers only)
   CUtensorMap tmb[kNSpec];
   CUtensorMap tmw[kNSpec];  // as tmy, 16 columns (the plane kernels, below r = 256)
@@ -417,7 +418,10 @@ struct Solve {
 };
 
 // Threads of a group FFT (Shape<r>::T), for the host.
-inline int group_threads(int r) { return r <= 16 ? 1 : (r == 32 ? 4 : (r <= 128 ? 8 : 16)); }
+constexpr int group_threads(int r) { return r <= 16 ? 1 : (r == 32 ? 4 : (r <= 128 ? 8 : 16)); }
+static_assert(group_threads(8) == Shape<8>::T && group_threads(16) == Shape<16>::T && group_threads(32) == Shape<32>::T &&
+              group_threads(64) == Shape<64>::T && group_threads(128) == Shape<128>::T &&
+              group_threads(256) == Shape<256>::T && group_threads(512) == Shape<512>::T, "one table");
 
 // Host side: the spectral tables of one plan, computed in FP64 and rounded
 // to FP32. tw[r]: twiddles exp(-2 pi i t k1 / r) at k1 T + t; tab[7r]: g1 (r), u2 (3r) and

@@ -332,7 +332,7 @@ __global__ void __launch_bounds__(ZfGeo<L>::NT, ZfGeo<L>::MINB) k_zfwd(const __g
 }
 
 // ===========================================================================
-// Forward y pass over 16 kz columns of plane X, by CTA kind (blockIdx.y):
+// Forward y pass over 16 (8) kz columns of plane X, by CTA kind (blockIdx.y):
 // 0: D = FFT(i u_z v_z) + i u_y FFT(v_y) from buffers 0 and 1 into kSpD;
 // 1: C = FFT(v_x) in place in kSpC; 2 (not with kHalfW): W~ = FFT(w) in place
 // in kSpW. BWD: FFT of the z-transformed dchi in place in kSpD, with kHalfW of
@@ -545,18 +545,17 @@ __global__ void __launch_bounds__(ynt<L>(), L == 256 ? 6 : (L >= 256 ? 3 : (BWD 
 }
 
 // ===========================================================================
-// Inverse y pass over 16 kz columns of plane X, out of place (the pass can
-// run again on the same inputs). NCH = 1: chi~ (kSpChi) -> kSpYa. NCH = 3:
-// the adjoint fields V_bar_x = IFFT_y(Q2) -> kSpC, V_bar_y = IFFT_y(-i u_y
-// Q1) -> kSpYa, V_bar_z = -i u_z IFFT_y(Q1) -> kSpYb, with Q1 in kSpD and
-// Q2 in kSpChi. Below r = 256 (yinv_split) the adjoint fields take two CTA
-// kinds (blockIdx.y): 0: V_bar_x from Q2; 1: V_bar_y and V_bar_z from Q1.
-// There the pass is bound by each CTA's latency and shorter CTAs win; at
-// r = 256, bound by bandwidth, one CTA does all three.
+// Inverse y pass over 16 (8) kz columns of plane X, out of place (the pass can
+// run again on the same inputs). NCH = 1: chi~ (kSpChi) -> kSpYa. NCH = 3
+// (below r = 64; k_yadj above): the adjoint fields V_bar_x = IFFT_y(Q2) -> kSpC,
+// V_bar_y = IFFT_y(-i u_y Q1) -> kSpYa, V_bar_z = -i u_z IFFT_y(Q1) -> kSpYb,
+// with Q1 in kSpD and Q2 in kSpChi, by two CTA kinds (blockIdx.y): 0: V_bar_x
+// from Q2; 1: V_bar_y and V_bar_z from Q1. The pass is bound by each CTA's
+// latency there, and shorter CTAs win.
 // ===========================================================================
 template <int L, int NCH>
 constexpr int yinv_boxes() {
-  return NCH == 1 && kHalfW<L> ? 2 : NCH;
+  return NCH == 3 || kHalfW<L> ? 2 : 1;
 }
 
 template <int L, int NCH>
@@ -564,26 +563,22 @@ constexpr size_t yinv_smem() {
   return box_align<L>() + sizeof(float2) * ((size_t)yinv_boxes<L, NCH>() * Pen<L>::BOX + ColFft<L>::TWN) + sizeof(float) * L;
 }
 
-// Thread 0: the TMA tile loads of an inverse y-pass tile (part: -1 all
-// fields, else the CTA kind of yinv_split), completion on `bar`.
-template <int L, int NCH>
-__device__ __forceinline__ void yinv_issue(const Solve& S, int X, int kz0, int part, float2* box,
+// Thread 0: the TMA loads of an inverse y-pass tile into box 0 (of CTA kind
+// `kind`: 0 chi~ or Q2, 1 Q1), completion on `bar`, which also awaits `more`
+// bytes.
+template <int L>
+__device__ __forceinline__ void yinv_issue(const Solve& S, int X, int kz0, int kind, float2* box,
                                            uint64_t* bar, uint32_t more = 0u) {
   using P = Pen<L>;
-  // NCH = 1: box 0 <- chi~; NCH = 3: box 0 <- Q2, box 1 <- Q1 (split: only
-  // the kind's own input)
-  const bool do0 = part != 1, do1 = NCH == 3 && part != 0;
-  mbar_expect_tx(bar, ((do0 ? 1 : 0) + (do1 ? 1 : 0)) * P::BOX * (uint32_t)sizeof(float2) + more);
-  for (int y = 0; y < L; y += tma_rows(L)) {
-    if (do0) tma_load_3d(box + y * P::W, &S.tmy[kSpChi], kz0, y, X, bar);
-    if (do1) tma_load_3d(box + P::BOX + y * P::W, &S.tmy[kSpD], kz0, y, X, bar);
-  }
+  mbar_expect_tx(bar, P::BOX * (uint32_t)sizeof(float2) + more);
+  for (int y = 0; y < L; y += tma_rows(L))
+    tma_load_3d(box + y * P::W, &S.tmy[kind ? kSpD : kSpChi], kz0, y, X, bar);
 }
 
 // All threads: wait, transform, TMA stores (thread 0 waits until they have
 // read shared memory). False if the bounded wait gave up.
 template <int L, int NCH>
-__device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int part, float2* box,
+__device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int kind, float2* box,
                                           const float2* twt, const float* iu, uint64_t* bar,
                                           uint32_t phase, unsigned rows = 0u) {
   using P = Pen<L>;
@@ -591,33 +586,30 @@ __device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int pa
   using F = ColFft<L>;
   const int tid = threadIdx.x, g = F::LN::group(tid), t = F::LN::lane(tid);
   float am = 0.f, as = 0.f;  // this thread's share of the sums of Eq. 4 (kHalfW)
-  constexpr int NIN = NCH == 1 ? 1 : 2;
-  const bool do0 = part != 1, do1 = NCH == 3 && part != 0;
+  const bool second = NCH == 3 && kind == 1;  // Q1 and its two fields
   const bool landed = __syncthreads_and(mbar_wait(bar, phase));
   if (!landed) {
     if (tid == 0) atomicOr(S.status, kStTimeout);
     mbar_wait(bar, phase);
     return false;
   }
-  if (kz0 == 0 && g < NIN && (g == 0 ? do0 : do1)) {
+  if (kz0 == 0 && g == 0) {
     // column 0 becomes X0 + i Xn (Xn: the Nyquist column); the same lanes
     // read these elements again below
-    float2* b = box + g * P::BOX;
-    const float2* nq = S.spec[g == 0 ? kSpChi : kSpD] + (size_t)X * L * P::KP + H;
+    const float2* nq = S.spec[second ? kSpD : kSpChi] + (size_t)X * L * P::KP + H;
     for (int j = 0; j < F::R1; ++j) {
       const int ky = t + F::T * j;
-      const float2 n = H >= 16 ? nq[(size_t)ky * P::KP] : b[bxl<L>(ky, H)];
-      const float2 x0 = b[bxl<L>(ky, 0)];
-      b[bxl<L>(ky, 0)] = make_float2(x0.x - n.y, x0.y + n.x);
+      const float2 n = H >= 16 ? nq[(size_t)ky * P::KP] : box[bxl<L>(ky, H)];
+      const float2 x0 = box[bxl<L>(ky, 0)];
+      box[bxl<L>(ky, 0)] = make_float2(x0.x - n.y, x0.y + n.x);
     }
   }
   __syncthreads();
   if (g < P::NCOL) {
     const int sz = kz0 + g;
-    auto cref = [&](int k) { return typename F::CL(box + k * P::BOX, t, g); };
     float2 v[F::R1];
-    const auto c0 = cref(0);
-    if (do0) {
+    const typename F::CL c0(box, t, g);
+    if (!second) {
 #pragma unroll
       for (int j = 0; j < F::R1; ++j) v[j] = c0.get(j);
       F::template run<+1>(v, c0, twt, t);
@@ -641,25 +633,26 @@ __device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int pa
         if (X == 0 && t == 0) as = sz == 0 ? v[0].x + v[0].y : 2.f * v[0].x;  // chi'(0) = sum over kz at x = y = 0
       }
     }
-    if (do1) {
-      const auto c1 = cref(1);
-      const auto c2 = cref(2);
+    if constexpr (NCH == 3) {
+      if (second) {  // V_bar_y in box 0, V_bar_z in box 1
+        const typename F::CL c1(box + P::BOX, t, g);
 #pragma unroll
-      for (int j = 0; j < F::R1; ++j) {
-        v[j] = c1.get(j);
-        c2.put(j, v[j]);
-        v[j] = cmul_iu(v[j], -iu[t + F::T * j]);
+        for (int j = 0; j < F::R1; ++j) {
+          v[j] = c0.get(j);
+          c1.put(j, v[j]);
+          v[j] = cmul_iu(v[j], -iu[t + F::T * j]);
+        }
+        F::template run<+1>(v, c0, twt, t);
+#pragma unroll
+        for (int j = 0; j < F::R1; ++j) c0.put(j, v[j]);
+        F::sync();
+#pragma unroll
+        for (int j = 0; j < F::R1; ++j) v[j] = c1.get(j);
+        F::template run<+1>(v, c1, twt, t);
+        const float ez = sz == 0 ? 0.f : -__ldg(S.iu + 2 * L + sz);  // z axis
+#pragma unroll
+        for (int j = 0; j < F::R1; ++j) c1.put(j, cmul_iu(v[j], ez));
       }
-      F::template run<+1>(v, c1, twt, t);
-#pragma unroll
-      for (int j = 0; j < F::R1; ++j) c1.put(j, v[j]);
-      F::sync();
-#pragma unroll
-      for (int j = 0; j < F::R1; ++j) v[j] = c2.get(j);
-      F::template run<+1>(v, c2, twt, t);
-      const float ez = sz == 0 ? 0.f : -__ldg(S.iu + 2 * L + sz);  // z axis
-#pragma unroll
-      for (int j = 0; j < F::R1; ++j) c2.put(j, cmul_iu(v[j], ez));
     }
   }
   fence_async_smem();
@@ -682,16 +675,10 @@ __device__ __forceinline__ bool yinv_tile(const Solve& S, int X, int kz0, int pa
     return true;
   }
   if (tid == 0) {
+    const int out = NCH == 1 || second ? kSpYa : kSpC;
     for (int y = 0; y < L; y += tma_rows(L)) {
-      if constexpr (NCH == 1) {
-        tma_store_3d(&S.tmy[kSpYa], kz0, y, X, box + y * P::W);
-      } else {
-        if (do0) tma_store_3d(&S.tmy[kSpC], kz0, y, X, box + y * P::W);
-        if (do1) {
-          tma_store_3d(&S.tmy[kSpYa], kz0, y, X, box + P::BOX + y * P::W);
-          tma_store_3d(&S.tmy[kSpYb], kz0, y, X, box + 2 * P::BOX + y * P::W);
-        }
-      }
+      tma_store_3d(&S.tmy[out], kz0, y, X, box + y * P::W);
+      if (second) tma_store_3d(&S.tmy[kSpYb], kz0, y, X, box + P::BOX + y * P::W);
     }
     tma_store_commit();
     tma_store_wait_read();
@@ -727,21 +714,21 @@ __global__ void __launch_bounds__(ynt<L>(), L == 256 ? 6 : (L >= 512 ? 3 : 4))
     if (tid == 0) finalize_scalars(S, ff_to_double(x), ff_to_double(y), false);
     return;
   }
-  const int part = NCH == 3 ? (int)blockIdx.y : -1;
+  const int kind = NCH == 3 ? (int)blockIdx.y : 0;
   unsigned rows = 0u;
   if constexpr (NCH == 1 && kHalfW<L>) {
     rows = reach_mask(tile_mask(S, L, X), P::NYB);
-    if (tid == 0) yinv_issue<L, NCH>(S, X, kz0, part, box, &bar, w_bytes<L>(rows));
+    if (tid == 0) yinv_issue<L>(S, X, kz0, kind, box, &bar, w_bytes<L>(rows));
     if (tid < 32) w_issue<L>(S, X, kz0, rows, box + P::BOX, &bar);
   } else if (tid == 0) {
-    yinv_issue<L, NCH>(S, X, kz0, part, box, &bar);
+    yinv_issue<L>(S, X, kz0, kind, box, &bar);
   }
   for (int i = tid; i < L; i += NT) {
     twt[ColFft<L>::tw_at(i)] = S.tw[i];
     iu[i] = S.iu[L + i];  // y axis
   }
   __syncthreads();
-  yinv_tile<L, NCH>(S, X, kz0, part, box, twt, iu, &bar, 0, rows);
+  yinv_tile<L, NCH>(S, X, kz0, kind, box, twt, iu, &bar, 0, rows);
 }
 
 // ===========================================================================
@@ -1232,7 +1219,7 @@ __global__ void __launch_bounds__(ZbGeo<L>::NT, L >= 512 ? 1 : 3) k_zbfwd(const 
   }
   // this CTA's partial sums, fixed order; the last CTA finalises
   block_sum_ff<NT>(dS, dD);
-  last_block_finalize<NT>(S, 1, (int)gridDim.x, (int)blockIdx.x, dS, dD, true);
+  last_block_finalize<NT>(S, 0, (int)gridDim.x, (int)blockIdx.x, dS, dD, true);
 }
 
 // ---------------------------------------------------------------------------

@@ -141,7 +141,6 @@ __global__ void __launch_bounds__(NT) k_bin_scatter(const __grid_constant__ Solv
       off[nb] = total;
       S.sc->ticket[0] = 0;
       S.sc->ticket[1] = 0;
-      S.sc->ticket[2] = 0;
     }
   }
   const double sx = S.gscale[0], sy = S.gscale[1], sz = S.gscale[2];
@@ -347,7 +346,7 @@ __global__ void __launch_bounds__(256) k_mse_grad(const __grid_constant__ Solve 
   if (threadIdx.x == 0) {
     S.part[blockIdx.x] = make_float4(acc.hi, acc.lo, 0.f, 0.f);
     __threadfence();
-    last = atomicAdd(&S.sc->ticket[2], 1u) == (unsigned)nblk - 1u ? 1u : 0u;
+    last = atomicAdd(&S.sc->ticket[1], 1u) == (unsigned)nblk - 1u ? 1u : 0u;
     if (last) __threadfence();
   }
   __syncthreads();
@@ -360,7 +359,7 @@ __global__ void __launch_bounds__(256) k_mse_grad(const __grid_constant__ Solve 
   block_sum_ff<NT>(x, y);
   if (threadIdx.x == 0) {
     S.sc->loss = ff_to_double(x) / ((double)S.r * S.r * S.r);
-    S.sc->ticket[2] = 0;
+    S.sc->ticket[1] = 0;
   }
 }
 

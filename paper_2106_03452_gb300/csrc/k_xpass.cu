@@ -36,8 +36,7 @@ struct XGeo {
   // W~'s tile. From r = 256 on W~ has no part in the x passes (kHalfW).
   static constexpr bool HW = kHalfW<L>;
   static constexpr bool TIGHT = L == 256;
-  template <bool BWD>
-  static constexpr int nch() { return 2; }
+  static constexpr int NCH = 2;
 };
 
 // G(k) = g(k) / (-2 pi |u|^2) with g separable: g1[kx] * (g1[ky] g1[kz]);
@@ -52,7 +51,7 @@ __device__ __forceinline__ float spectral_G(int kx, float gyz, float u2yz, const
 template <int L, bool BWD>
 constexpr size_t xpass_smem() {
   using P = XGeo<L>;
-  constexpr int NCH = P::template nch<BWD>();
+  constexpr int NCH = P::NCH;
   // r = 256: the boxes at the start of an allocation aligned for them, and no
   // static shared memory (the barriers lie in the twiddles of k1 = 0, which are
   // one and not read): six CTAs an SM to the byte instead of five, forward 52.4 ->
@@ -68,7 +67,7 @@ template <int L, bool BWD>
 __global__ void __launch_bounds__(XGeo<L>::NT, L >= 512 ? 3 : (L >= 256 ? 6 : 5))
     k_xpass(const __grid_constant__ Solve s0, const Solve* __restrict__ tab) {
   using P = XGeo<L>;
-  constexpr int NCH = P::template nch<BWD>();
+  constexpr int NCH = P::NCH;
   const Solve& S = tab ? tab[blockIdx.z] : s0;
   const int kz0 = blockIdx.x * P::KC, ky = blockIdx.y;
   using F = ColFft<L>;

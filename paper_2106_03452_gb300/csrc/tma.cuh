@@ -19,8 +19,8 @@ __device__ __forceinline__ int bx(int q, int c) {
   return q * 16 + ((((c >> 1) ^ (q & 7)) << 1) | (c & 1));
 }
 
-// The same for a box of tile_cols(L) columns: 8 columns (64-byte rows) at
-// L = 512 under the 64-byte swizzle (chunks XOR-ed by bits 1-2 of the row).
+// The same for a box of tile_cols(L) columns: 8 columns (64-byte rows) from
+// L = 256 on, under the 64-byte swizzle (chunks XOR-ed by bits 1-2 of the row).
 template <int L>
 __device__ __forceinline__ int bxl(int q, int c) {
   if constexpr (tile_cols(L) == 16) return bx(q, c);
