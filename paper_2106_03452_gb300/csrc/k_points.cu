@@ -311,9 +311,11 @@ __global__ void __launch_bounds__(256) k_grid_splat(float* __restrict__ grid, in
 // block to arrive writes sc->loss), deterministic. n = r^3 is a power of two, so
 // 2/n and 1/n are exact.
 // ---------------------------------------------------------------------------
-// float4 of each grid per thread. Every block costs a ticket (a fence and an
-// atomic on its instance's counter): a batch's two classes 45.4 us with 2, 40.9 with 8.
-constexpr int kMsePer = 8;
+// float4 of each grid per thread: 8 where that leaves two blocks to an SM, for
+// every block costs a ticket (a fence and an atomic on its instance's counter): a
+// batch's two classes 45.4 us with 2, 40.9 with 8. Fewer blocks leave SMs idle: one
+// grid of r = 32 takes 5.3 us with 2 and 6.7 with 8, one of r = 64 5.6 and 6.9.
+constexpr int kMsePer = 8, kMseFew = 2;
 __global__ void __launch_bounds__(256) k_mse_grad(const __grid_constant__ Solve s0,
                                                   const Solve* __restrict__ tab) {
   constexpr int NT = 256;
@@ -325,9 +327,7 @@ __global__ void __launch_bounds__(256) k_mse_grad(const __grid_constant__ Solve 
   const float4* chi = reinterpret_cast<const float4*>(S.chi);
   const float4* tg = reinterpret_cast<const float4*>(S.target);
   float4* g = reinterpret_cast<float4*>(S.dchi_rw);
-  // this instance's blocks (a batch launch sizes the grid for its largest r)
-  const int nblk = (int)min((int64_t)gridDim.x, max(n4 / (kMsePer * NT), (int64_t)1));
-  if ((int)blockIdx.x >= nblk) return;
+  const int nblk = (int)gridDim.x;  // a launch's instances are of one size
   FF acc = {0.f, 0.f}, z = acc;
   auto squares = [&](int64_t i) {
     const float4 a = __ldcs(chi + i), b = __ldcs(tg + i);
@@ -363,16 +363,16 @@ __global__ void __launch_bounds__(256) k_mse_grad(const __grid_constant__ Solve 
   }
 }
 
-// Blocks of the loss pass for grid size r: kMsePer float4 per thread, at most
-// the r * 16 block partials the workspace holds.
-int mse_blocks(int r) {
+// Blocks of the loss pass for `count` grids of size r, for each: at most the
+// r * 16 partial sums that the workspace holds.
+static int mse_blocks(int r, int count) {
   const int64_t n4 = (int64_t)r * r * r / 4;
-  const int64_t b = n4 / (kMsePer * 256);
-  return (int)std::max<int64_t>(1, std::min<int64_t>(b, (int64_t)r * 16));
+  const int per = n4 / (kMsePer * 256) * count >= 2 * 152 ? kMsePer : kMseFew;
+  return (int)std::max<int64_t>(1, std::min<int64_t>(n4 / (per * 256), (int64_t)r * 16));
 }
 
 cudaError_t launch_mse_grad(const Solve& s, const Solve* tab, int count, int r, cudaStream_t st) {
-  return launch_k(k_mse_grad, dim3(mse_blocks(r), 1, count), dim3(256), 0, st, 0, s, tab);
+  return launch_k(k_mse_grad, dim3(mse_blocks(r, count), 1, count), dim3(256), 0, st, 0, s, tab);
 }
 
 // A bounded wait on a barrier that nothing completes (see
