@@ -90,7 +90,7 @@ struct Tet {
 constexpr int kMeshNT = 256;
 
 // Cubes are classified V = 4 consecutive ones along z to a thread (vector
-// loads of the four grid rows they touch; V = 1 for r = 2 and for grids off a
+// loads of the four grid rows they touch; V = 1 below r = 64 and for grids off a
 // 16-byte boundary), the few that the level set crosses (1 in 70 at r = 128)
 // are compacted into a list in shared memory, and the block then works through
 // (cube, tetrahedron) pairs, a thread each, at output places known from one
@@ -244,7 +244,9 @@ static int launch_mesh_extract(const float* chi, int r, float level, float* tris
   if (cudaMemsetAsync(count, 0, sizeof(unsigned long long), st) != cudaSuccess) return DPSR_ECUDA;
   int lg = 0;
   while ((1 << lg) < r) ++lg;
-  const int v = r >= 4 && ((uintptr_t)chi & 15) == 0 ? 4 : 1;
+  // Four cubes a thread from r = 64 on: below, a block of 1 024 cubes leaves SMs idle
+  // (32 blocks at r = 32: a sphere 12.5 us, noise 58.1; by single cubes 9.8 and 21.7).
+  const int v = r >= 64 && ((uintptr_t)chi & 15) == 0 ? 4 : 1;
   const int64_t n = (int64_t)r * r * r;
   const unsigned blocks = (unsigned)((n + kMeshNT * v - 1) / (kMeshNT * v));
   auto go = [&](auto fn) {
