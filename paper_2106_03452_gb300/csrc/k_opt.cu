@@ -3,10 +3,12 @@
 // points sampled on the mesh and the input cloud (with its gradient with
 // respect to the mesh points), the largest component of the mesh for the
 // resampling step, and area-weighted sampling of points on the mesh.
+#include <limits.h>
 #include <math.h>
 #include <stdint.h>
 
 #include <algorithm>
+#include <atomic>
 
 #include "dpsr.h"
 #include "dpsr_dev.cuh"
@@ -319,23 +321,42 @@ __global__ void __launch_bounds__(kScanNT) k_block_offsets(double* __restrict__ 
 // live in L1, and the grid is small: launched early it would crowd onto the SMs
 // that the scan leaves free, so it waits (20 000 points on 150 001 triangles,
 // both kernels: 40 us early with the offsets in a launch of their own, 20.5).
+//
+// The searches compare bits (non-negative doubles are ordered as their bits are):
+// the narrow FP64 pipe, which many samples keep busy, has the coordinates to do.
+// And half of an SM's memory stays L1, for both kernels alike (a change between
+// them empties the SM): the offsets of 13 blocks would take all of it, and the
+// searches' reads miss. A million samples of 150 000 triangles: 176 us without
+// either, 140 with the comparisons, 103 with both; 20 000: 25.4, 23.5 and 23.5.
 constexpr int kOffShared = 2048;
-constexpr int kSampleNT = 64;  // 20 000 samples: 313 blocks, two per SM (the searches compare on the FP64 pipe)
-__global__ void __launch_bounds__(kSampleNT) k_sample(const float* __restrict__ tris, const float* __restrict__ nrm,
-                                                int64_t T, const double* __restrict__ cum,
-                                                const double* __restrict__ tot, int nblocks, int64_t M, uint64_t seed,
-                                                float* __restrict__ p, float* __restrict__ n) {
+constexpr int kSampleCarve = 50;  // per cent of shared memory: seven blocks
+// Threads of a block: 64 up to what the GPU holds of those at a time (20 000 samples:
+// 313 blocks, two per SM), 128 beyond.
+constexpr int kSampleBlocks = 152 * 7, kSampleFew = 64, kSampleMany = 128;
+
+// The bits of a non-negative sum; a NaN (areas that are not finite) above all.
+__device__ __forceinline__ long long sum_bits(double v) {
+  const long long k = __double_as_longlong(v);
+  return (k & LLONG_MAX) > 0x7ff0000000000000ll ? LLONG_MAX : k;
+}
+
+template <int NT>
+__global__ void __launch_bounds__(NT) k_sample(const float* __restrict__ tris, const float* __restrict__ nrm,
+                                               int64_t T, const double* __restrict__ cum,
+                                               const double* __restrict__ tot, int nblocks, int64_t M, uint64_t seed,
+                                               float* __restrict__ p, float* __restrict__ n) {
   __shared__ double sh[kOffShared];
-  __shared__ double wtot[kSampleNT / 32];
+  __shared__ double wtot[NT / 32];
   pdl_trigger();
   pdl_wait();
   const double* off = tot;
+  const long long* sums = reinterpret_cast<const long long*>(cum);
   double A;
   if (nblocks <= kOffShared) {
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    for (int i = tid; i < nblocks; i += kSampleNT) sh[i] = tot[i];
+    for (int i = tid; i < nblocks; i += NT) sh[i] = tot[i];
     __syncthreads();
-    const int per = (nblocks + kSampleNT - 1) / kSampleNT;
+    const int per = (nblocks + NT - 1) / NT;
     const int b0 = std::min(tid * per, nblocks), b1 = std::min(b0 + per, nblocks);
     double run = 0.0;
     for (int b = b0; b < b1; ++b) run += sh[b];
@@ -350,7 +371,7 @@ __global__ void __launch_bounds__(kSampleNT) k_sample(const float* __restrict__ 
     if (lane == 0) acc = 0.0;
     __syncthreads();
     A = 0.0;
-    for (int k = 0; k < kSampleNT / 32; ++k) {
+    for (int k = 0; k < NT / 32; ++k) {
       if (k == w) acc += A;
       A += wtot[k];
     }
@@ -365,27 +386,32 @@ __global__ void __launch_bounds__(kSampleNT) k_sample(const float* __restrict__ 
     A = tot[nblocks];
   }
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < M; s += (int64_t)gridDim.x * blockDim.x) {
-    const double x = u01(seed, 3 * s) * A;
-    int b = 0, e = nblocks;  // off[b] <= x (off[0] = 0), off[e] > x or e the end
-    while (e - b > 1) {
-      const int mid = (b + e) >> 1;
-      if (off[mid] > x) e = mid;
-      else b = mid;  // NaN areas too: the last triangle answers, as in the second search
-    }
-    const double base = off[b];
-    int64_t lo = (int64_t)b * kScanBlock, hi = std::min<int64_t>(lo + kScanBlock, T) - 1;
-    while (lo < hi) {
-      const int len = (int)(hi - lo);
-      const int64_t m1 = lo + len / 4, m2 = lo + len / 2, m3 = lo + 3 * len / 4;  // lo <= m1 <= m2 <= m3 < hi
-      const double c1 = cum[m1], c2 = cum[m2], c3 = cum[m3];
-      if (c2 + base > x) {
-        hi = m2;
-        if (c1 + base > x) hi = m1;
-        else lo = m1 + 1;
-      } else {
-        lo = m2 + 1;
-        if (c3 + base > x) hi = m3;
-        else lo = m3 + 1;
+    int64_t lo = 0;
+    if (T > 1) {
+      const double x = u01(seed, 3 * s) * A;
+      const long long xk = sum_bits(x);
+      int b = 0, e = nblocks;  // off[b] <= x (off[0] = 0), off[e] > x or e the end
+      while (e - b > 1) {
+        const int mid = (b + e) >> 1;
+        if (__double_as_longlong(off[mid]) > xk) e = mid;
+        else b = mid;  // NaN areas too: the last triangle answers, as in the second search
+      }
+      const long long yk = sum_bits(x - off[b]);
+      lo = (int64_t)b * kScanBlock;
+      int64_t hi = std::min<int64_t>(lo + kScanBlock, T) - 1;
+      while (lo < hi) {
+        const int len = (int)(hi - lo);
+        const int64_t m1 = lo + len / 4, m2 = lo + len / 2, m3 = lo + 3 * len / 4;  // lo <= m1 <= m2 <= m3 < hi
+        const long long c1 = sums[m1], c2 = sums[m2], c3 = sums[m3];
+        if (c2 > yk) {
+          hi = m2;
+          if (c1 > yk) hi = m1;
+          else lo = m1 + 1;
+        } else {
+          lo = m2 + 1;
+          if (c3 > yk) hi = m3;
+          else lo = m3 + 1;
+        }
       }
     }
     double u = u01(seed, 3 * s + 1), v = u01(seed, 3 * s + 2);
@@ -400,6 +426,20 @@ __global__ void __launch_bounds__(kSampleNT) k_sample(const float* __restrict__ 
       n[3 * s + d] = nrm[3 * lo + d];
     }
   }
+}
+
+// The share of shared memory of the sampling kernels, once per device.
+static cudaError_t sample_carve() {
+  static std::atomic<uint64_t> done{0};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess || (dev < 64 && (done.load() >> dev) & 1u)) return e;
+  const auto share = cudaFuncAttributePreferredSharedMemoryCarveout;
+  e = cudaFuncSetAttribute(k_area_scan, share, kSampleCarve);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_sample<kSampleFew>, share, kSampleCarve);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_sample<kSampleMany>, share, kSampleCarve);
+  if (e == cudaSuccess && dev < 64) done.fetch_or(1ull << dev);
+  return e;
 }
 
 }  // namespace dpsr
@@ -450,13 +490,19 @@ int dpsr_mesh_sample(const float* tris, const float* normals, int64_t T, int64_t
   const int nblk = (int)((T + dpsr::kScanBlock - 1) / dpsr::kScanBlock);
   double* cum = ws;
   double* tot = ws + T;  // nblk + 1 entries
-  cudaError_t e = dpsr::launch_k(dpsr::k_area_scan, dim3(nblk), dim3(dpsr::kScanNT), 0, st, 0, tris, T, cum, tot);
+  cudaError_t e = dpsr::sample_carve();
+  if (e == cudaSuccess)
+    e = dpsr::launch_k(dpsr::k_area_scan, dim3(nblk), dim3(dpsr::kScanNT), 0, st, 0, tris, T, cum, tot);
   if (e == cudaSuccess && nblk > dpsr::kOffShared)
     e = dpsr::launch_k(dpsr::k_block_offsets, dim3(1), dim3(dpsr::kScanNT), 0, st, 0, tot, nblk);
-  const unsigned sb = (unsigned)std::min<int64_t>((M + dpsr::kSampleNT - 1) / dpsr::kSampleNT, 4736);
+  auto sample = [&](auto fn, int nt) {
+    const unsigned blocks = (unsigned)std::min<int64_t>((M + nt - 1) / nt, dpsr::kSampleBlocks);
+    return dpsr::launch_after(fn, dim3(blocks), dim3(nt), 0, st, 0, tris, normals, T, (const double*)cum,
+                              (const double*)tot, nblk, M, seed, points, pnormals);
+  };
   if (e == cudaSuccess)
-    e = dpsr::launch_after(dpsr::k_sample, dim3(sb), dim3(dpsr::kSampleNT), 0, st, 0, tris, normals, T, (const double*)cum,
-                       (const double*)tot, nblk, M, seed, points, pnormals);
+    e = M <= (int64_t)dpsr::kSampleBlocks * dpsr::kSampleFew ? sample(dpsr::k_sample<dpsr::kSampleFew>, dpsr::kSampleFew)
+                                                            : sample(dpsr::k_sample<dpsr::kSampleMany>, dpsr::kSampleMany);
   if (e != cudaSuccess) cudaGetLastError();
   return e == cudaSuccess ? DPSR_OK : DPSR_ECUDA;
 }

@@ -107,3 +107,18 @@ def test_areas_that_are_not_finite(T, bad):
     nrm = torch.arange(T, device="cuda", dtype=torch.float32)[:, None].expand(T, 3).contiguous()
     _, n = sample(tris, nrm, 500, 3)
     assert torch.equal(n, nrm[-1].expand(500, 3))
+
+
+@pytest.mark.parametrize("T", [1, 2, 1025, 2048 * 1024 + 5])
+def test_many_samples_are_the_few(T):
+    """A draw depends on its index alone: calls of few and of many samples (blocks
+    of 64 and of 128 threads, one and several samples a thread) share theirs."""
+    import torch
+    from paper_2106_03452_gb300.mesh import sample
+    g = torch.Generator("cuda").manual_seed(T)
+    tris, nrm = torch.rand((T, 3, 3), device="cuda", generator=g), torch.rand((T, 3), device="cuda", generator=g)
+    few = sample(tris, nrm, 68096, 9)
+    for M in (1, 68097, 300001):
+        many = sample(tris, nrm, M, 9)
+        n = min(M, 68096)
+        assert torch.equal(many[0][:n], few[0][:n]) and torch.equal(many[1][:n], few[1][:n])
