@@ -140,18 +140,21 @@ def _barrier(dist):
 
 # ----------------------------------------------------------------------------
 # algorithmic byte model (per launch / per solve): the bytes each plane kind
-# must move at least, whichever path (cluster or pencil) runs it
+# must move at least for a cloud in every tile, whichever path (cluster or
+# pencil) runs it. From r = 64 on tiles and planes without points are neither
+# written nor read, and the traffic may lie below it.
 # ----------------------------------------------------------------------------
 def kernel_bytes(r: int, N: int):
     U = 4 * r ** 3                      # one FP32 real grid
     H = 8 * r * r * (r // 2 + 1)        # one complex half spectrum
     rec = 32                            # sorted point record
+    x = 4 if r < 256 else 3             # from r = 256 on the weights stay out of the x passes
     return {
         "plane_fwd": 3 * H + 2 * rec * N,
-        "xpass_fwd": 4 * H,
+        "xpass_fwd": x * H,
         "plane_inv": H + U + 2 * (rec + 16) * N,
         "plane_bfwd": 2 * U + H,
-        "xpass_bwd": 4 * H,
+        "xpass_bwd": x * H,
         "plane_binv": 2 * H + 2 * (rec + 24) * N,
         "bin": 2 * 24 * N + 4 * N + (rec + 4) * N,
         "combine": (32 * 2 + 16 * 2 + 8 + 24) * N,
@@ -164,9 +167,10 @@ def kernel_bytes(r: int, N: int):
 # a kind, size or path not listed reports traffic as null.
 MEASURED_TRAFFIC = {
     # k_zfwd<128> + k_yfwd<128, 0> (the pencil forward plane kind), r = 128 ellipsoids, N = 20000
-    ("plane_fwd", 128, 0): 682240 + 37711872,
-    ("plane_binv", 128, 1): 21772288,   # k_plane_binv<128, 1> (512 threads), same workload
-    ("plane_binv", 128, 3): 21667072,   # k_plane_binv_ch<128> (one CTA per plane and channel)
+    ("plane_fwd", 128, 0): 674048 + 14125824,
+    ("plane_binv", 128, 0): 12479488 + 8448512,  # k_yadj<128> + k_zinv<128, 3>, same workload
+    ("plane_binv", 128, 1): 13232640,   # k_plane_binv<128, 1> (512 threads)
+    ("plane_binv", 128, 3): 13141248,   # k_plane_binv_ch<128> (one CTA per plane and channel)
 }
 
 
