@@ -21,6 +21,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <atomic>
 #include <complex>
 #include <mutex>
 #include <new>
@@ -335,7 +336,7 @@ int grow_points(dpsr_plan p, int64_t n) {
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
+  static std::atomic<PFN_cuTensorMapEncodeTiled_v12000> fn{nullptr};
   if (!fn) {
     void* p = nullptr;
     cudaDriverEntryPointQueryResult q;

@@ -24,6 +24,8 @@
 //
 // Half spectra along z are stored "packed" between the passes: slot 0 holds
 // the DC and Nyquist terms of a real row as one complex number.
+#include <atomic>
+
 #include "col.cuh"
 #include "coldir.cuh"
 #include "dpsr_dev.cuh"
@@ -1237,7 +1239,7 @@ static cudaError_t launch_pencil_t(int kind, const Solve& s, const Solve* tab, i
                                    cudaStream_t st) {
   using P = Pen<L>;
   const dim3 gy(L * P::NKC, 1, count);
-  static bool attr_set[4] = {false, false, false, false};
+  static std::atomic<bool> attr_set[4];  // set last: other threads may launch meanwhile
   cudaError_t e = cudaSuccess;
   switch (kind) {
     case 0: {
@@ -1257,7 +1259,7 @@ static cudaError_t launch_pencil_t(int kind, const Solve& s, const Solve* tab, i
     case 1: {
       constexpr size_t a = yinv_smem<L, 1>(), b = zinv_smem<L, 1>();
       constexpr int nt = ynt<L>();
-      static int nz = 0;
+      static std::atomic<int> nz{0};
       if (!attr_set[1]) {
         e = set_smem(k_yinv<L, 1>, a);
         if (e == cudaSuccess) e = set_smem(k_zinv<L, 1>, b);
@@ -1273,7 +1275,7 @@ static cudaError_t launch_pencil_t(int kind, const Solve& s, const Solve* tab, i
     }
     case 2: {
       constexpr size_t a = zbfwd_smem<L>(), b = yfwd_smem<L, true>();
-      static int nz = 0;
+      static std::atomic<int> nz{0};
       if (!attr_set[2]) {
         e = set_smem(k_zbfwd<L>, a);
         if (e == cudaSuccess) e = set_smem(k_yfwd<L, true>, b);
@@ -1287,7 +1289,7 @@ static cudaError_t launch_pencil_t(int kind, const Solve& s, const Solve* tab, i
     }
     default: {
       constexpr size_t b = zinv_smem<L, 3>();
-      static int nz = 0;
+      static std::atomic<int> nz{0};
       if constexpr (L >= 64) {
         constexpr size_t a = ydir_smem<L>();
         if (!attr_set[3]) {

@@ -16,6 +16,8 @@
 //   k_plane_binv (backward) IFFT along y -> C2R along z of the three adjoint
 //                           fields V_bar_a, then the adjoint of the splat
 //                           (gather and weight derivatives) at the points.
+#include <atomic>
+
 #include "dpsr_dev.cuh"
 #include "finalize.cuh"
 #include "launch.h"
@@ -1098,7 +1100,7 @@ static cudaError_t launch_binv_ch_t(const Solve& s, const Solve* tab, int count,
     return cudaErrorInvalidValue;
   } else {
     constexpr size_t smem = binv_ch_smem<L>();
-    static bool attr_set = false;
+    static std::atomic<bool> attr_set{false};
     if (!attr_set) {
       const cudaError_t e =
           cudaFuncSetAttribute(k_plane_binv_ch<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1134,7 +1136,7 @@ static cudaError_t launch_plane_t(int kind, const Solve& s, const Solve* tab, in
   }
   if (kind == 3) smem = binv_smem<L, C>();
   if (smem > 227 * 1024) return cudaErrorInvalidConfiguration;
-  static bool attr_set[4] = {false, false, false, false};  // per instantiation and kind
+  static std::atomic<bool> attr_set[4];  // per instantiation and kind
   if (!attr_set[kind]) {
     cudaError_t e =
         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

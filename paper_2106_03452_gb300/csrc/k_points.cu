@@ -2,6 +2,7 @@
 // stencil (a counting sort, so that each x-plane cluster reads only the points
 // that touch its plane), and the final combine of the backward pass.
 #include <algorithm>
+#include <atomic>
 
 #include "dpsr_dev.cuh"
 #include "finalize.cuh"
@@ -175,7 +176,7 @@ template <int NT>
 static cudaError_t launch_bin_t(const Solve& s, const Solve* tab, int count, int nmax, int r, cudaStream_t st) {
   const int blocks = min(max((nmax + NT - 1) / NT, 1), 1184 * 256 / NT);
   const size_t hc = sizeof(int) * nbins(r), hs = sizeof(int) * scan_slot(nbins(r));
-  static bool attr_set = false;  // 16384 bins at r = 512 need more than the default 48 KB
+  static std::atomic<bool> attr_set{false};  // 16384 bins at r = 512 need more than the default 48 KB
   if (!attr_set) {
     cudaError_t e = cudaFuncSetAttribute(k_bin_count<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)(sizeof(int) * nbins(512)));

@@ -11,6 +11,8 @@
 //           to r = 128 and by the y pass above (kHalfW);  Q1 = IFFT_x(F),
 //           Q2 = IFFT_x(-i u_x F)  (the adjoint of Eq. 3, conj(H_a) = -H_a).
 // Three FFTs of length r per column in each direction.
+#include <atomic>
+
 #include "col.cuh"
 #include "dpsr_dev.cuh"
 #include "launch.h"
@@ -316,7 +318,7 @@ template <int L, bool BWD>
 static cudaError_t launch_xpass_t(const Solve& s, const Solve* tab, int count, cudaStream_t st) {
   using P = XGeo<L>;
   constexpr size_t smem = xpass_smem<L, BWD>();
-  static bool attr_set = false;
+  static std::atomic<bool> attr_set{false};
   if (!attr_set) {
     cudaError_t e = cudaFuncSetAttribute(k_xpass<L, BWD>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -177,3 +177,59 @@ def test_a_plan_without_a_name_answers_as_another():
     (got,) = torch.autograd.grad(chi, a, w)
     assert float((got - want).abs().max()) <= 1e-5 * float(want.abs().max())
     plan.close()
+
+
+def test_threads_with_plans_of_their_own(tmp_path):
+    """Eight threads solve at once from the first call of a process on, each with
+    its plan and stream (the kernels' set-up is shared): the results of one thread."""
+    import os
+    import subprocess
+    import sys
+    code = """
+import sys, threading
+import torch
+from paper_2106_03452_gb300.dpsr import Plan, dpsr
+from paper_2106_03452_gb300.mesh import MeshPoints
+from paper_2106_03452_gb300.optimize import chamfer
+def cloud(k):
+    g = torch.Generator("cuda").manual_seed(k)
+    d = torch.nn.functional.normalize(torch.randn((2000 + 300 * k, 3), device="cuda", generator=g), dim=1)
+    return (0.5 + 0.3 * d).contiguous(), d, torch.randn((R[k],) * 3, device="cuda", generator=g)
+R = (32, 64, 128, 256, 32, 64, 128, 256)
+def solve(k, plan):
+    p, d, w = IN[k]
+    a = p.clone().requires_grad_(True)
+    chi = dpsr(a, d, plan)
+    (g,) = torch.autograd.grad(chi, a, w)
+    m, _ = MeshPoints.apply(chi.detach(), 0.0, 500, k)
+    return [chi.detach(), g, chamfer(p, p.flip(0) + 0.01), torch.tensor(float(m.shape[0]))]
+IN = [cloud(k) for k in range(8)]
+torch.cuda.synchronize()
+out, err, go = [None] * 8, [], threading.Barrier(8)
+def work(k):
+    try:
+        st = torch.cuda.Stream()
+        with torch.cuda.stream(st):
+            plan = Plan(R[k], 2.0)
+            go.wait()
+            for _ in range(5):
+                out[k] = solve(k, plan)
+            st.synchronize()
+            assert plan.sync() == 0
+    except BaseException as e:
+        err.append(repr(e))
+        go.abort()
+ts = [threading.Thread(target=work, args=(k,)) for k in range(8)]
+[t.start() for t in ts]
+[t.join() for t in ts]
+assert not err, err
+for k in range(8):
+    for x, y in zip(out[k], solve(k, Plan(R[k], 2.0))):
+        assert float((x - y).abs().max()) <= 1e-5 * float(y.abs().max()), k
+print("fine")
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    for tune in ("1", "0"):
+        r = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300,
+                           env={**os.environ, "DPSR_TUNE": tune, "PYTHONPATH": root})
+        assert r.returncode == 0 and "fine" in r.stdout, r.stderr[-3000:]
